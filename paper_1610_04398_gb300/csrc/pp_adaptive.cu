@@ -1,25 +1,26 @@
-// Pressure at every cell of an adaptive (multiresolution) grid in FP64, Eq. greenSum with
-// each source cell clamped at its own rho_h: the fast multipole method on the tree and the
-// interaction lists of pp_atree (dual-tree walk).  Leaves are blocks of 8 x 8 cells; a box of
-// level l has side s = 2^-l of the unit domain and centre ((ix + 1/2) s, (iy + 1/2) s).
-// Expansions are kept in units of their own box side (multipole M_k = alpha_k / s^k, local
-// L_l = b_l s^l, Appendix A.2's series and their standard local shifts, for 2 pi P):
-//   P2M   S = sum q, M_k = sum q w^k / k, w = (z - c) / s
-//   M2M   parent M_k += S u^k / k + sum_{l<=k} M_l 2^-l u^(k-l) C(k-1, l-1), u = (c_child - c) / s
-//   M2L   with tau = (c_src - c_tgt) / s_tgt, rho = s_src / s_tgt, x_k = -M_k (-1)^k (rho/tau)^k:
-//         L_0 += S (log|tau| + log s_tgt) + sum_k x_k,
+// Pressure at every cell of an adaptive (multiresolution) grid, Eq. greenSum with each source
+// cell clamped at its own rho_h: the fast multipole method on the tree and the interaction
+// lists of pp_atree (dual-tree walk), in FP64 and in mixed precision.  Leaves are blocks of
+// 8 x 8 cells; a box of level l has side s = 2^-l of the unit domain and centre
+// ((ix + 1/2) s, (iy + 1/2) s).  Expansions are kept in units of their own box side (multipole
+// M_k = alpha_k / s^k, local L_l = b_l s^l, Appendix A.2's series and their standard local
+// shifts, for 2 pi P), every translation factored as diagonal * real matrix * diagonal:
+//   P2M   S = sum q, M_k = sum q w^k / k, w = (z - c) / s (table of w^k / k)
+//   M2M   parent M_k = zeta^k [S / k + sum_{j<=k} C(k-1, j-1) (2 zeta)^-j M_j], zeta = (+-1 +- i) / 4
+//   M2L   with tau = (c_src - c_tgt) / s_tgt, rho = s_src / s_tgt, x_k = -M_k (-rho/tau)^k:
+//         L_0 += S (log|tau| + log s_tgt) + Re sum_k x_k,
 //         L_l += tau^-l (-S / l + sum_k x_k C(l+k-1, k-1))
-//   L2L   child L_l += 2^-l sum_{k>=l} L_k C(k, l) v^(k-l), v = (c_child - c) / s
-//   L2P   P = Re sum_l L_l w^l / (2 pi); near field over the near-field leaf pairs: between
-//         leaves of one level every cell pair sits at an integer offset D (in cells of side h),
-//         so q log max(h|D|, rho_h) = q (log h + T[D]) with T[D] = log|D| (T[0] = c0) tabulated
-//         once in FP64; leaves of different levels are summed directly.
-// One launch per step and level; every sum runs in a fixed order, so results repeat bitwise.
-// The first solve on a tree uploads the tree, the lists and the table and allocates the
-// expansions; they stay with the tree for later solves.
+//   L2L   child L_l += (2 zeta)^-l sum_{k>=l} C(k, l) zeta^k L_k
+//   L2P   P = Re sum_l L_l w^l / (2 pi); near field over the near-field leaf pairs from tables
+//         of log|D| over the integer cell offsets D of the pair (below).
+// A solve is three launches: the upward pass (k_aup), the translations (k_am2l) and, per
+// leaf, the shifts down its path, the local evaluation and the near field (k_aleaf).  Every
+// sum runs in a fixed order, so results repeat bitwise.  The first solve on a tree uploads
+// the tree, the lists and the tables and allocates the expansions; they stay with the tree.
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdint>
 #include <cstdlib>
@@ -28,12 +29,21 @@
 
 #include "../../include/pp.h"
 #include "pp_atree_state.h"
+#include "pp_common.h"
+#include "pp_log.cuh"
 
 namespace {
 
+using pp::cplx_of;
+using pp::df_add;
+using pp::df_fma;
+using pp::df_to;
+
 constexpr int kMaxOrderA = 30;
+constexpr int kTP = 32;  // stride (coefficients) of the expansion arrays and of the tables
 constexpr double kInv2PiA = 0.15915494309189533576888376337251;
 constexpr double kC0A = 0.78539816339744830962 - 1.5 - 0.34657359027997265471;  // pi/4 - 3/2 - ln2/2
+constexpr double kLn2A = 0.69314718055994530941723212145818;
 
 struct AGeo {
     double cx, cy, s;     // centre and side
@@ -43,269 +53,648 @@ struct AGeo {
 __host__ __device__ __forceinline__ double2 zmul(double2 a, double2 b) {
     return double2{a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};
 }
-__host__ __device__ __forceinline__ double2 zadd(double2 a, double2 b) { return double2{a.x + b.x, a.y + b.y}; }
 __host__ __device__ __forceinline__ double2 zscale(double2 a, double f) { return double2{a.x * f, a.y * f}; }
-__host__ __device__ __forceinline__ double2 zinv(double2 a) {
-    const double d = a.x * a.x + a.y * a.y;
-    return double2{a.x / d, -a.y / d};
-}
 
 // Cell (cx, cy) of a leaf block, index cy * 8 + cx, in units of the block side about its centre.
 __host__ __device__ __forceinline__ double2 cell_w(int c) {
     return double2{((c & 7) + 0.5) / 8.0 - 0.5, ((c >> 3) + 0.5) / 8.0 - 0.5};
 }
 
-// Each step is a body over (CTA index, thread index) with no shared memory and no barrier,
-// wrapped by a kernel; the threads of a step are independent.
+template <typename T>
+__device__ __forceinline__ typename cplx_of<T>::type cx(T x, T y) {
+    typename cplx_of<T>::type r;
+    r.x = x;
+    r.y = y;
+    return r;
+}
+template <typename T, typename C>
+__device__ __forceinline__ C cmulT(C a, C b) {
+    return cx<T>(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
+}
 
-// P2M: one CTA of 32 threads per leaf, thread k forms coefficient k (k = 0 is S).
-__host__ __device__ inline void ap2m_body(int i, int k, int nleaf, const int* __restrict__ leafbox,
-                                          const double* __restrict__ q, int p, double* __restrict__ S,
-                                          double2* __restrict__ M) {
-    if (i >= nleaf || k > p) return;
-    const int b = leafbox[i];
-    const double* qq = q + int64_t(i) * 64;
+// Constant tables of the factored steps, built on the host in FP64, stored in the precision of
+// the expansions.  Rows of 32: lane l of a warp reads column l.
+template <typename T>
+struct AConst {
+    typedef typename cplx_of<T>::type C;
+    T m2l[kTP][kTP];  // [k][l]: C(l+k-1, k-1) for l >= 1, 1 for l = 0
+    T m2m[kTP][kTP];  // [j][k]: C(k-1, j-1) for 1 <= j <= k; [0][k] = 1/k
+    T l2l[kTP][kTP];  // [k][l]: C(k, l) for l <= k
+    C W[64][kTP];     // [cell][k]: w^k / k
+    C V[kTP][64];     // [l][cell]: w^l
+    C Z[4][kTP];      // [child quadrant][k]: zeta^k
+    C ZI[4][kTP];     // [child quadrant][k]: (2 zeta)^-k
+};
+
+// Near-field leaf pair of a target leaf: the source leaf, how the levels relate (kind 0: the
+// same level; kappa > 0: the source is kappa levels finer; kappa < 0: coarser; kDirect: summed
+// directly) and the offsets of the pair's cells (see k_aleaf).
+struct APair {
+    int src, kind, ox, oy;
+};
+constexpr int kDirect = 64;
+constexpr int kMaxKappa = 3;     // level differences served from the table
+constexpr int kMaxOddSide = 192;  // its largest side
+
+// ------------------------------------------------------------------------------------
+// Upward pass, one warp per leaf: the leaf's multipole from the table of w^k / k (lane k
+// forms M_k), then up the tree: the warp that arrives last at a parent (an arrival counter it
+// resets; no warp waits) shifts the four children, whichever warp that is: the arithmetic and
+// its order do not depend on it.  One launch in place of one per level: 0.24 ms (FP64) and 21 us
+// (mixed) a level for 1629 boxes before, most of it latency and powers formed per lane.
+// The children's zeta are 90 degree rotations of each other, zeta_q = i^m(q) zeta_3, so with
+// G_r[j] = sum_q i^(m(q) r) M_j of child q the four shifts are one real product,
+//   M_k = zeta_3^k [G_k[0] / k + sum_j C(k-1, j-1) (2 zeta_3)^-j G_(k-j)[j]]
+// (indices of G mod 4, G[0] from the monopoles): 76 FP64 instructions a parent instead of 192.
+// FP64 solves also write each leaf's weights in fixed point for the near field: v = q 2^(54-e)
+// rounded, e the leaf's exponent (|q| < 2^e), kBadExp for a leaf with a non-finite weight.
+// ------------------------------------------------------------------------------------
+// Mixed solves copy theirs (q need not be aligned for the near field's 16-byte reads).
+constexpr int kBadExp = INT_MAX;
+
+template <typename T>
+struct NearSrc {
+    typedef T type;
+};
+template <>
+struct NearSrc<double> {
+    typedef long long type;
+};
+
+template <typename T>
+__global__ void __launch_bounds__(128) k_aup(int nleaf, const int* __restrict__ leafbox,
+                                             const int* __restrict__ parent, const int* __restrict__ first_child,
+                                             const T* __restrict__ q, int p, const AConst<T>* __restrict__ ct,
+                                             double* __restrict__ S, float2* __restrict__ Sf,
+                                             typename cplx_of<T>::type* __restrict__ M, unsigned* __restrict__ cnt,
+                                             typename NearSrc<T>::type* __restrict__ qfix, int* __restrict__ qexp) {
+    typedef typename cplx_of<T>::type C;
+    __shared__ T Rm[kTP][kTP];
+    __shared__ C G[4][kTP][4];
+    __shared__ T qs[4][64];
+    const int w = threadIdx.x >> 5, k = threadIdx.x & 31;
+    for (int i = threadIdx.x; i < kTP * kTP; i += 128) (&Rm[0][0])[i] = (&ct->m2m[0][0])[i];
+    __syncthreads();
+    const int leaf = blockIdx.x * 4 + w;
+    if (leaf >= nleaf) return;  // warp-uniform; no block barrier follows
+    const T q0 = q[int64_t(leaf) * 64 + k], q1 = q[int64_t(leaf) * 64 + 32 + k];
+    qs[w][k] = q0;
+    qs[w][k + 32] = q1;
+    T s = q0 + q1;
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    int b = leafbox[leaf];
+    if constexpr (sizeof(T) == 8) {
+        const bool bad = __any_sync(0xffffffffu, !(isfinite(q0) && isfinite(q1)));
+        double m = fmax(fabs(q0), fabs(q1));
+        for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+        int e = -900;
+        if (!bad && m > 0.0) e = max(ilogb(m) + 1, -900);
+        const double f = __hiloint2double((1023 + 54 - (bad ? 0 : e)) << 20, 0);  // 2^(54 - e)
+        qfix[int64_t(leaf) * 64 + k] = bad ? 0 : __double2ll_rn(q0 * f);
+        qfix[int64_t(leaf) * 64 + 32 + k] = bad ? 0 : __double2ll_rn(q1 * f);
+        if (k == 0) qexp[leaf] = bad ? kBadExp : e;
+    } else {
+        qfix[int64_t(leaf) * 64 + k] = q0;
+        qfix[int64_t(leaf) * 64 + 32 + k] = q1;
+    }
+    __syncwarp();
+    C acc = cx<T>(T(0), T(0));
+    if (k >= 1 && k <= p) {
+#pragma unroll 8
+        for (int c = 0; c < 64; ++c) {
+            const C wk = ct->W[c][k];
+            acc.x = fma(qs[w][c], wk.x, acc.x);
+            acc.y = fma(qs[w][c], wk.y, acc.y);
+        }
+    }
+    if (k <= p) M[int64_t(b) * kTP + k] = acc;
     if (k == 0) {
-        double s = 0.0;
-        for (int c = 0; c < 64; ++c) s += qq[c];
-        S[b] = s;
-        M[int64_t(b) * (p + 1)] = double2{0.0, 0.0};
+        S[b] = double(s);
+        if (sizeof(T) == 4) Sf[b] = make_float2(float(s), 0.f);
+    }
+    const C zk = ct->Z[3][k], zik = ct->ZI[3][k];
+    for (;;) {
+        const int pa = parent[b];
+        if (pa < 0) return;
+        __threadfence();  // this warp's expansion before its arrival
+        __syncwarp();
+        unsigned arrived = 0;
+        if (k == 0) arrived = atomicAdd(cnt + pa, 1u);
+        if (__shfl_sync(0xffffffffu, arrived, 0) != 3u) return;
+        __threadfence();  // the other children's after it
+        if (k == 0) cnt[pa] = 0u;
+        b = pa;
+        const int fc = first_child[b];
+        C m[4];
+        double sq[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            sq[c] = __ldcg(S + fc + c);
+            m[c] = k >= 1 && k <= p ? __ldcg(M + int64_t(fc + c) * kTP + k) : cx<T>(T(0), T(0));
+            if (k == 0) m[c] = cx<T>(T(sq[c]), T(0));
+        }
+        // i^m(q): m(3) = 0, m(2) = 1, m(0) = 2, m(1) = 3
+        const C e = cx<T>(m[3].x + m[0].x, m[3].y + m[0].y), f = cx<T>(m[2].x + m[1].x, m[2].y + m[1].y);
+        const C g = cx<T>(m[3].x - m[0].x, m[3].y - m[0].y), h = cx<T>(m[2].x - m[1].x, m[2].y - m[1].y);
+        __syncwarp();  // the last level's reads of G are done
+        G[w][k][0] = cmulT<T>(cx<T>(e.x + f.x, e.y + f.y), zik);
+        G[w][k][1] = cmulT<T>(cx<T>(g.x - h.y, g.y + h.x), zik);
+        G[w][k][2] = cmulT<T>(cx<T>(e.x - f.x, e.y - f.y), zik);
+        G[w][k][3] = cmulT<T>(cx<T>(g.x + h.y, g.y - h.x), zik);
+        __syncwarp();
+        C y = cx<T>(T(0), T(0));
+#pragma unroll 4
+        for (int j = 0; j <= p; ++j) {
+            const T r = Rm[j][k];
+            const C v = G[w][j][(k - j) & 3];
+            y.x = fma(r, v.x, y.x);
+            y.y = fma(r, v.y, y.y);
+        }
+        const double ssum = sq[0] + sq[1] + sq[2] + sq[3];
+        if (k >= 1 && k <= p) M[int64_t(b) * kTP + k] = cmulT<T>(y, zk);
+        if (k == 0) {
+            M[int64_t(b) * kTP] = cx<T>(T(0), T(0));
+            S[b] = ssum;
+            if (sizeof(T) == 4) Sf[b] = pp::df_from(ssum);
+        }
+    }
+}
+
+template <typename T>
+struct OpLog {  // log|tau| of an operator: FP64, or a double-float pair
+    typedef double type;
+};
+template <>
+struct OpLog<float> {
+    typedef float2 type;
+};
+
+// ------------------------------------------------------------------------------------
+// M2L: one CTA of four warps per target box, its entries dealt to the warps in turn.  The
+// diagonals (rho/tau)^k and tau^-l come from a table per distinct operator (a few hundred for
+// the tens of thousands of pairs; the powers were formed per pair and lane before).  Lane k
+// forms x_k in shared memory, lane l sums its row of the real product.  Mixed precision: the
+// constant term S log|tau| and the sums of S in double-float.
+// ------------------------------------------------------------------------------------
+template <typename T>
+__global__ void __launch_bounds__(128) k_am2l(const int* __restrict__ ptr, const int2* __restrict__ pair,
+                                              const AGeo* __restrict__ geo, const typename OpLog<T>::type* __restrict__ oplog,
+                                              const typename cplx_of<T>::type* __restrict__ op, int p,
+                                              const AConst<T>* __restrict__ ct, const double* __restrict__ S,
+                                              const float2* __restrict__ Sf,
+                                              const typename cplx_of<T>::type* __restrict__ M,
+                                              typename cplx_of<T>::type* __restrict__ L, double* __restrict__ L0) {
+    typedef typename cplx_of<T>::type C;
+    __shared__ T R[kTP][kTP];
+    __shared__ C xs[4][kTP];
+    __shared__ C red[4][kTP];
+    __shared__ double red0[4];
+    const int a = blockIdx.x, w = threadIdx.x >> 5, t = threadIdx.x & 31;
+    const int e0 = ptr[a], e1 = ptr[a + 1];
+    if (e0 == e1) {  // no sources (block-uniform)
+        if (w == 0 && t <= p) L[int64_t(a) * kTP + t] = cx<T>(T(0), T(0));
+        if (w == 0 && t == 0) L0[a] = 0.0;
         return;
     }
-    double2 acc{0.0, 0.0};
-    for (int c = 0; c < 64; ++c) {
-        const double2 w = cell_w(c);
-        double2 wk = w;
-        for (int j = 1; j < k; ++j) wk = zmul(wk, w);
-        acc = zadd(acc, zscale(wk, qq[c]));
-    }
-    M[int64_t(b) * (p + 1) + k] = zscale(acc, 1.0 / k);
-}
-
-__global__ void k_ap2m(int nleaf, const int* __restrict__ leafbox, const double* __restrict__ q, int p,
-                       double* __restrict__ S, double2* __restrict__ M) {
-    ap2m_body(blockIdx.x, threadIdx.x, nleaf, leafbox, q, p, S, M);
-}
-
-// M2M for the internal boxes in [b0, b1): thread k of CTA (b - b0) forms the parent's M_k.
-__host__ __device__ inline void am2m_body(int blk, int k, int b0, int b1, const int* __restrict__ first_child,
-                                          const AGeo* __restrict__ geo, int p, double* __restrict__ S,
-                                          double2* __restrict__ M) {
-    const int b = b0 + blk;
-    if (b >= b1 || k > p) return;
-    const int fc = first_child[b];
-    if (fc < 0) return;  // a leaf: its expansion came from P2M
-    double2 acc{0.0, 0.0};
-    double ssum = 0.0;
-    for (int ch = fc; ch < fc + 4; ++ch) {
-        const double Sc = S[ch];
-        ssum += Sc;
-        if (k == 0) continue;
-        const double2 u{(geo[ch].cx - geo[b].cx) / geo[b].s, (geo[ch].cy - geo[b].cy) / geo[b].s};
-        // S u^k / k
-        double2 uk = u;
-        for (int j = 1; j < k; ++j) uk = zmul(uk, u);
-        acc = zadd(acc, zscale(uk, Sc / k));
-        // sum_{l=1..k} M_l 2^-l u^(k-l) C(k-1, l-1), u^(k-l) built downwards from u^0
-        double binom = 1.0;  // C(k-1, l-1) at l = 1
-        for (int l = 1; l <= k; ++l) {
-            double2 ukl{1.0, 0.0};
-            for (int j = 0; j < k - l; ++j) ukl = zmul(ukl, u);
-            const double2 ml = M[int64_t(ch) * (p + 1) + l];
-            acc = zadd(acc, zscale(zmul(ml, ukl), ldexp(binom, -l)));
-            binom = binom * double(k - l) / double(l);  // C(k-1, l) from C(k-1, l-1)
+    for (int i = threadIdx.x; i < kTP * kTP; i += 128) (&R[0][0])[i] = (&ct->m2l[0][0])[i];
+    __syncthreads();
+    C acc = cx<T>(T(0), T(0));
+    const double lns = -kLn2A * geo[a].level;  // log of the target's side
+    const T cl = t == 0 ? T(0) : T(-1) / T(t);
+    float ah = 0.f, al = 0.f, sh = 0.f, sl = 0.f;  // mixed: constant term, sum of S
+    for (int e = e0 + w; e < e1; e += 4) {
+        const int2 pr = pair[e];
+        const C* o = op + int64_t(pr.y) * (2 * kTP);
+        const C m = M[int64_t(pr.x) * kTP + t], tk = o[t], tl = o[kTP + t];
+        __syncwarp();  // the last entry's reads are done
+        xs[w][t] = cmulT<T>(m, tk);
+        __syncwarp();
+        C y = cx<T>(T(0), T(0));
+        if constexpr (sizeof(T) == 8) {
+            y.x = S[pr.x] * (t == 0 ? oplog[pr.y] + lns : cl);
+        } else {
+            const float2 Sb = Sf[pr.x];
+            const float2 lt = oplog[pr.y];
+            y.x = Sb.x * cl;
+            df_fma(ah, al, Sb.x, Sb.y, lt.x, lt.y);
+            df_add(sh, sl, Sb.x, Sb.y);
         }
-    }
-    if (k == 0) {
-        S[b] = ssum;
-        M[int64_t(b) * (p + 1)] = double2{0.0, 0.0};
-    } else {
-        M[int64_t(b) * (p + 1) + k] = acc;
-    }
-}
-
-__global__ void k_am2m(int b0, int b1, const int* __restrict__ first_child, const AGeo* __restrict__ geo, int p,
-                       double* __restrict__ S, double2* __restrict__ M) {
-    am2m_body(blockIdx.x, threadIdx.x, b0, b1, first_child, geo, p, S, M);
-}
-
-// M2L: CTA per target box, thread l forms L_l from the box's sources in list order.
-__host__ __device__ inline void am2l_body(int a, int l, int nb, const int* __restrict__ ptr,
-                                          const int* __restrict__ src, const AGeo* __restrict__ geo, int p,
-                                          const double* __restrict__ S, const double2* __restrict__ M,
-                                          double2* __restrict__ L) {
-    if (a >= nb || l > p) return;
-    double2 acc{0.0, 0.0};
-    for (int e = ptr[a]; e < ptr[a + 1]; ++e) {
-        const int b = src[e];
-        const double st = geo[a].s;
-        const double2 tau{(geo[b].cx - geo[a].cx) / st, (geo[b].cy - geo[a].cy) / st};
-        const double rho = geo[b].s / st;
-        const double2 rt = zscale(zinv(tau), rho);  // rho / tau
-        const double Sb = S[b];
-        // sum_k x_k C(l+k-1, k-1), x_k = -M_k (-1)^k (rho/tau)^k
-        double2 sum{0.0, 0.0};
-        double2 pw = rt;
-        double binom = 1.0;  // C(l+k-1, k-1) at k = 1
+#pragma unroll 4
         for (int k = 1; k <= p; ++k) {
-            const double2 x = zscale(zmul(M[int64_t(b) * (p + 1) + k], pw), (k & 1) ? 1.0 : -1.0);
-            sum = zadd(sum, l == 0 ? x : zscale(x, binom));
-            pw = zmul(pw, rt);
-            binom = binom * double(l + k) / double(k);  // C(l+k, k) from C(l+k-1, k-1)
+            const T r = R[k][t];
+            const C x = xs[w][k];
+            y.x = fma(r, x.x, y.x);
+            y.y = fma(r, x.y, y.y);
         }
-        if (l == 0) {
-            const double lt = 0.5 * log(tau.x * tau.x + tau.y * tau.y) + log(st);
-            acc = zadd(acc, zadd(double2{Sb * lt, 0.0}, sum));
-        } else {
-            double2 tl = zinv(tau);  // tau^-l
-            const double2 ti = tl;
-            for (int j = 1; j < l; ++j) tl = zmul(tl, ti);
-            acc = zadd(acc, zmul(tl, zadd(double2{-Sb / l, 0.0}, sum)));
+        if constexpr (sizeof(T) == 4) df_add(ah, al, y.x, 0.f);  // lane 0: Re sum x_k
+        acc.x = fma(tl.x, y.x, fma(-tl.y, y.y, acc.x));
+        acc.y = fma(tl.x, y.y, fma(tl.y, y.x, acc.y));
+    }
+    red[w][t] = acc;
+    if (t == 0) red0[w] = sizeof(T) == 8 ? double(acc.x) : df_to(ah, al) + lns * df_to(sh, sl);
+    __syncthreads();
+    if (w == 0 && t <= p) {
+        C s = red[0][t];
+#pragma unroll
+        for (int i = 1; i < 4; ++i) {
+            s.x += red[i][t].x;
+            s.y += red[i][t].y;
+        }
+        L[int64_t(a) * kTP + t] = s;
+        if (t == 0) L0[a] = red0[0] + red0[1] + red0[2] + red0[3];
+    }
+}
+
+// ------------------------------------------------------------------------------------
+// Leaves: one CTA per leaf.  Eight warps sum the near field, a ninth shifts the locals down
+// the leaf's path from the root (each leaf repeats its ancestors' shifts: no launch per level)
+// and forms the constant terms; then one thread per cell evaluates the local expansion.
+//
+// Near field.  Cell centres of two leaves differ by integer multiples of half the finer cell's
+// side, so log|x - x'| is log(unit) plus a table over integers.  Same level: offset m =
+// ox + rx - tx in cells (source cell column rx, target column tx), table `te` of log|(mx, my)|,
+// its [0][0] the self term c0.  Levels kappa apart: the offset is 2 m + 1 half cells of the finer
+// side with m = ox + 2^kappa rx - tx (source coarser) or ox + rx - 2^kappa tx (source finer), table
+// `to` over (|2 m_x + 1|, |2 m_y + 1|); the source's clamp never acts between different cells.
+// log(unit) times the source leaf's S is added once per leaf (FP64).  Pairs beyond the table
+// (kDirect) and, in FP64, leaves with non-finite weights are summed cell by cell.
+// A thread owns one row of 8 target cells and one row of 8 source cells of every fourth pair: its 64
+// cell pairs need 15 (same level) or 22 (kappa 1) kernel values, kept in registers.  Before, each
+// pair took its own table read, and pairs of different levels a square root and a logarithm.
+//
+// FP64 runs the cell pairs on the integer pipe: FP64 multiply-adds issue at 1.67 lanes a clock
+// and SM, 32 x 32 + 64 bit integer ones at 32 to 64.  Source weights are 55-bit integers v
+// (relative to the largest exponent et of the target's sources), kernel values 55-bit integers
+// (2^-52 units, |log| < 8), both split v = h 2^28 + l with l in [-2^27, 2^27); hh and hl + lh
+// accumulate exactly in 64 bits (32 source leaves a thread before they are added to the FP64
+// sum), ll (below 2^-56 of full scale a pair) is dropped.
+// ------------------------------------------------------------------------------------
+template <typename T>
+struct NearAcc;
+
+template <>
+struct NearAcc<float> {
+    typedef float Kv;  // kernel value
+    float part[8], acc[8], comp[8];
+    float q[8];
+    __device__ void init() {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) part[j] = acc[j] = comp[j] = 0.f;
+    }
+    __device__ void load(const float* src, int) {
+        const float4 a = __ldg(reinterpret_cast<const float4*>(src)), b = __ldg(reinterpret_cast<const float4*>(src) + 1);
+        q[0] = a.x, q[1] = a.y, q[2] = a.z, q[3] = a.w, q[4] = b.x, q[5] = b.y, q[6] = b.z, q[7] = b.w;
+    }
+    __device__ __forceinline__ void add(int j, int r, float k) { part[j] = fmaf(q[r], k, part[j]); }
+    __device__ void leaf_done(int, int) {  // Kahan sum of the leaves' partial sums
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const float y = part[j] - comp[j];
+            const float s = acc[j] + y;
+            comp[j] = (s - acc[j]) - y;
+            acc[j] = s;
+            part[j] = 0.f;
         }
     }
-    L[int64_t(a) * (p + 1) + l] = acc;
-}
-
-__global__ void k_am2l(int nb, const int* __restrict__ ptr, const int* __restrict__ src, const AGeo* __restrict__ geo,
-                       int p, const double* __restrict__ S, const double2* __restrict__ M, double2* __restrict__ L) {
-    am2l_body(blockIdx.x, threadIdx.x, nb, ptr, src, geo, p, S, M, L);
-}
-
-// L2L for the boxes in [b0, b1) (one level, parents final): thread l of CTA (b - b0).
-__host__ __device__ inline void al2l_body(int blk, int l, int b0, int b1, const int* __restrict__ parent,
-                                          const AGeo* __restrict__ geo, int p, double2* __restrict__ L) {
-    const int b = b0 + blk;
-    if (b >= b1 || l > p) return;
-    const int pa = parent[b];
-    if (pa < 0) return;
-    const double2 v{(geo[b].cx - geo[pa].cx) / geo[pa].s, (geo[b].cy - geo[pa].cy) / geo[pa].s};
-    double2 acc{0.0, 0.0};
-    double2 vp{1.0, 0.0};  // v^(k-l)
-    double binom = 1.0;    // C(k, l) at k = l
-    for (int k = l; k <= p; ++k) {
-        acc = zadd(acc, zscale(zmul(L[int64_t(pa) * (p + 1) + k], vp), binom));
-        vp = zmul(vp, v);
-        binom = binom * double(k + 1) / double(k + 1 - l);  // C(k+1, l) from C(k, l)
+    __device__ void finish(int) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[j] -= comp[j];
     }
-    L[int64_t(b) * (p + 1) + l] = zadd(L[int64_t(b) * (p + 1) + l], zscale(acc, ldexp(1.0, -l)));
-}
+};
 
-__global__ void k_al2l(int b0, int b1, const int* __restrict__ parent, const AGeo* __restrict__ geo, int p,
-                       double2* __restrict__ L) {
-    al2l_body(blockIdx.x, threadIdx.x, b0, b1, parent, geo, p, L);
-}
-
-// Leaves: CTA of 64 threads per leaf, thread = target cell: local expansion, then the near
-// field over the leaf's near-field sources in list order (sources clamped at their own rho_h).
-// tab: (2R + 1)^2 values T[dy][dx] = log sqrt(dx^2 + dy^2) for |dx|, |dy| <= R (T[0][0] = c0),
-// R covering every same-level near-field offset; S: leaf sums of q (from P2M).
-__host__ __device__ inline void aleaf_body(int i, int c, int nleaf, const int* __restrict__ leafbox,
-                                           const int* __restrict__ ptr, const int* __restrict__ src,
-                                           const AGeo* __restrict__ geo, int p, const double2* __restrict__ L,
-                                           const double* __restrict__ tab, int R, const double* __restrict__ S,
-                                           const double* __restrict__ q, double* __restrict__ p_out) {
-    if (i >= nleaf || c >= 64) return;
-    const int b = leafbox[i];
-    const AGeo g = geo[b];
-    const double2 w = cell_w(c);
-    // Horner: Re sum_l L_l w^l
-    double2 h = L[int64_t(b) * (p + 1) + p];
-    for (int l = p - 1; l >= 0; --l) h = zadd(zmul(h, w), L[int64_t(b) * (p + 1) + l]);
-    const double xt = g.cx + g.s * w.x, yt = g.cy + g.s * w.y;
-    const double logh = log(g.s / 8.0);
-    const int W = 2 * R + 1;
-    double near = 0.0;
-    for (int e = ptr[i]; e < ptr[i + 1]; ++e) {
-        const int j = src[e];
-        const int bj = leafbox[j];
-        const AGeo gs = geo[bj];
-        const double* qs = q + int64_t(j) * 64;
-        if (gs.level == g.level) {  // offsets (source cell - target cell) in cells, |.| <= R
-            const int ox = 8 * (gs.ix - g.ix) - (c & 7) + R, oy = 8 * (gs.iy - g.iy) - (c >> 3) + R;
-            double t = 0.0;
-            for (int cs = 0; cs < 64; ++cs) t += qs[cs] * tab[(oy + (cs >> 3)) * W + ox + (cs & 7)];
-            near += S[bj] * logh + t;
-        } else {
-            const double rho = gs.s / 8.0 * exp(kC0A);
-            for (int cs = 0; cs < 64; ++cs) {
-                const double2 ws = cell_w(cs);
-                const double dx = xt - (gs.cx + gs.s * ws.x), dy = yt - (gs.cy + gs.s * ws.y);
-                const double r = fmax(sqrt(dx * dx + dy * dy), rho);
-                near += qs[cs] * log(r);
+template <>
+struct NearAcc<double> {
+    typedef int2 Kv;  // (high, low) halves
+    long long hh[8], mid[8];
+    double acc[8];
+    int qh[8], ql[8];
+    __device__ void init() {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            hh[j] = mid[j] = 0;
+            acc[j] = 0.0;
+        }
+    }
+    // the row's fixed-point weights, shifted right (rounded) to the common exponent
+    __device__ void load(const long long* src, int sh) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const longlong2 v2 = __ldg(reinterpret_cast<const longlong2*>(src) + i);
+            long long v[2] = {v2.x, v2.y};
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                if (sh > 0) v[u] = sh > 60 ? 0 : (v[u] + (1ll << (sh - 1))) >> sh;
+                const int l = int(unsigned(v[u]) << 4) >> 4;
+                ql[2 * i + u] = l;
+                qh[2 * i + u] = int((v[u] - l) >> 28);
             }
         }
     }
-    p_out[int64_t(i) * 64 + c] = (h.x + near) * kInv2PiA;
-}
+    __device__ __forceinline__ void add(int j, int r, int2 k) {
+        hh[j] += (long long)qh[r] * k.x;
+        mid[j] += (long long)qh[r] * k.y;
+        mid[j] += (long long)ql[r] * k.x;
+    }
+    __device__ void drain(int et) {
+        const double f1 = __hiloint2double((1023 + et - 50) << 20, 0), f2 = f1 * 3.7252902984619140625e-09;  // 2^-28
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            acc[j] = fma(double(hh[j]), f1, fma(double(mid[j]), f2, acc[j]));
+            hh[j] = mid[j] = 0;
+        }
+    }
+    __device__ void leaf_done(int n, int et) {
+        if ((n & 31) == 31) drain(et);
+    }
+    __device__ void finish(int et) { drain(et); }
+};
 
-__global__ void k_aleaf(int nleaf, const int* __restrict__ leafbox, const int* __restrict__ ptr,
-                        const int* __restrict__ src, const AGeo* __restrict__ geo, int p,
-                        const double2* __restrict__ L, const double* __restrict__ tab, int R,
-                        const double* __restrict__ S, const double* __restrict__ q, double* __restrict__ p_out) {
-    aleaf_body(blockIdx.x, threadIdx.x, nleaf, leafbox, ptr, src, geo, p, L, tab, R, S, q, p_out);
+constexpr int kLeafThreads = 288;  // eight near-field warps and the path's warp
+
+template <typename T>
+__global__ void __launch_bounds__(kLeafThreads)
+k_aleaf(const int* __restrict__ leafbox, const int* __restrict__ anc, int nlev, const int* __restrict__ ptr,
+        const APair* __restrict__ pairs, const AGeo* __restrict__ geo, int p, const AConst<T>* __restrict__ ct,
+        const typename cplx_of<T>::type* __restrict__ L, const double* __restrict__ L0,
+        const typename NearAcc<T>::Kv* __restrict__ te, int R, const typename NearAcc<T>::Kv* __restrict__ to, int Wo,
+        const double* __restrict__ S, const T* __restrict__ q, const typename NearSrc<T>::type* __restrict__ qfix,
+        const int* __restrict__ qexp, T* __restrict__ p_out) {
+    typedef typename cplx_of<T>::type C;
+    typedef typename NearAcc<T>::Kv Kv;
+    extern __shared__ __align__(16) unsigned char smem_leaf[];
+    Kv* tab = reinterpret_cast<Kv*>(smem_leaf);  // (R + 1) rows of stride R + 2
+    __shared__ T near[4][64];
+    __shared__ C Ls[kTP];
+    __shared__ double c0s;
+    const int i = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int b = leafbox[i];
+    const int e0 = ptr[i], e1 = ptr[i + 1];
+    const int W = R + 2;
+    for (int m = tid; m < (R + 1) * W; m += kLeafThreads) tab[m] = te[m];
+    __syncthreads();
+    if (warp < 8) {
+        const int g = warp >> 1, sy = lane & 7, ty = (lane >> 3) + 4 * (warp & 1);
+        int et = -900;
+        if constexpr (sizeof(T) == 8) {  // the largest exponent of the target's sources
+            for (int e = e0 + lane; e < e1; e += 32) {
+                const int x = qexp[pairs[e].src];
+                if (x != kBadExp) et = max(et, x);
+            }
+            et = __reduce_max_sync(0xffffffffu, et);
+        }
+        NearAcc<T> A;
+        A.init();
+        int n = 0;
+        for (int e = e0 + g; e < e1; e += 4) {
+            const APair pr = pairs[e];
+            int sh = 0;
+            bool direct = pr.kind == kDirect;
+            if constexpr (sizeof(T) == 8) {
+                const int x = qexp[pr.src];
+                direct = direct || x == kBadExp;
+                sh = et - x;
+            }
+            if (!direct) {
+                A.load(qfix + int64_t(pr.src) * 64 + sy * 8, sh);
+                if (pr.kind == 0) {
+                    const Kv* kr = tab + abs(pr.oy + sy - ty) * W;
+                    Kv kc[15];
+#pragma unroll
+                    for (int m = 0; m < 15; ++m) kc[m] = kr[abs(pr.ox - 7 + m)];
+#pragma unroll
+                    for (int r = 0; r < 8; ++r)
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) A.add(j, r, kc[r - j + 7]);
+                } else {
+                    const int kap = abs(pr.kind);
+                    const int my = pr.kind < 0 ? pr.oy + (sy << kap) - ty : pr.oy + sy - (ty << kap);
+                    const Kv* kr = to + (my ^ (my >> 31)) * Wo;
+                    if (kap == 1) {
+                        Kv kc[22];
+                        const int m0 = pr.kind < 0 ? pr.ox - 7 : pr.ox - 14;
+#pragma unroll
+                        for (int m = 0; m < 22; ++m) kc[m] = __ldg(kr + ((m0 + m) ^ ((m0 + m) >> 31)));
+                        if (pr.kind < 0) {
+#pragma unroll
+                            for (int r = 0; r < 8; ++r)
+#pragma unroll
+                                for (int j = 0; j < 8; ++j) A.add(j, r, kc[2 * r - j + 7]);
+                        } else {
+#pragma unroll
+                            for (int r = 0; r < 8; ++r)
+#pragma unroll
+                                for (int j = 0; j < 8; ++j) A.add(j, r, kc[r - 2 * j + 14]);
+                        }
+                    } else {
+                        const int sr = pr.kind < 0 ? kap : 0, sj = pr.kind < 0 ? 0 : kap;
+#pragma unroll
+                        for (int r = 0; r < 8; ++r)
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) {
+                                const int m = pr.ox + (r << sr) - (j << sj);
+                                A.add(j, r, __ldg(kr + (m ^ (m >> 31))));
+                            }
+                    }
+                }
+            } else if constexpr (sizeof(T) == 8) {
+                const AGeo gt = geo[b], gs = geo[leafbox[pr.src]];
+                const double rho = gs.s / 8.0 * exp(kC0A);
+                const double yt = gt.cy + gt.s * ((ty + 0.5) / 8.0 - 0.5), ys = gs.cy + gs.s * ((sy + 0.5) / 8.0 - 0.5);
+                for (int r = 0; r < 8; ++r) {
+                    const double xs = gs.cx + gs.s * ((r + 0.5) / 8.0 - 0.5), qv = q[int64_t(pr.src) * 64 + sy * 8 + r];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const double dx = gt.cx + gt.s * ((j + 0.5) / 8.0 - 0.5) - xs, dy = yt - ys;
+                        A.acc[j] += qv * log(fmax(sqrt(dx * dx + dy * dy), rho));
+                    }
+                }
+            } else {
+                // source cell centres relative to the target cell, in units of the target's cell side
+                const AGeo gt = geo[b], gs = geo[leafbox[pr.src]];
+                const double hc = gt.s / 8.0;
+                const float ox = float((gs.cx - 0.5 * gs.s - (gt.cx - 0.5 * gt.s)) / hc) - 0.5f;
+                const float oy = float((gs.cy - 0.5 * gs.s - (gt.cy - 0.5 * gt.s)) / hc) - (ty + 0.5f);
+                const float step = float(gs.s / 8.0 / hc);      // source cell side / target cell side
+                const float rho = step * 0.34604881609982794f;  // rho_h of the source cell: exp(pi/4 - 3/2 - ln2/2) h
+                const float lhc = float(log(hc));
+                const float dy = oy + (sy + 0.5f) * step;
+                for (int r = 0; r < 8; ++r) {
+                    const float qv = q[int64_t(pr.src) * 64 + sy * 8 + r];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const float dx = ox + (r + 0.5f) * step - float(j);
+                        A.part[j] = fmaf(qv, logf(fmaxf(sqrtf(dx * dx + dy * dy), rho)) + lhc, A.part[j]);
+                    }
+                }
+            }
+            A.leaf_done(n++, et);
+        }
+        A.finish(et);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {  // the eight source rows (lanes of one target row), then one lane a target
+            T v = A.acc[j];
+            v += __shfl_xor_sync(0xffffffffu, v, 1);
+            v += __shfl_xor_sync(0xffffffffu, v, 2);
+            v += __shfl_xor_sync(0xffffffffu, v, 4);
+            if (sy == j) near[g][ty * 8 + j] = v;
+        }
+    } else {
+        // the path's locals: cur is this lane's coefficient of the box above
+        const int lev = geo[b].level;
+        double c0 = 0.0;
+        C cur = cx<T>(T(0), T(0));
+        for (int l = 0; l <= lev; ++l) {
+            const int bx = anc[int64_t(i) * nlev + l];
+            const C m = lane <= p ? L[int64_t(bx) * kTP + lane] : cx<T>(T(0), T(0));
+            const double m0 = L0[bx];
+            if (l > 0) {
+                const AGeo gb = geo[bx];
+                const int qd = (gb.ix & 1) + 2 * (gb.iy & 1);
+                __syncwarp();
+                Ls[lane] = cmulT<T>(cur, ct->Z[qd][lane]);
+                __syncwarp();
+                C y = cx<T>(T(0), T(0));
+#pragma unroll 4
+                for (int k = 1; k <= p; ++k) {
+                    const T r = ct->l2l[k][lane];
+                    const C v = Ls[k];
+                    y.x = fma(r, v.x, y.x);
+                    y.y = fma(r, v.y, y.y);
+                }
+                c0 += double(y.x);  // lane 0: Re sum_k zeta^k L_k
+                cur = cmulT<T>(y, ct->ZI[qd][lane]);
+            }
+            cur.x += m.x;
+            cur.y += m.y;
+            c0 += m0;
+        }
+        // log(unit) S over the near sources served from a table
+        double sl = 0.0;
+        for (int e = e0 + lane; e < e1; e += 32) {
+            const APair pr = pairs[e];
+            bool direct = pr.kind == kDirect;
+            if constexpr (sizeof(T) == 8) direct = direct || qexp[pr.src] == kBadExp;
+            const int unit = pr.kind == 0 ? lev + 3 : lev + 4 + max(pr.kind, 0);
+            if (!direct) sl += S[leafbox[pr.src]] * (-kLn2A * unit);
+        }
+        for (int o = 16; o > 0; o >>= 1) sl += __shfl_xor_sync(0xffffffffu, sl, o);
+        __syncwarp();
+        Ls[lane] = cur;
+        if (lane == 0) c0s = c0 + sl;
+    }
+    __syncthreads();
+    if (tid < 64) {
+        T ser = T(0);
+#pragma unroll 4
+        for (int l = 1; l <= p; ++l) {
+            const C v = ct->V[l][tid], m = Ls[l];
+            ser = fma(m.x, v.x, fma(-m.y, v.y, ser));
+        }
+        const T nr = (near[0][tid] + near[1][tid]) + (near[2][tid] + near[3][tid]);
+        p_out[int64_t(i) * 64 + tid] = T((c0s + double(ser) + double(nr)) * kInv2PiA);
+    }
 }
 
 // Surface pressure at off-grid points by the tree-code over the adaptive tree (Sec. 2.3.1's
-// targets; Appendix A.2's group acceptance): depth-first from the root, a box is accepted for
-// the point when its half-diagonal r is below theta d (d the distance from its centre) and its
-// multipole is evaluated there, S log|w| - Re sum_k M_k (s / w)^k with w = z - c (Eq.
-// pressTruncated about the box centre); a leaf that is not accepted is summed directly over its
-// 64 cells, each clamped at its own rho_h; any other box opens its four children.  One thread
-// per point; the stack holds at most 3 boxes per level plus 4.
-constexpr int kSurfStack = 3 * 21 + 4;
+// targets; Appendix A.2's group acceptance), one warp per point: level by level from the root, a
+// box is accepted for the point when its half-diagonal r is below theta d (d the distance from
+// its centre) and its multipole is evaluated there, S log|w| - Re sum_k M_k (s / w)^k with w = z - c
+// (Eq. pressTruncated about the box centre); a leaf that is not accepted is summed directly over
+// its 64 cells, each clamped at its own rho_h; any other box opens its four children.  Accepted
+// boxes are collected and evaluated 32 at a time, a lane each, so the FP64 pipe, which bounds
+// the walk, works on full warps; logarithms come from the table method.  A level's open boxes lie
+// within s / (sqrt 2 theta) of the point: at most 37 for theta >= 0.25, 148 children.
+constexpr int kSurfCand = 256;
 
-__host__ __device__ inline void asurf_body(int i, int npts, const double* __restrict__ pts, const AGeo* __restrict__ geo,
-                                           const int* __restrict__ fchild, const int* __restrict__ boxleaf, int p,
-                                           const double* __restrict__ S, const double2* __restrict__ M,
-                                           const double* __restrict__ q, double theta, double* __restrict__ P_out,
-                                           bool* overflow_out) {
-    if (i >= npts) return;
+__global__ void __launch_bounds__(128) k_asurf(int npts, const double* __restrict__ pts, const AGeo* __restrict__ geo,
+                                               const int* __restrict__ fchild, const int* __restrict__ boxleaf, int p,
+                                               const double* __restrict__ S, const double2* __restrict__ M,
+                                               const double* __restrict__ q, double theta, double* __restrict__ P_out,
+                                               int* __restrict__ err) {
+    __shared__ int cand[4][2][kSurfCand];
+    __shared__ int acc_list[4][64];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int i = blockIdx.x * 4 + w;
+    if (i >= npts) return;  // warp-uniform, no block barriers
     const double zx = pts[2 * i], zy = pts[2 * i + 1];
-    int stack[kSurfStack];
-    int top = 0;
-    stack[top++] = 0;
+    const double th2 = theta * theta, rho8 = exp(kC0A) / 8.0;
+    const unsigned below = (1u << lane) - 1u;
     double acc = 0.0;
     bool overflow = false;
-    const double th2 = theta * theta;
-    while (top > 0) {
-        const int b = stack[--top];
+    const auto evaluate = [&](int b) {  // an accepted box: u = s / w, Horner for sum_k M_k u^k
         const AGeo g = geo[b];
         const double dx = zx - g.cx, dy = zy - g.cy;
-        const double d2 = dx * dx + dy * dy;
-        if (0.5 * g.s * g.s < th2 * d2) {
-            // u = s / w; Horner for sum_k M_k u^k
-            const double2 u = zscale(double2{dx / d2, -dy / d2}, g.s);
-            const double2* Mb = M + int64_t(b) * (p + 1);
-            double2 h = Mb[p];
-            for (int k = p - 1; k >= 1; --k) h = zadd(zmul(h, u), Mb[k]);
-            const double2 ser = zmul(h, u);
-            acc += S[b] * 0.5 * log(d2) - ser.x;
-        } else if (fchild[b] < 0) {
-            const int lf = boxleaf[b];
-            const double* qs = q + int64_t(lf) * 64;
-            const double rho = g.s / 8.0 * exp(kC0A);
-            for (int c = 0; c < 64; ++c) {
-                const double2 w = cell_w(c);
-                const double ex = zx - (g.cx + g.s * w.x), ey = zy - (g.cy + g.s * w.y);
-                acc += qs[c] * log(fmax(sqrt(ex * ex + ey * ey), rho));
-            }
-        } else if (top + 4 <= kSurfStack) {
-            for (int c = 3; c >= 0; --c) stack[top++] = fchild[b] + c;
-        } else {
-            overflow = true;
+        const double d2 = dx * dx + dy * dy, sd = g.s / d2;
+        const double2 u{dx * sd, -dy * sd};
+        const double2* Mb = M + int64_t(b) * kTP;
+        double2 h = Mb[p];
+#pragma unroll 4
+        for (int k = p - 1; k >= 1; --k) {
+            const double2 m = Mb[k];
+            h = double2{fma(h.x, u.x, fma(-h.y, u.y, m.x)), fma(h.x, u.y, fma(h.y, u.x, m.y))};
         }
+        acc = fma(S[b], 0.5 * pp::log_table(d2), acc) - (h.x * u.x - h.y * u.y);
+    };
+    if (lane == 0) cand[w][0][0] = 0;
+    __syncwarp();
+    int cur = 0, n = 1, na = 0;
+    while (n > 0) {
+        int next = 0;
+        for (int base = 0; base < n; base += 32) {
+            const bool act = base + lane < n;
+            const int b = act ? cand[w][cur][base + lane] : 0;
+            bool take = false, leaf = false, inner = false;
+            int fc = -1;
+            if (act) {
+                const AGeo g = geo[b];
+                const double dx = zx - g.cx, dy = zy - g.cy;
+                take = 0.5 * g.s * g.s < th2 * (dx * dx + dy * dy);
+                fc = fchild[b];
+                leaf = !take && fc < 0;
+                inner = !take && fc >= 0;
+            }
+            const unsigned tm = __ballot_sync(0xffffffffu, take);
+            if (take) acc_list[w][na + __popc(tm & below)] = b;
+            na += __popc(tm);
+            __syncwarp();
+            if (na >= 32) {
+                evaluate(acc_list[w][lane]);
+                na -= 32;
+                const int v = acc_list[w][32 + lane];
+                __syncwarp();
+                acc_list[w][lane] = v;
+                __syncwarp();
+            }
+            for (unsigned lm = __ballot_sync(0xffffffffu, leaf); lm; lm &= lm - 1) {
+                const int lb = __shfl_sync(0xffffffffu, b, __ffs(lm) - 1);
+                const AGeo g = geo[lb];
+                const double* qs = q + int64_t(boxleaf[lb]) * 64;
+                const double rho = g.s * rho8, rho2 = rho * rho;
+                const double2 c0 = cell_w(lane);
+                const double ex = zx - fma(g.s, c0.x, g.cx), ey = zy - fma(g.s, c0.y, g.cy), ey1 = ey - 0.5 * g.s;
+                const double x2 = ex * ex;  // cells `lane` and `lane + 32`, four rows on
+                acc = fma(qs[lane], 0.5 * pp::log_table(fmax(fma(ey, ey, x2), rho2)), acc);
+                acc = fma(qs[lane + 32], 0.5 * pp::log_table(fmax(fma(ey1, ey1, x2), rho2)), acc);
+            }
+            const unsigned im = __ballot_sync(0xffffffffu, inner);
+            if (inner) {
+                const int at = next + 4 * __popc(im & below);
+                if (at + 4 <= kSurfCand) {
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) cand[w][cur ^ 1][at + c] = fc + c;
+                } else {
+                    overflow = true;
+                }
+            }
+            next += 4 * __popc(im);
+        }
+        __syncwarp();
+        cur ^= 1;
+        n = min(next, kSurfCand);
     }
-    P_out[i] = acc * kInv2PiA;
-    *overflow_out = overflow;
-}
-
-__global__ void k_asurf(int npts, const double* __restrict__ pts, const AGeo* __restrict__ geo,
-                        const int* __restrict__ fchild, const int* __restrict__ boxleaf, int p,
-                        const double* __restrict__ S, const double2* __restrict__ M, const double* __restrict__ q,
-                        double theta, double* __restrict__ P_out, int* __restrict__ err) {
-    bool overflow = false;
-    asurf_body(blockIdx.x * blockDim.x + threadIdx.x, npts, pts, geo, fchild, boxleaf, p, S, M, q, theta, P_out,
-               &overflow);
+    if (lane < na) evaluate(acc_list[w][lane]);
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) P_out[i] = acc * kInv2PiA;
     if (overflow) atomicExch(err, 1);
 }
 
@@ -319,13 +708,66 @@ cudaError_t upload(std::vector<void*>& bufs, T** dst, const std::vector<T>& src,
     return e;
 }
 
-// Host arrays of one solve: box geometry, leaf -> box, level ranges (boxes are stored level by
-// level, parents first), and both interaction lists as CSR by target.
+template <typename T>
+cudaError_t dev_alloc(std::vector<void*>& bufs, T** dst, size_t n) {
+    const cudaError_t e = cudaMalloc(reinterpret_cast<void**>(dst), sizeof(T) * std::max<size_t>(n, 1));
+    if (e == cudaSuccess) bufs.push_back(*dst);
+    return e;
+}
+
+// Host arrays of one solve: box geometry, leaf -> box, each leaf's path, and both interaction
+// lists as CSR by target.
 struct AdaptivePrep {
-    int nb = 0, nleaf = 0, L = 0, R = 0;
+    int nb = 0, nleaf = 0, L = 0, R = 0, Wo = 1;
     std::vector<AGeo> geo;
-    std::vector<int> fchild, parent, leafbox, boxleaf, lev_start, m2l_ptr, m2l_src, p2p_ptr, p2p_src;
-    std::vector<double> tab;  // the same-level near-field table, (2R + 1)^2
+    std::vector<int> fchild, parent, leafbox, boxleaf, anc, m2l_ptr, p2p_ptr;
+    std::vector<int2> m2l;     // source box, operator
+    std::vector<APair> p2p;
+    std::vector<double> op;    // tau_x, tau_y, rho per distinct operator
+};
+
+// Index of the operator (level difference, offset in units of the deepest box's half side) in a
+// table that grows by insertion: open addressing over the integer key.
+struct OpTable {
+    struct Key {
+        int64_t x, y;
+        int dl;
+    };
+    std::vector<Key> keys;
+    std::vector<int> slot;
+    OpTable() : slot(1024, -1) {}
+    static size_t hash(const Key& k) {
+        uint64_t h = uint64_t(k.x) * 0x9E3779B97F4A7C15ull ^ uint64_t(k.y) * 0xC2B2AE3D27D4EB4Full ^
+                     uint64_t(k.dl + 64) * 0x165667B19E3779F9ull;
+        return size_t(h ^ (h >> 29));
+    }
+    int find(const Key& k, bool* fresh) {
+        *fresh = false;
+        for (size_t i = hash(k);; ++i) {
+            int& s = slot[i & (slot.size() - 1)];
+            if (s < 0) {
+                *fresh = true;
+                s = int(keys.size());
+                keys.push_back(k);
+                const int id = s;
+                if (2 * keys.size() > slot.size()) grow();
+                return id;
+            }
+            const Key& o = keys[s];
+            if (o.x == k.x && o.y == k.y && o.dl == k.dl) return s;
+        }
+    }
+    void grow() {
+        slot.assign(2 * slot.size(), -1);
+        for (size_t n = 0; n < keys.size(); ++n)
+            for (size_t i = hash(keys[n]);; ++i) {
+                int& s = slot[i & (slot.size() - 1)];
+                if (s < 0) {
+                    s = int(n);
+                    break;
+                }
+            }
+    }
 };
 
 int prepare_adaptive(pp_atree tree, AdaptivePrep& a) {
@@ -345,152 +787,217 @@ int prepare_adaptive(pp_atree tree, AdaptivePrep& a) {
         a.geo.resize(nb);
         a.leafbox.assign(a.nleaf, -1);
         a.boxleaf = leaf;
-        a.lev_start.assign(L + 2, nb);
-        a.m2l_ptr.assign(nb + 1, 0);
-        a.m2l_src.resize(nm);
-        a.p2p_ptr.assign(a.nleaf + 1, 0);
-        a.p2p_src.resize(np2);
-        for (int b = nb - 1; b >= 0; --b) a.lev_start[level[b]] = b;
         for (int b = 0; b < nb; ++b) {
             const double s = std::ldexp(1.0, -level[b]);
             a.geo[b] = AGeo{(ix[b] + 0.5) * s, (iy[b] + 0.5) * s, s, level[b], ix[b], iy[b]};
             if (leaf[b] >= 0) a.leafbox[leaf[b]] = b;
         }
-        for (int e = 0; e < nm; ++e) {  // pairs are sorted by target
-            ++a.m2l_ptr[m2l[2 * e] + 1];
-            a.m2l_src[e] = m2l[2 * e + 1];
+        a.anc.assign(size_t(a.nleaf) * (L + 1), 0);
+        for (int i = 0; i < a.nleaf; ++i)
+            for (int b = a.leafbox[i]; b >= 0; b = a.parent[b]) a.anc[size_t(i) * (L + 1) + level[b]] = b;
+        // translations: pairs are sorted by target; the operator depends on the level difference
+        // and the offset in target sides
+        a.m2l_ptr.assign(nb + 1, 0);
+        a.m2l.resize(nm);
+        OpTable ops;
+        for (int e = 0; e < nm; ++e) {
+            const int t = m2l[2 * e], s = m2l[2 * e + 1];
+            ++a.m2l_ptr[t + 1];
+            const int f = std::max(level[t], level[s]);
+            const auto at = [&](int i, int l) { return (2 * int64_t(i) + 1) << (f - l); };
+            const OpTable::Key k{at(ix[s], level[s]) - at(ix[t], level[t]), at(iy[s], level[s]) - at(iy[t], level[t]),
+                                 level[s] - level[t]};
+            bool fresh;
+            const int id = ops.find(k, &fresh);
+            if (fresh) {
+                const double unit = std::ldexp(0.5, level[t] - f);  // half the finer side, in target sides
+                a.op.push_back(double(k.x) * unit);
+                a.op.push_back(double(k.y) * unit);
+                a.op.push_back(std::ldexp(1.0, -k.dl));
+            }
+            a.m2l[e] = make_int2(s, id);
         }
         for (int b = 0; b < nb; ++b) a.m2l_ptr[b + 1] += a.m2l_ptr[b];
+        // near-field pairs with their table offsets, and the sides of the two tables
+        a.p2p_ptr.assign(a.nleaf + 1, 0);
+        a.p2p.resize(np2);
+        int dmax = 0, odd = -1;
+        const auto fold = [](int64_t m) { return m >= 0 ? m : ~m; };
         for (int e = 0; e < np2; ++e) {
             ++a.p2p_ptr[p2p[2 * e] + 1];
-            a.p2p_src[e] = p2p[2 * e + 1];
+            const AGeo &gt = a.geo[a.leafbox[p2p[2 * e]]], &gs = a.geo[a.leafbox[p2p[2 * e + 1]]];
+            const int kind = gs.level - gt.level, k = std::abs(kind);
+            APair pr{p2p[2 * e + 1], kind, 0, 0};
+            if (kind == 0) {
+                pr.ox = 8 * (gs.ix - gt.ix);
+                pr.oy = 8 * (gs.iy - gt.iy);
+                dmax = std::max(dmax, std::max(std::abs(gs.ix - gt.ix), std::abs(gs.iy - gt.iy)));
+            } else if (k <= kMaxKappa) {
+                const auto off = [&](int64_t is, int64_t it) {
+                    return kind < 0 ? ((8 * is) << k) + (int64_t(1) << (k - 1)) - 1 - 8 * it
+                                    : 8 * is - ((8 * it) << k) - (int64_t(1) << (k - 1));
+                };
+                const int64_t lo = kind < 0 ? 7 : 7 << k, hi = kind < 0 ? 7 << k : 7;
+                const int64_t ox = off(gs.ix, gt.ix), oy = off(gs.iy, gt.iy);
+                const int64_t big = std::max(std::max(fold(ox - lo), fold(ox + hi)), std::max(fold(oy - lo), fold(oy + hi)));
+                if (big < kMaxOddSide) {
+                    pr.ox = int(ox);
+                    pr.oy = int(oy);
+                    odd = std::max(odd, int(big));
+                } else {
+                    pr.kind = kDirect;
+                }
+            } else {
+                pr.kind = kDirect;
+            }
+            a.p2p[e] = pr;
         }
         for (int i = 0; i < a.nleaf; ++i) a.p2p_ptr[i + 1] += a.p2p_ptr[i];
-        // the largest same-level near-field leaf offset, and the table of log|D| over cell offsets
-        int dmax = 0;
-        for (int e = 0; e < np2; ++e) {
-            const AGeo& gt = a.geo[a.leafbox[p2p[2 * e]]];
-            const AGeo& gs = a.geo[a.leafbox[p2p[2 * e + 1]]];
-            if (gt.level == gs.level) dmax = std::max(dmax, std::max(std::abs(gs.ix - gt.ix), std::abs(gs.iy - gt.iy)));
-        }
         a.R = 8 * dmax + 7;
-        const int W = 2 * a.R + 1;
-        a.tab.resize(size_t(W) * W);
-        for (int dy = -a.R; dy <= a.R; ++dy)
-            for (int dx = -a.R; dx <= a.R; ++dx)
-                a.tab[size_t(dy + a.R) * W + dx + a.R] =
-                    (dx == 0 && dy == 0) ? kC0A : 0.5 * std::log(double(dx * dx + dy * dy));
+        a.Wo = (odd + 1) | 1;
     } catch (const std::bad_alloc&) {
         return PP_ERR_OOM;
     }
     return PP_OK;
 }
 
-// What a tree keeps between solves: the prepared arrays on the device and the expansions
-// (sized for the largest order solved so far).
+// What a tree keeps between solves: the prepared arrays on the device and, per precision (set up
+// on its first solve), the constant tables, the operators' diagonals, the near-field tables and
+// the expansions.
+template <typename T>
+struct AdaptiveSide {
+    typedef typename cplx_of<T>::type C;
+    bool ready = false;
+    AConst<T>* ct = nullptr;
+    C *op = nullptr, *M = nullptr, *L = nullptr;
+    typename OpLog<T>::type* oplog = nullptr;
+    typename NearAcc<T>::Kv *te = nullptr, *to = nullptr;
+};
+
 struct AdaptiveState {
     AdaptivePrep a;
     std::vector<void*> bufs;
-    int *d_leafbox = nullptr, *d_fchild = nullptr, *d_parent = nullptr, *d_mptr = nullptr, *d_msrc = nullptr,
-        *d_pptr = nullptr, *d_psrc = nullptr, *d_boxleaf = nullptr, *d_err = nullptr;
+    int *d_leafbox = nullptr, *d_fchild = nullptr, *d_parent = nullptr, *d_mptr = nullptr, *d_pptr = nullptr,
+        *d_anc = nullptr, *d_boxleaf = nullptr, *d_err = nullptr, *d_qexp = nullptr;
+    int2* d_mpair = nullptr;
+    APair* d_ppair = nullptr;
+    unsigned* d_cnt = nullptr;  // arrivals per box, zero between solves
     AGeo* d_geo = nullptr;
-    double *d_tab = nullptr, *d_S = nullptr;
-    double2 *d_M = nullptr, *d_L = nullptr;
-    int p_cap = 0;
-    int last_p = 0;  // order of the last solve: the multipoles the surface tree-code reads
-    // mixed-precision solve (set up on its first call): FP32 expansions with the FP64 monopoles
-    // and constant terms, per-pair translation geometry, the shift and P2M tables, the FP32
-    // near-field table
-    bool mixed_ready = false;
-    float2 *d_Mf = nullptr, *d_Lf = nullptr;
-    double* d_L0 = nullptr;
-    float4* d_mgeo = nullptr;   // per M2L pair: tau (target side units), rho, unused
-    double* d_mlog = nullptr;   // per M2L pair: log|tau| + log s_target
-    float2 *d_Wf = nullptr, *d_Af = nullptr, *d_Bf = nullptr, *d_Cf = nullptr;
-    float* d_tabf = nullptr;
+    double *d_S = nullptr, *d_L0 = nullptr;
+    float2* d_Sf = nullptr;
+    long long* d_qfix = nullptr;
+    AdaptiveSide<double> f64;
+    AdaptiveSide<float> mixed;
+    int last_p = 0;  // order of the last FP64 solve: the multipoles the surface tree-code reads
 };
 
 void release_state(void* v) {
     AdaptiveState* s = static_cast<AdaptiveState*>(v);
     for (void* b : s->bufs) cudaFree(b);
-    cudaFree(s->d_M);
-    cudaFree(s->d_L);
     delete s;
 }
 
-// Host tables of the mixed-precision solve, order up to kMaxOrderA (stride kTP = 31), built in
-// FP64: W[c][k] = w_c^k / k (P2M at the 64 cells), and per child quadrant q with
-// u_q = (c_child - c_parent) / s_parent = (+-1/4, +-1/4):
-//   B[q][k] = u_q^k / k, A[q][l][k] = 2^-l u_q^(k-l) C(k-1, l-1) (M2M),
-//   C[q][k][l] = 2^-l C(k, l) u_q^(k-l) (L2L).
-constexpr int kTP = kMaxOrderA + 1;
-
-struct MixedTables {
-    std::vector<float2> W, A, B, C;
-};
-
-MixedTables mixed_tables() {
-    MixedTables t;
-    t.W.assign(size_t(64) * kTP, float2{0.f, 0.f});
-    t.A.assign(size_t(4) * kTP * kTP, float2{0.f, 0.f});
-    t.B.assign(size_t(4) * kTP, float2{0.f, 0.f});
-    t.C.assign(size_t(4) * kTP * kTP, float2{0.f, 0.f});
-    auto f2 = [](double2 z) { return float2{float(z.x), float(z.y)}; };
-    auto zpow = [](double2 z, int k) {
-        double2 r{1.0, 0.0};
-        for (int j = 0; j < k; ++j) r = zmul(r, z);
-        return r;
+template <typename T>
+AConst<T>* fill_const() {
+    AConst<T>* c = new (std::nothrow) AConst<T>();
+    if (!c) return nullptr;
+    const auto put = [](typename cplx_of<T>::type& d, double2 z) {
+        d.x = T(z.x);
+        d.y = T(z.y);
     };
-    auto binom = [](int n, int r) {
-        double c = 1.0;
-        for (int i = 1; i <= r; ++i) c = c * double(n - r + i) / double(i);
-        return c;
+    const auto binom = [](int n, int r) {
+        if (r < 0 || r > n) return 0.0;
+        double v = 1.0;
+        for (int i = 1; i <= r; ++i) v = v * double(n - r + i) / double(i);
+        return v;
     };
-    for (int c = 0; c < 64; ++c)
-        for (int k = 1; k < kTP; ++k) t.W[size_t(c) * kTP + k] = f2(zscale(zpow(cell_w(c), k), 1.0 / k));
-    for (int q = 0; q < 4; ++q) {
-        const double2 u{((q & 1) - 0.5) * 0.5, ((q >> 1) - 0.5) * 0.5};
-        for (int k = 1; k < kTP; ++k) {
-            t.B[size_t(q) * kTP + k] = f2(zscale(zpow(u, k), 1.0 / k));
-            for (int l = 1; l <= k; ++l)
-                t.A[(size_t(q) * kTP + l) * kTP + k] = f2(zscale(zpow(u, k - l), std::ldexp(binom(k - 1, l - 1), -l)));
+    for (int k = 0; k < kTP; ++k)
+        for (int l = 0; l < kTP; ++l) {
+            c->m2l[k][l] = T(k < 1 ? 0.0 : l == 0 ? 1.0 : binom(l + k - 1, k - 1));
+            c->m2m[k][l] = T(l < 1 ? 0.0 : k == 0 ? 1.0 / l : binom(l - 1, k - 1));
+            c->l2l[k][l] = T(binom(k, l));
         }
-        for (int k = 0; k < kTP; ++k)
-            for (int l = 0; l <= k; ++l)
-                t.C[(size_t(q) * kTP + k) * kTP + l] = f2(zscale(zpow(u, k - l), std::ldexp(binom(k, l), -l)));
+    for (int n = 0; n < 64; ++n) {
+        double2 w{1.0, 0.0};
+        for (int k = 0; k < kTP; ++k) {
+            put(c->V[k][n], w);
+            put(c->W[n][k], k ? zscale(w, 1.0 / k) : double2{0.0, 0.0});
+            w = zmul(w, cell_w(n));
+        }
     }
-    return t;
+    for (int n = 0; n < 4; ++n) {
+        const double2 z{((n & 1) - 0.5) * 0.5, ((n >> 1) - 0.5) * 0.5};
+        const double2 i2{z.x * 4.0, -z.y * 4.0};  // 1 / (2 zeta), |2 zeta|^2 = 1/2
+        double2 a{1.0, 0.0}, b{1.0, 0.0};
+        for (int k = 0; k < kTP; ++k) {
+            put(c->Z[n][k], a);
+            put(c->ZI[n][k], b);
+            a = zmul(a, z);
+            b = zmul(b, i2);
+        }
+    }
+    return c;
 }
 
-cudaError_t setup_mixed(AdaptiveState* s, cudaStream_t st) {
+void put_log(double& d, double v) { d = v; }
+void put_log(float2& d, double v) { d = make_float2(float(v), float(v - double(float(v)))); }
+void put_kernel(float& d, double v) { d = float(v); }
+void put_kernel(int2& d, double v) {  // 2^-52 units as h 2^28 + l, |l| <= 2^27
+    const int64_t t = std::llrint(std::ldexp(v, 52));
+    const int l = int(uint32_t(t) << 4) >> 4;
+    d = make_int2(int((t - l) >> 28), l);
+}
+
+template <typename T>
+cudaError_t setup_side(AdaptiveState* s, AdaptiveSide<T>& d, cudaStream_t st) {
+    typedef typename cplx_of<T>::type C;
     const AdaptivePrep& a = s->a;
-    std::vector<float4> mg(a.m2l_src.size());
-    std::vector<double> ml(a.m2l_src.size());
-    for (int t = 0; t < a.nb; ++t)
-        for (int e = a.m2l_ptr[t]; e < a.m2l_ptr[t + 1]; ++e) {
-            const AGeo& gt = a.geo[t];
-            const AGeo& gs = a.geo[a.m2l_src[e]];
-            const double tx = (gs.cx - gt.cx) / gt.s, ty = (gs.cy - gt.cy) / gt.s;
-            mg[e] = make_float4(float(tx), float(ty), float(gs.s / gt.s), 0.f);
-            ml[e] = 0.5 * std::log(tx * tx + ty * ty) + std::log(gt.s);
-        }
-    std::vector<float> tf(a.tab.size());
-    for (size_t i = 0; i < tf.size(); ++i) tf[i] = float(a.tab[i]);
-    const MixedTables mt = mixed_tables();
+    const size_t nop = a.op.size() / 3;
+    AConst<T>* hc = fill_const<T>();
+    if (!hc) return cudaErrorMemoryAllocation;
     cudaError_t e;
-    if ((e = upload(s->bufs, &s->d_mgeo, mg, st)) || (e = upload(s->bufs, &s->d_mlog, ml, st)) ||
-        (e = upload(s->bufs, &s->d_tabf, tf, st)) || (e = upload(s->bufs, &s->d_Wf, mt.W, st)) ||
-        (e = upload(s->bufs, &s->d_Af, mt.A, st)) || (e = upload(s->bufs, &s->d_Bf, mt.B, st)) ||
-        (e = upload(s->bufs, &s->d_Cf, mt.C, st)))
-        return e;
-    const size_t ne = size_t(a.nb) * kTP;
-    if ((e = cudaMalloc(reinterpret_cast<void**>(&s->d_Mf), sizeof(float2) * ne)) != cudaSuccess) return e;
-    s->bufs.push_back(s->d_Mf);
-    if ((e = cudaMalloc(reinterpret_cast<void**>(&s->d_Lf), sizeof(float2) * ne)) != cudaSuccess) return e;
-    s->bufs.push_back(s->d_Lf);
-    if ((e = cudaMalloc(reinterpret_cast<void**>(&s->d_L0), sizeof(double) * a.nb)) != cudaSuccess) return e;
-    s->bufs.push_back(s->d_L0);
-    return cudaSuccess;
+    try {
+        std::vector<C> op(nop * 2 * kTP);
+        std::vector<typename OpLog<T>::type> lg(nop);
+        for (size_t i = 0; i < nop; ++i) {
+            const double tx = a.op[3 * i], ty = a.op[3 * i + 1], rho = a.op[3 * i + 2], r2 = tx * tx + ty * ty;
+            put_log(lg[i], 0.5 * std::log(r2));
+            const double2 ti{tx / r2, -ty / r2}, x{-rho * ti.x, -rho * ti.y};  // 1 / tau, -rho / tau
+            double2 px{-1.0, 0.0}, pt{1.0, 0.0};                              // -(-rho / tau)^k, tau^-l
+            for (int k = 0; k < kTP; ++k) {
+                C& u = op[(2 * i) * kTP + k];
+                C& v = op[(2 * i + 1) * kTP + k];
+                u.x = T(px.x), u.y = T(px.y), v.x = T(pt.x), v.y = T(pt.y);
+                px = zmul(px, x);
+                pt = zmul(pt, ti);
+            }
+        }
+        std::vector<typename NearAcc<T>::Kv> te(size_t(a.R + 1) * (a.R + 2)), to(size_t(a.Wo) * a.Wo);
+        for (int y = 0; y <= a.R; ++y)
+            for (int x = 0; x <= a.R; ++x)
+                put_kernel(te[size_t(y) * (a.R + 2) + x], x + y == 0 ? kC0A : 0.5 * std::log(double(x * x + y * y)));
+        for (int y = 0; y < a.Wo; ++y)
+            for (int x = 0; x <= y; ++x) {
+                const double v = 0.5 * std::log(double((2 * x + 1) * (2 * x + 1) + (2 * y + 1) * (2 * y + 1)));
+                put_kernel(to[size_t(y) * a.Wo + x], v);
+                put_kernel(to[size_t(x) * a.Wo + y], v);
+            }
+        const size_t ne = size_t(a.nb) * kTP;
+        if ((e = upload(s->bufs, &d.op, op, st)) || (e = upload(s->bufs, &d.oplog, lg, st)) ||
+            (e = upload(s->bufs, &d.te, te, st)) || (e = upload(s->bufs, &d.to, to, st)) ||
+            (e = dev_alloc(s->bufs, &d.ct, 1)) || (e = dev_alloc(s->bufs, &d.M, ne)) ||
+            (e = dev_alloc(s->bufs, &d.L, ne)) ||
+            (e = cudaMemcpyAsync(d.ct, hc, sizeof(AConst<T>), cudaMemcpyHostToDevice, st))) {
+            delete hc;
+            return e;
+        }
+        e = cudaStreamSynchronize(st);  // uploads done before the host arrays go
+    } catch (const std::bad_alloc&) {
+        e = cudaErrorMemoryAllocation;
+    }
+    delete hc;
+    d.ready = e == cudaSuccess;
+    return e;
 }
 
 cudaError_t setup_state(AdaptiveState* s, cudaStream_t st) {
@@ -498,209 +1005,20 @@ cudaError_t setup_state(AdaptiveState* s, cudaStream_t st) {
     cudaError_t e;
     if ((e = upload(s->bufs, &s->d_leafbox, a.leafbox, st)) || (e = upload(s->bufs, &s->d_fchild, a.fchild, st)) ||
         (e = upload(s->bufs, &s->d_parent, a.parent, st)) || (e = upload(s->bufs, &s->d_mptr, a.m2l_ptr, st)) ||
-        (e = upload(s->bufs, &s->d_msrc, a.m2l_src, st)) || (e = upload(s->bufs, &s->d_pptr, a.p2p_ptr, st)) ||
-        (e = upload(s->bufs, &s->d_psrc, a.p2p_src, st)) || (e = upload(s->bufs, &s->d_geo, a.geo, st)) ||
-        (e = upload(s->bufs, &s->d_tab, a.tab, st)) || (e = upload(s->bufs, &s->d_boxleaf, a.boxleaf, st)))
+        (e = upload(s->bufs, &s->d_mpair, a.m2l, st)) || (e = upload(s->bufs, &s->d_pptr, a.p2p_ptr, st)) ||
+        (e = upload(s->bufs, &s->d_ppair, a.p2p, st)) || (e = upload(s->bufs, &s->d_geo, a.geo, st)) ||
+        (e = upload(s->bufs, &s->d_anc, a.anc, st)) || (e = upload(s->bufs, &s->d_boxleaf, a.boxleaf, st)) ||
+        (e = dev_alloc(s->bufs, &s->d_err, 1)) || (e = dev_alloc(s->bufs, &s->d_S, a.nb)) ||
+        (e = dev_alloc(s->bufs, &s->d_L0, a.nb)) || (e = dev_alloc(s->bufs, &s->d_Sf, a.nb)) ||
+        (e = dev_alloc(s->bufs, &s->d_cnt, a.nb)) || (e = dev_alloc(s->bufs, &s->d_qexp, a.nleaf)) ||
+        (e = dev_alloc(s->bufs, &s->d_qfix, size_t(a.nleaf) * 64)))
         return e;
-    if ((e = cudaMalloc(reinterpret_cast<void**>(&s->d_err), sizeof(int))) != cudaSuccess) return e;
-    s->bufs.push_back(s->d_err);
-    if ((e = cudaMalloc(reinterpret_cast<void**>(&s->d_S), sizeof(double) * a.nb)) != cudaSuccess) return e;
-    s->bufs.push_back(s->d_S);
-    return cudaSuccess;
+    return cudaMemsetAsync(s->d_cnt, 0, sizeof(unsigned) * a.nb, st);
 }
 
-// ------------------------------------------------------------------------------------
-// Mixed precision: the same steps with FP32 expansions (and FP32 q and output), the box
-// monopoles S and the constant terms L_0 in FP64 (they carry the log terms whose sum
-// cancels across the domain), the shifts and the leaf P2M from the FP64-built tables, the
-// translations' geometry per pair from the host, the near field in FP32 with compensated
-// sums.  One warp (32 threads) per box for the expansion steps, thread k forming coefficient
-// k; 64 threads per leaf, one per cell, for the evaluation.
-// ------------------------------------------------------------------------------------
-__device__ __forceinline__ float2 cmulf(float2 a, float2 b) { return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
-__device__ __forceinline__ float2 cfmaf(float2 a, float2 b, float2 c) {  // a b + c
-    return make_float2(fmaf(a.x, b.x, fmaf(-a.y, b.y, c.x)), fmaf(a.x, b.y, fmaf(a.y, b.x, c.y)));
-}
-__device__ __forceinline__ int child_quadrant(const AGeo& g) { return (g.ix & 1) + 2 * (g.iy & 1); }
-
-// P2M: S (FP64 of the FP32 warp sum) and M_k = sum_c q_c w_c^k / k from the table.
-__global__ void k_ap2m_f(int nleaf, const int* __restrict__ leafbox, const float* __restrict__ q, int p,
-                         const float2* __restrict__ W, double* __restrict__ S, float2* __restrict__ M) {
-    const int i = blockIdx.x, k = threadIdx.x;
-    const float* qq = q + int64_t(i) * 64;
-    const int b = leafbox[i];
-    float s = qq[k] + qq[k + 32];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (k == 0) {
-        S[b] = double(s);
-        M[int64_t(b) * kTP] = make_float2(0.f, 0.f);
-    } else if (k <= p) {
-        float2 acc = make_float2(0.f, 0.f);
-        for (int c = 0; c < 64; ++c) {
-            const float2 w = W[c * kTP + k];
-            acc.x = fmaf(qq[c], w.x, acc.x);
-            acc.y = fmaf(qq[c], w.y, acc.y);
-        }
-        M[int64_t(b) * kTP + k] = acc;
-    }
-}
-
-// M2M for the internal boxes in [b0, b1): M_k = sum_children [S u^k / k + sum_{l<=k} A[q][l][k] M_l].
-__global__ void k_am2m_f(int b0, int b1, const int* __restrict__ first_child, const AGeo* __restrict__ geo, int p,
-                         const float2* __restrict__ A, const float2* __restrict__ B, double* __restrict__ S,
-                         float2* __restrict__ M) {
-    const int b = b0 + blockIdx.x, k = threadIdx.x;
-    const int fc = first_child[b];
-    if (fc < 0 || k > p) return;  // a leaf: its expansion came from P2M
-    float2 acc = make_float2(0.f, 0.f);
-    double ssum = 0.0;
-    for (int ch = fc; ch < fc + 4; ++ch) {
-        const double Sc = S[ch];
-        ssum += Sc;
-        if (k == 0) continue;
-        const int q = child_quadrant(geo[ch]);
-        const float2 bk = B[q * kTP + k];
-        acc.x = fmaf(float(Sc), bk.x, acc.x);
-        acc.y = fmaf(float(Sc), bk.y, acc.y);
-        const float2* Mc = M + int64_t(ch) * kTP;
-        const float2* Aq = A + size_t(q) * kTP * kTP;
-        for (int l = 1; l <= k; ++l) acc = cfmaf(Aq[l * kTP + k], Mc[l], acc);
-    }
-    if (k == 0) {
-        S[b] = ssum;
-        M[int64_t(b) * kTP] = make_float2(0.f, 0.f);
-    } else {
-        M[int64_t(b) * kTP + k] = acc;
-    }
-}
-
-// M2L: one warp per target box.  Per pair (tau, rho from the host, in target-side units):
-// thread k forms x_k = -M_k (-1)^k (rho / tau)^k into shared memory; thread l >= 1 adds
-// tau^-l (-S / l + sum_k x_k C(l+k-1, k-1)); thread 0 adds S (log|tau| + log s) + Re sum_k x_k
-// to the FP64 constant.
-__global__ void k_am2l_f(int nb, const int* __restrict__ ptr, const int* __restrict__ src,
-                         const float4* __restrict__ mgeo, const double* __restrict__ mlog, int p,
-                         const double* __restrict__ S, const float2* __restrict__ M, float2* __restrict__ L,
-                         double* __restrict__ L0) {
-    __shared__ float2 xs[32];
-    const int a = blockIdx.x, t = threadIdx.x;
-    float2 acc = make_float2(0.f, 0.f);
-    double acc0 = 0.0;
-    for (int e = ptr[a]; e < ptr[a + 1]; ++e) {
-        const int b = src[e];
-        const float4 g = mgeo[e];
-        const float d = g.x * g.x + g.y * g.y;
-        const float2 ti = make_float2(g.x / d, -g.y / d);  // 1 / tau
-        const double Sb = S[b];
-        float2 x = make_float2(0.f, 0.f);
-        if (t >= 1 && t <= p) {
-            const float2 rt = make_float2(g.z * ti.x, g.z * ti.y);  // rho / tau
-            float2 pw = rt;
-            for (int j = 1; j < t; ++j) pw = cmulf(pw, rt);
-            x = cmulf(M[int64_t(b) * kTP + t], pw);
-            if (!(t & 1)) x = make_float2(-x.x, -x.y);  // -M_k (-1)^k: the sign flips for even k
-        }
-        xs[t] = x;
-        __syncwarp();
-        if (t == 0) {
-            float r = 0.f;
-            for (int k = 1; k <= p; ++k) r += xs[k].x;
-            acc0 += Sb * mlog[e] + double(r);
-        } else if (t <= p) {
-            float2 sum = make_float2(0.f, 0.f);
-            float binom = 1.f;  // C(l+k-1, k-1) at k = 1
-            for (int k = 1; k <= p; ++k) {
-                sum.x = fmaf(binom, xs[k].x, sum.x);
-                sum.y = fmaf(binom, xs[k].y, sum.y);
-                binom = binom * float(t + k) / float(k);
-            }
-            sum.x -= float(Sb) / float(t);
-            float2 tl = ti;  // tau^-l
-            for (int j = 1; j < t; ++j) tl = cmulf(tl, ti);
-            acc = cfmaf(tl, sum, acc);
-        }
-        __syncwarp();
-    }
-    if (t == 0) L0[a] = acc0;
-    else if (t <= p) L[int64_t(a) * kTP + t] = acc;
-}
-
-// L2L for the boxes in [b0, b1) (parents final): L_l += sum_{k>=l} C[q][k][l] L_k(parent), and the
-// FP64 constant L_0 += L_0(parent) + Re sum_{k>=1} C[q][k][0] L_k(parent).
-__global__ void k_al2l_f(int b0, int b1, const int* __restrict__ parent, const AGeo* __restrict__ geo, int p,
-                         const float2* __restrict__ C, float2* __restrict__ L, double* __restrict__ L0) {
-    const int b = b0 + blockIdx.x, l = threadIdx.x;
-    const int pa = parent[b];
-    if (pa < 0 || l > p) return;
-    const int q = child_quadrant(geo[b]);
-    const float2* Lp = L + int64_t(pa) * kTP;
-    const float2* Cq = C + size_t(q) * kTP * kTP;
-    float2 acc = make_float2(0.f, 0.f);
-    for (int k = (l == 0 ? 1 : l); k <= p; ++k) acc = cfmaf(Cq[k * kTP + l], Lp[k], acc);
-    if (l == 0) {
-        L0[b] += L0[pa] + double(acc.x);
-    } else {
-        float2* Lb = L + int64_t(b) * kTP + l;
-        *Lb = make_float2(Lb->x + acc.x, Lb->y + acc.y);
-    }
-}
-
-// Leaves: 64 threads per leaf, one per cell: Re sum_{l>=1} L_l w^l (FP32 Horner) plus the FP64
-// constant, and the near field in FP32 with a compensated sum: same-level source leaves from
-// the FP32 table of log|D| (their log h part, S log h, in FP64), other levels directly.
-__global__ void k_aleaf_f(int nleaf, const int* __restrict__ leafbox, const int* __restrict__ ptr,
-                          const int* __restrict__ src, const AGeo* __restrict__ geo, int p,
-                          const float2* __restrict__ L, const double* __restrict__ L0, const float* __restrict__ tab,
-                          int R, const double* __restrict__ S, const float* __restrict__ q, float* __restrict__ p_out) {
-    const int i = blockIdx.x, c = threadIdx.x;
-    const int b = leafbox[i];
-    const AGeo g = geo[b];
-    const float wx = ((c & 7) + 0.5f) * 0.125f - 0.5f, wy = ((c >> 3) + 0.5f) * 0.125f - 0.5f;
-    const float2* Lb = L + int64_t(b) * kTP;
-    float2 h = Lb[p];
-    for (int l = p - 1; l >= 1; --l) h = cfmaf(h, make_float2(wx, wy), Lb[l]);
-    const float ser = h.x * wx - h.y * wy;
-    const double logh = log(g.s / 8.0);
-    const int W = 2 * R + 1;
-    float sum = 0.f, comp = 0.f;  // Kahan
-    double slog = 0.0;            // sum of S log h over the same-level source leaves
-    for (int e = ptr[i]; e < ptr[i + 1]; ++e) {
-        const int j = src[e];
-        const int bj = leafbox[j];
-        const AGeo gs = geo[bj];
-        const float* qs = q + int64_t(j) * 64;
-        float t = 0.f;
-        if (gs.level == g.level) {  // offsets (source cell - target cell) in cells, |.| <= R
-            const int ox = 8 * (gs.ix - g.ix) - (c & 7) + R, oy = 8 * (gs.iy - g.iy) - (c >> 3) + R;
-            for (int cs = 0; cs < 64; ++cs) t = fmaf(qs[cs], tab[(oy + (cs >> 3)) * W + ox + (cs & 7)], t);
-            slog += S[bj];
-        } else {
-            // source cell centres relative to the target cell, in units of the target's cell side
-            const double hc = g.s / 8.0;
-            const float ox = float((gs.cx - 0.5 * gs.s - (g.cx + g.s * double(wx))) / hc);
-            const float oy = float((gs.cy - 0.5 * gs.s - (g.cy + g.s * double(wy))) / hc);
-            const float step = float(gs.s / 8.0 / hc);   // source cell side / target cell side
-            const float rho = step * 0.34604881609982794f;  // rho_h of the source cell: exp(pi/4 - 3/2 - ln2/2) h
-            const float lhc = float(log(hc));
-            for (int cs = 0; cs < 64; ++cs) {
-                const float dx = ox + ((cs & 7) + 0.5f) * step, dy = oy + ((cs >> 3) + 0.5f) * step;
-                const float r = fmaxf(sqrtf(dx * dx + dy * dy), rho);
-                t = fmaf(qs[cs], logf(r) + lhc, t);
-            }
-        }
-        const float y = t - comp;
-        const float tt = sum + y;
-        comp = (tt - sum) - y;
-        sum = tt;
-    }
-    p_out[int64_t(i) * 64 + c] = float((L0[b] + slog * logh + double(ser) + double(sum)) * kInv2PiA);
-}
-
-}  // namespace
-
-extern "C" int pp_atree_solve(pp_atree tree, int order, const double* q, double* p_out, void* stream) {
-    if (!tree || !q || !p_out || order < 2 || order > kMaxOrderA) return PP_ERR_ARG;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
+// The tree's state and one precision's side of it, made on first use.
+template <typename T>
+int ensure_side(pp_atree tree, AdaptiveSide<T> AdaptiveState::* side, cudaStream_t st, AdaptiveState** out) {
     AdaptiveState* s = static_cast<AdaptiveState*>(pp::atree_state(tree));
     if (!s) {
         s = new (std::nothrow) AdaptiveState();
@@ -715,86 +1033,52 @@ extern "C" int pp_atree_solve(pp_atree tree, int order, const double* q, double*
         }
         pp::atree_set_state(tree, s, release_state);
     }
-    const AdaptivePrep& a = s->a;
-    const int nb = a.nb, nleaf = a.nleaf, L = a.L, p = order;
-    if (p > s->p_cap) {  // expansions for a higher order than before
-        cudaStreamSynchronize(st);
-        cudaFree(s->d_M);
-        cudaFree(s->d_L);
-        s->d_M = s->d_L = nullptr;
-        s->p_cap = 0;
-        cudaError_t e;
-        if ((e = cudaMalloc(reinterpret_cast<void**>(&s->d_M), sizeof(double2) * size_t(nb) * (p + 1))) ||
-            (e = cudaMalloc(reinterpret_cast<void**>(&s->d_L), sizeof(double2) * size_t(nb) * (p + 1)))) {
+    if (!(s->*side).ready) {
+        const cudaError_t e = setup_side<T>(s, s->*side, st);
+        if (e != cudaSuccess) {
             cudaGetLastError();
             return e == cudaErrorMemoryAllocation ? PP_ERR_OOM : PP_ERR_CUDA;
         }
-        s->p_cap = p;
     }
-    if (cudaMemsetAsync(s->d_L, 0, sizeof(double2) * size_t(nb) * (p + 1), st) != cudaSuccess) return PP_ERR_CUDA;
-    k_ap2m<<<nleaf, 32, 0, st>>>(nleaf, s->d_leafbox, q, p, s->d_S, s->d_M);
-    for (int l = L - 1; l >= 0; --l) {  // upward, deepest internal level first
-        const int b0 = a.lev_start[l], b1 = a.lev_start[l + 1];
-        if (b1 > b0) k_am2m<<<b1 - b0, 32, 0, st>>>(b0, b1, s->d_fchild, s->d_geo, p, s->d_S, s->d_M);
-    }
-    k_am2l<<<nb, 32, 0, st>>>(nb, s->d_mptr, s->d_msrc, s->d_geo, p, s->d_S, s->d_M, s->d_L);
-    for (int l = 1; l <= L; ++l) {  // downward, parents before children
-        const int b0 = a.lev_start[l], b1 = a.lev_start[l + 1];
-        if (b1 > b0) k_al2l<<<b1 - b0, 32, 0, st>>>(b0, b1, s->d_parent, s->d_geo, p, s->d_L);
-    }
-    k_aleaf<<<nleaf, 64, 0, st>>>(nleaf, s->d_leafbox, s->d_pptr, s->d_psrc, s->d_geo, p, s->d_L, s->d_tab, a.R,
-                                  s->d_S, q, p_out);
-    if (cudaGetLastError() != cudaSuccess) return PP_ERR_CUDA;
-    s->last_p = p;
+    *out = s;
     return PP_OK;
+}
+
+template <typename T>
+int solve_adaptive(AdaptiveState* s, const AdaptiveSide<T>& d, int p, const T* q, T* p_out, cudaStream_t st) {
+    const AdaptivePrep& a = s->a;
+    typename NearSrc<T>::type* qs = reinterpret_cast<typename NearSrc<T>::type*>(s->d_qfix);
+    k_aup<T><<<(a.nleaf + 3) / 4, 128, 0, st>>>(a.nleaf, s->d_leafbox, s->d_parent, s->d_fchild, q, p, d.ct, s->d_S,
+                                               s->d_Sf, d.M, s->d_cnt, qs, s->d_qexp);
+    k_am2l<T><<<a.nb, 128, 0, st>>>(s->d_mptr, s->d_mpair, s->d_geo, d.oplog, d.op, p, d.ct, s->d_S, s->d_Sf, d.M,
+                                    d.L, s->d_L0);
+    const size_t smem = sizeof(typename NearAcc<T>::Kv) * size_t(a.R + 1) * (a.R + 2);
+    k_aleaf<T><<<a.nleaf, kLeafThreads, smem, st>>>(s->d_leafbox, s->d_anc, a.L + 1, s->d_pptr, s->d_ppair, s->d_geo,
+                                                    p, d.ct, d.L, s->d_L0, d.te, a.R, d.to, a.Wo, s->d_S, q,
+                                                    qs, s->d_qexp, p_out);
+    return cudaGetLastError() == cudaSuccess ? PP_OK : PP_ERR_CUDA;
+}
+
+}  // namespace
+
+extern "C" int pp_atree_solve(pp_atree tree, int order, const double* q, double* p_out, void* stream) {
+    if (!tree || !q || !p_out || order < 2 || order > kMaxOrderA) return PP_ERR_ARG;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    AdaptiveState* s = nullptr;
+    int r = ensure_side<double>(tree, &AdaptiveState::f64, st, &s);
+    if (r == PP_OK) r = solve_adaptive<double>(s, s->f64, order, q, p_out, st);
+    if (r == PP_OK) s->last_p = order;
+    return r;
 }
 
 extern "C" int pp_atree_solve_mixed(pp_atree tree, int order, const float* q, float* p_out, void* stream) {
     if (!tree || !q || !p_out || order < 2 || order > kMaxOrderA) return PP_ERR_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    AdaptiveState* s = static_cast<AdaptiveState*>(pp::atree_state(tree));
-    if (!s) {
-        s = new (std::nothrow) AdaptiveState();
-        if (!s) return PP_ERR_OOM;
-        const int pst = prepare_adaptive(tree, s->a);
-        cudaError_t e = pst == PP_OK ? setup_state(s, st) : cudaSuccess;
-        if (pst == PP_OK && e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (pst != PP_OK || e != cudaSuccess) {
-            release_state(s);
-            cudaGetLastError();
-            return pst != PP_OK ? pst : e == cudaErrorMemoryAllocation ? PP_ERR_OOM : PP_ERR_CUDA;
-        }
-        pp::atree_set_state(tree, s, release_state);
-    }
-    if (!s->mixed_ready) {
-        cudaError_t e = setup_mixed(s, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // uploads done before the host arrays go
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            return e == cudaErrorMemoryAllocation ? PP_ERR_OOM : PP_ERR_CUDA;
-        }
-        s->mixed_ready = true;
-    }
-    const AdaptivePrep& a = s->a;
-    const int nb = a.nb, nleaf = a.nleaf, L = a.L, p = order;
-    if (cudaMemsetAsync(s->d_Lf, 0, sizeof(float2) * size_t(nb) * kTP, st) != cudaSuccess) return PP_ERR_CUDA;
-    k_ap2m_f<<<nleaf, 32, 0, st>>>(nleaf, s->d_leafbox, q, p, s->d_Wf, s->d_S, s->d_Mf);
-    for (int l = L - 1; l >= 0; --l) {  // upward, deepest internal level first
-        const int b0 = a.lev_start[l], b1 = a.lev_start[l + 1];
-        if (b1 > b0)
-            k_am2m_f<<<b1 - b0, 32, 0, st>>>(b0, b1, s->d_fchild, s->d_geo, p, s->d_Af, s->d_Bf, s->d_S, s->d_Mf);
-    }
-    k_am2l_f<<<nb, 32, 0, st>>>(nb, s->d_mptr, s->d_msrc, s->d_mgeo, s->d_mlog, p, s->d_S, s->d_Mf, s->d_Lf,
-                                s->d_L0);
-    for (int l = 1; l <= L; ++l) {  // downward, parents before children
-        const int b0 = a.lev_start[l], b1 = a.lev_start[l + 1];
-        if (b1 > b0) k_al2l_f<<<b1 - b0, 32, 0, st>>>(b0, b1, s->d_parent, s->d_geo, p, s->d_Cf, s->d_Lf, s->d_L0);
-    }
-    k_aleaf_f<<<nleaf, 64, 0, st>>>(nleaf, s->d_leafbox, s->d_pptr, s->d_psrc, s->d_geo, p, s->d_Lf, s->d_L0,
-                                    s->d_tabf, a.R, s->d_S, q, p_out);
-    if (cudaGetLastError() != cudaSuccess) return PP_ERR_CUDA;
-    s->last_p = 0;  // the FP64 multipoles no longer match S: the surface tree-code needs an FP64 solve
-    return PP_OK;
+    AdaptiveState* s = nullptr;
+    int r = ensure_side<float>(tree, &AdaptiveState::mixed, st, &s);
+    if (r == PP_OK) r = solve_adaptive<float>(s, s->mixed, order, q, p_out, st);
+    if (r == PP_OK) s->last_p = 0;  // S is the mixed solve's now: the surface tree-code needs an FP64 solve
+    return r;
 }
 
 extern "C" int pp_atree_surface_pressure(pp_atree tree, const double* q, int npts, const double* points, double theta,
@@ -805,8 +1089,8 @@ extern "C" int pp_atree_surface_pressure(pp_atree tree, const double* q, int npt
     if (!s || s->last_p < 1) return PP_ERR_STATE;  // the multipoles come from a solve
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (cudaMemsetAsync(s->d_err, 0, sizeof(int), st) != cudaSuccess) return PP_ERR_CUDA;
-    k_asurf<<<(npts + 127) / 128, 128, 0, st>>>(npts, points, s->d_geo, s->d_fchild, s->d_boxleaf, s->last_p, s->d_S,
-                                               s->d_M, q, theta, P_out, s->d_err);
+    k_asurf<<<(npts + 3) / 4, 128, 0, st>>>(npts, points, s->d_geo, s->d_fchild, s->d_boxleaf, s->last_p, s->d_S,
+                                               s->f64.M, q, theta, P_out, s->d_err);
     if (cudaGetLastError() != cudaSuccess) return PP_ERR_CUDA;
     int err = 0;
     if (cudaMemcpyAsync(&err, s->d_err, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
