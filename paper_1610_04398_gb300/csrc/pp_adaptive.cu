@@ -230,14 +230,31 @@ struct OpLog<float> {
 };
 
 // ------------------------------------------------------------------------------------
-// M2L: one CTA of four warps per target box, its entries dealt to the warps in turn.  The
-// diagonals (rho/tau)^k and tau^-l come from a table per distinct operator (a few hundred for
-// the tens of thousands of pairs; the powers were formed per pair and lane before).  Lane k
-// forms x_k in shared memory, lane l sums its row of the real product.  Mixed precision: the
-// constant term S log|tau| and the sums of S in double-float.
+// M2L: one CTA of 64-thread units (two; mixed four) per target box, its entries dealt to the units in turn, as
+// many entries at once as rows of p + 1 coefficients fit a unit (3 at p = 20, 4 at p = 12; one a
+// warp left a third to a half of the lanes idle: 198 against 130 us at p = 20 in FP64, whose
+// pipe bounds the kernel).  The diagonals (rho/tau)^k and tau^-l come from a table per distinct
+// operator (a few hundred for the tens of thousands of pairs).  Thread k of an entry forms x_k
+// in shared memory, thread l sums its row of the real product.  Mixed precision: the constant
+// term S log|tau| and the sums of S in double-float.
 // ------------------------------------------------------------------------------------
+__device__ __forceinline__ void unit_sync(int unit) {  // literal barrier numbers: five reserved, not sixteen
+    switch (unit) {
+        case 0: asm volatile("bar.sync 1, 64;" ::: "memory"); break;
+        case 1: asm volatile("bar.sync 2, 64;" ::: "memory"); break;
+        case 2: asm volatile("bar.sync 3, 64;" ::: "memory"); break;
+        default: asm volatile("bar.sync 4, 64;" ::: "memory"); break;
+    }
+}
+
+// Units a target: the mixed kernel is bound by the latency of an entry's loads, so four.
 template <typename T>
-__global__ void __launch_bounds__(128) k_am2l(const int* __restrict__ ptr, const int2* __restrict__ pair,
+struct M2LUnits {
+    static constexpr int value = sizeof(T) == 8 ? 2 : 4;
+};
+
+template <typename T>
+__global__ void __launch_bounds__(64 * M2LUnits<T>::value) k_am2l(const int* __restrict__ ptr, const int2* __restrict__ pair,
                                               const AGeo* __restrict__ geo, const typename OpLog<T>::type* __restrict__ oplog,
                                               const typename cplx_of<T>::type* __restrict__ op, int p,
                                               const AConst<T>* __restrict__ ct, const double* __restrict__ S,
@@ -245,68 +262,84 @@ __global__ void __launch_bounds__(128) k_am2l(const int* __restrict__ ptr, const
                                               const typename cplx_of<T>::type* __restrict__ M,
                                               typename cplx_of<T>::type* __restrict__ L, double* __restrict__ L0) {
     typedef typename cplx_of<T>::type C;
+    constexpr int kUnits = M2LUnits<T>::value, kThreads = 64 * kUnits;
     __shared__ T R[kTP][kTP];
-    __shared__ C xs[4][kTP];
-    __shared__ C red[4][kTP];
-    __shared__ double red0[4];
-    const int a = blockIdx.x, w = threadIdx.x >> 5, t = threadIdx.x & 31;
+    __shared__ C xs[kUnits][2][64];
+    __shared__ C red[kThreads];
+    __shared__ double red0[kThreads];
+    const int a = blockIdx.x, tid = threadIdx.x, unit = tid >> 6;
     const int e0 = ptr[a], e1 = ptr[a + 1];
     if (e0 == e1) {  // no sources (block-uniform)
-        if (w == 0 && t <= p) L[int64_t(a) * kTP + t] = cx<T>(T(0), T(0));
-        if (w == 0 && t == 0) L0[a] = 0.0;
+        if (tid <= p) L[int64_t(a) * kTP + tid] = cx<T>(T(0), T(0));
+        if (tid == 0) L0[a] = 0.0;
         return;
     }
-    for (int i = threadIdx.x; i < kTP * kTP; i += 128) (&R[0][0])[i] = (&ct->m2l[0][0])[i];
+    const int P1 = p + 1, slots = 64 / P1;              // entries a unit takes at once (2 at p = 30)
+    const int slot = (tid & 63) / P1, t = (tid & 63) - slot * P1;  // slot == slots: an idle thread
+    for (int i = tid; i < kTP * kTP; i += kThreads) (&R[0][0])[i] = (&ct->m2l[0][0])[i];
     __syncthreads();
     C acc = cx<T>(T(0), T(0));
     const double lns = -kLn2A * geo[a].level;  // log of the target's side
     const T cl = t == 0 ? T(0) : T(-1) / T(t);
     float ah = 0.f, al = 0.f, sh = 0.f, sl = 0.f;  // mixed: constant term, sum of S
-    for (int e = e0 + w; e < e1; e += 4) {
-        const int2 pr = pair[e];
-        const C* o = op + int64_t(pr.y) * (2 * kTP);
-        const C m = M[int64_t(pr.x) * kTP + t], tk = o[t], tl = o[kTP + t];
-        __syncwarp();  // the last entry's reads are done
-        xs[w][t] = cmulT<T>(m, tk);
-        __syncwarp();
-        C y = cx<T>(T(0), T(0));
-        if constexpr (sizeof(T) == 8) {
-            y.x = S[pr.x] * (t == 0 ? oplog[pr.y] + lns : cl);
-        } else {
-            const float2 Sb = Sf[pr.x];
-            const float2 lt = oplog[pr.y];
-            y.x = Sb.x * cl;
-            df_fma(ah, al, Sb.x, Sb.y, lt.x, lt.y);
-            df_add(sh, sl, Sb.x, Sb.y);
+    int buf = 0;
+    int2 ahead = make_int2(0, 0);  // mixed: the pair of the next round, read a round early
+    if (sizeof(T) == 4 && slot < slots && e0 + unit * slots + slot < e1) ahead = pair[e0 + unit * slots + slot];
+    for (int base = e0 + unit * slots; base < e1; base += kUnits * slots, buf ^= 1) {  // uniform over the unit
+        const int e = base + slot;
+        const bool act = slot < slots && e < e1;
+        C tl = cx<T>(T(0), T(0));
+        const int2 pr = sizeof(T) == 4 ? ahead : act ? pair[e] : ahead;
+        if (sizeof(T) == 4 && slot < slots && e + kUnits * slots < e1) ahead = pair[e + kUnits * slots];
+        if (act) {
+            const C* o = op + int64_t(pr.y) * (2 * kTP);
+            tl = o[kTP + t];
+            xs[unit][buf][tid & 63] = cmulT<T>(M[int64_t(pr.x) * kTP + t], o[t]);
         }
+        unit_sync(unit);  // two buffers: one barrier an entry
+        if (act) {
+            const C* x = &xs[unit][buf][slot * P1];
+            C y = cx<T>(T(0), T(0));
+            if constexpr (sizeof(T) == 8) {
+                y.x = S[pr.x] * (t == 0 ? oplog[pr.y] + lns : cl);
+            } else {
+                const float2 Sb = Sf[pr.x], lt = oplog[pr.y];
+                y.x = Sb.x * cl;
+                df_fma(ah, al, Sb.x, Sb.y, lt.x, lt.y);
+                df_add(sh, sl, Sb.x, Sb.y);
+            }
 #pragma unroll 4
-        for (int k = 1; k <= p; ++k) {
-            const T r = R[k][t];
-            const C x = xs[w][k];
-            y.x = fma(r, x.x, y.x);
-            y.y = fma(r, x.y, y.y);
+            for (int k = 1; k <= p; ++k) {
+                const T r = R[k][t];
+                const C v = x[k];
+                y.x = fma(r, v.x, y.x);
+                y.y = fma(r, v.y, y.y);
+            }
+            if constexpr (sizeof(T) == 4) df_add(ah, al, y.x, 0.f);  // thread 0: Re sum x_k
+            acc.x = fma(tl.x, y.x, fma(-tl.y, y.y, acc.x));
+            acc.y = fma(tl.x, y.y, fma(tl.y, y.x, acc.y));
         }
-        if constexpr (sizeof(T) == 4) df_add(ah, al, y.x, 0.f);  // lane 0: Re sum x_k
-        acc.x = fma(tl.x, y.x, fma(-tl.y, y.y, acc.x));
-        acc.y = fma(tl.x, y.y, fma(tl.y, y.x, acc.y));
     }
-    red[w][t] = acc;
-    if (t == 0) red0[w] = sizeof(T) == 8 ? double(acc.x) : df_to(ah, al) + lns * df_to(sh, sl);
+    red[tid] = acc;
+    red0[tid] = sizeof(T) == 8 ? double(acc.x) : df_to(ah, al) + lns * df_to(sh, sl);
     __syncthreads();
-    if (w == 0 && t <= p) {
-        C s = red[0][t];
-#pragma unroll
-        for (int i = 1; i < 4; ++i) {
-            s.x += red[i][t].x;
-            s.y += red[i][t].y;
-        }
-        L[int64_t(a) * kTP + t] = s;
-        if (t == 0) L0[a] = red0[0] + red0[1] + red0[2] + red0[3];
+    if (tid <= p) {
+        C s = cx<T>(T(0), T(0));
+        double s0 = 0.0;
+        for (int u = 0; u < kUnits; ++u)
+            for (int i = 0; i < slots; ++i) {
+                const C v = red[u * 64 + i * P1 + tid];
+                s.x += v.x;
+                s.y += v.y;
+                if (tid == 0) s0 += red0[u * 64 + i * P1];
+            }
+        L[int64_t(a) * kTP + tid] = s;
+        if (tid == 0) L0[a] = s0;
     }
 }
 
 // ------------------------------------------------------------------------------------
-// Leaves: one CTA per leaf.  Eight warps sum the near field, a ninth shifts the locals down
+// Leaves: one CTA per leaf.  All its warps but one sum the near field, the last shifts the locals down
 // the leaf's path from the root (each leaf repeats its ancestors' shifts: no launch per level)
 // and forms the constant terms; then one thread per cell evaluates the local expansion.
 //
@@ -318,7 +351,7 @@ __global__ void __launch_bounds__(128) k_am2l(const int* __restrict__ ptr, const
 // `to` over (|2 m_x + 1|, |2 m_y + 1|); the source's clamp never acts between different cells.
 // log(unit) times the source leaf's S is added once per leaf (FP64).  Pairs beyond the table
 // (kDirect) and, in FP64, leaves with non-finite weights are summed cell by cell.
-// A thread owns one row of 8 target cells and one row of 8 source cells of every fourth pair: its 64
+// A thread owns one row of 8 target cells and one row of 8 source cells of its share of the pairs: its 64
 // cell pairs need 15 (same level) or 22 (kappa 1) kernel values, kept in registers.  Before, each
 // pair took its own table read, and pairs of different levels a square root and a logarithm.
 //
@@ -329,6 +362,12 @@ __global__ void __launch_bounds__(128) k_am2l(const int* __restrict__ ptr, const
 // accumulate exactly in 64 bits (32 source leaves a thread before they are added to the FP64
 // sum), ll (below 2^-56 of full scale a pair) is dropped.
 // ------------------------------------------------------------------------------------
+// s += a b, 32 x 32 + 64 bits in one instruction (the compiler's own choice for the C expression
+// took about six).
+__device__ __forceinline__ void mad_wide(long long& s, int a, int b) {
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(s) : "r"(a), "r"(b));
+}
+
 template <typename T>
 struct NearAcc;
 
@@ -391,9 +430,9 @@ struct NearAcc<double> {
         }
     }
     __device__ __forceinline__ void add(int j, int r, int2 k) {
-        hh[j] += (long long)qh[r] * k.x;
-        mid[j] += (long long)qh[r] * k.y;
-        mid[j] += (long long)ql[r] * k.x;
+        mad_wide(hh[j], qh[r], k.x);
+        mad_wide(mid[j], qh[r], k.y);
+        mad_wide(mid[j], ql[r], k.x);
     }
     __device__ void drain(int et) {
         const double f1 = __hiloint2double((1023 + et - 50) << 20, 0), f2 = f1 * 3.7252902984619140625e-09;  // 2^-28
@@ -409,10 +448,16 @@ struct NearAcc<double> {
     __device__ void finish(int et) { drain(et); }
 };
 
-constexpr int kLeafThreads = 288;  // eight near-field warps and the path's warp
+// Pairs of near-field warps per CTA, and the path's warp: FP64 needs 128 registers a thread, and
+// three CTAs of five warps fit an SM.
+template <typename T>
+struct LeafCta {
+    static constexpr int groups = sizeof(T) == 8 ? 2 : 4;
+    static constexpr int threads = 64 * groups + 32;
+};
 
 template <typename T>
-__global__ void __launch_bounds__(kLeafThreads)
+__global__ void __launch_bounds__(LeafCta<T>::threads, 3)
 k_aleaf(const int* __restrict__ leafbox, const int* __restrict__ anc, int nlev, const int* __restrict__ ptr,
         const APair* __restrict__ pairs, const AGeo* __restrict__ geo, int p, const AConst<T>* __restrict__ ct,
         const typename cplx_of<T>::type* __restrict__ L, const double* __restrict__ L0,
@@ -423,16 +468,17 @@ k_aleaf(const int* __restrict__ leafbox, const int* __restrict__ anc, int nlev, 
     typedef typename NearAcc<T>::Kv Kv;
     extern __shared__ __align__(16) unsigned char smem_leaf[];
     Kv* tab = reinterpret_cast<Kv*>(smem_leaf);  // (R + 1) rows of stride R + 2
-    __shared__ T near[4][64];
+    constexpr int kGroups = LeafCta<T>::groups;
+    __shared__ T near[kGroups][64];
     __shared__ C Ls[kTP];
     __shared__ double c0s;
     const int i = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int b = leafbox[i];
     const int e0 = ptr[i], e1 = ptr[i + 1];
     const int W = R + 2;
-    for (int m = tid; m < (R + 1) * W; m += kLeafThreads) tab[m] = te[m];
+    for (int m = tid; m < (R + 1) * W; m += LeafCta<T>::threads) tab[m] = te[m];
     __syncthreads();
-    if (warp < 8) {
+    if (warp < 2 * kGroups) {
         const int g = warp >> 1, sy = lane & 7, ty = (lane >> 3) + 4 * (warp & 1);
         int et = -900;
         if constexpr (sizeof(T) == 8) {  // the largest exponent of the target's sources
@@ -445,7 +491,7 @@ k_aleaf(const int* __restrict__ leafbox, const int* __restrict__ anc, int nlev, 
         NearAcc<T> A;
         A.init();
         int n = 0;
-        for (int e = e0 + g; e < e1; e += 4) {
+        for (int e = e0 + g; e < e1; e += kGroups) {
             const APair pr = pairs[e];
             int sh = 0;
             bool direct = pr.kind == kDirect;
@@ -590,7 +636,8 @@ k_aleaf(const int* __restrict__ leafbox, const int* __restrict__ anc, int nlev, 
             const C v = ct->V[l][tid], m = Ls[l];
             ser = fma(m.x, v.x, fma(-m.y, v.y, ser));
         }
-        const T nr = (near[0][tid] + near[1][tid]) + (near[2][tid] + near[3][tid]);
+        T nr = near[0][tid] + near[1][tid];
+        if constexpr (kGroups == 4) nr += near[2][tid] + near[3][tid];
         p_out[int64_t(i) * 64 + tid] = T((c0s + double(ser) + double(nr)) * kInv2PiA);
     }
 }
@@ -1050,10 +1097,10 @@ int solve_adaptive(AdaptiveState* s, const AdaptiveSide<T>& d, int p, const T* q
     typename NearSrc<T>::type* qs = reinterpret_cast<typename NearSrc<T>::type*>(s->d_qfix);
     k_aup<T><<<(a.nleaf + 3) / 4, 128, 0, st>>>(a.nleaf, s->d_leafbox, s->d_parent, s->d_fchild, q, p, d.ct, s->d_S,
                                                s->d_Sf, d.M, s->d_cnt, qs, s->d_qexp);
-    k_am2l<T><<<a.nb, 128, 0, st>>>(s->d_mptr, s->d_mpair, s->d_geo, d.oplog, d.op, p, d.ct, s->d_S, s->d_Sf, d.M,
+    k_am2l<T><<<a.nb, 64 * M2LUnits<T>::value, 0, st>>>(s->d_mptr, s->d_mpair, s->d_geo, d.oplog, d.op, p, d.ct, s->d_S, s->d_Sf, d.M,
                                     d.L, s->d_L0);
     const size_t smem = sizeof(typename NearAcc<T>::Kv) * size_t(a.R + 1) * (a.R + 2);
-    k_aleaf<T><<<a.nleaf, kLeafThreads, smem, st>>>(s->d_leafbox, s->d_anc, a.L + 1, s->d_pptr, s->d_ppair, s->d_geo,
+    k_aleaf<T><<<a.nleaf, LeafCta<T>::threads, smem, st>>>(s->d_leafbox, s->d_anc, a.L + 1, s->d_pptr, s->d_ppair, s->d_geo,
                                                     p, d.ct, d.L, s->d_L0, d.te, a.R, d.to, a.Wo, s->d_S, q,
                                                     qs, s->d_qexp, p_out);
     return cudaGetLastError() == cudaSuccess ? PP_OK : PP_ERR_CUDA;
