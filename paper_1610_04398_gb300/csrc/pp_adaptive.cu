@@ -30,6 +30,7 @@
 #include "../../include/pp.h"
 #include "pp_atree_state.h"
 #include "pp_common.h"
+#include "pp_fixed.cuh"
 #include "pp_log.cuh"
 
 namespace {
@@ -38,6 +39,7 @@ using pp::cplx_of;
 using pp::df_add;
 using pp::df_fma;
 using pp::df_to;
+using pp::mad_wide;
 
 constexpr int kMaxOrderA = 30;
 constexpr int kTP = 32;  // stride (coefficients) of the expansion arrays and of the tables
@@ -266,7 +268,7 @@ __global__ void __launch_bounds__(64 * M2LUnits<T>::value) k_am2l(const int* __r
     __shared__ T R[kTP][kTP];
     __shared__ C xs[kUnits][2][64];
     __shared__ C red[kThreads];
-    __shared__ double red0[kThreads];
+    __shared__ float4 red0[sizeof(T) == 4 ? kThreads : 1];  // mixed: constant term and sum of S, pairs
     const int a = blockIdx.x, tid = threadIdx.x, unit = tid >> 6;
     const int e0 = ptr[a], e1 = ptr[a + 1];
     if (e0 == e1) {  // no sources (block-uniform)
@@ -321,20 +323,24 @@ __global__ void __launch_bounds__(64 * M2LUnits<T>::value) k_am2l(const int* __r
         }
     }
     red[tid] = acc;
-    red0[tid] = sizeof(T) == 8 ? double(acc.x) : df_to(ah, al) + lns * df_to(sh, sl);
+    if constexpr (sizeof(T) == 4) red0[tid] = make_float4(ah, al, sh, sl);
     __syncthreads();
     if (tid <= p) {
         C s = cx<T>(T(0), T(0));
-        double s0 = 0.0;
+        float rh = 0.f, rl = 0.f, qh = 0.f, ql = 0.f;
         for (int u = 0; u < kUnits; ++u)
             for (int i = 0; i < slots; ++i) {
                 const C v = red[u * 64 + i * P1 + tid];
                 s.x += v.x;
                 s.y += v.y;
-                if (tid == 0) s0 += red0[u * 64 + i * P1];
+                if constexpr (sizeof(T) == 4) {
+                    const float4 r = red0[u * 64 + i * P1];
+                    df_add(rh, rl, r.x, r.y);
+                    df_add(qh, ql, r.z, r.w);
+                }
             }
         L[int64_t(a) * kTP + tid] = s;
-        if (tid == 0) L0[a] = s0;
+        if (tid == 0) L0[a] = sizeof(T) == 4 ? df_to(rh, rl) + lns * df_to(qh, ql) : double(s.x);
     }
 }
 
@@ -355,19 +361,11 @@ __global__ void __launch_bounds__(64 * M2LUnits<T>::value) k_am2l(const int* __r
 // cell pairs need 15 (same level) or 22 (kappa 1) kernel values, kept in registers.  Before, each
 // pair took its own table read, and pairs of different levels a square root and a logarithm.
 //
-// FP64 runs the cell pairs on the integer pipe: FP64 multiply-adds issue at 1.67 lanes a clock
-// and SM, 32 x 32 + 64 bit integer ones at 32 to 64.  Source weights are 55-bit integers v
-// (relative to the largest exponent et of the target's sources), kernel values 55-bit integers
-// (2^-52 units, |log| < 8), both split v = h 2^28 + l with l in [-2^27, 2^27); hh and hl + lh
-// accumulate exactly in 64 bits (32 source leaves a thread before they are added to the FP64
-// sum), ll (below 2^-56 of full scale a pair) is dropped.
+// FP64 runs the cell pairs in fixed point on the integer pipe (pp_fixed.cuh).  Source weights are
+// 55-bit integers (relative to the largest exponent et of the target's sources), kernel values
+// 56-bit integers (2^-52 units, |log| < 8); 32 source leaves a thread are summed before they are
+// added to the FP64 sum.
 // ------------------------------------------------------------------------------------
-// s += a b, 32 x 32 + 64 bits in one instruction (the compiler's own choice for the C expression
-// took about six).
-__device__ __forceinline__ void mad_wide(long long& s, int a, int b) {
-    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(s) : "r"(a), "r"(b));
-}
-
 template <typename T>
 struct NearAcc;
 
@@ -423,9 +421,9 @@ struct NearAcc<double> {
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
                 if (sh > 0) v[u] = sh > 60 ? 0 : (v[u] + (1ll << (sh - 1))) >> sh;
-                const int l = int(unsigned(v[u]) << 4) >> 4;
-                ql[2 * i + u] = l;
-                qh[2 * i + u] = int((v[u] - l) >> 28);
+                const int2 h = pp::split28(v[u]);
+                qh[2 * i + u] = h.x;
+                ql[2 * i + u] = h.y;
             }
         }
     }
@@ -990,9 +988,7 @@ void put_log(double& d, double v) { d = v; }
 void put_log(float2& d, double v) { d = make_float2(float(v), float(v - double(float(v)))); }
 void put_kernel(float& d, double v) { d = float(v); }
 void put_kernel(int2& d, double v) {  // 2^-52 units as h 2^28 + l, |l| <= 2^27
-    const int64_t t = std::llrint(std::ldexp(v, 52));
-    const int l = int(uint32_t(t) << 4) >> 4;
-    d = make_int2(int((t - l) >> 28), l);
+    d = pp::split28(std::llrint(std::ldexp(v, 52)));
 }
 
 template <typename T>

@@ -162,6 +162,9 @@ struct pp_plan_s {
     int m2l_margin = -1;
     float m2l_inv_sb = 1.f;
     int sms = 0;
+    // FP64 plans of the fixed-point path (pp_fp64.cuh)
+    bool use_f64 = false;
+    pp::F64Scales f64sc = {};
     std::vector<double> op_geo;            // [op][tau_x, tau_y, side ratio]
     std::vector<pp::M2LEntry> il_host;     // the interaction lists as uploaded
     void* ktc = nullptr;
@@ -388,6 +391,13 @@ int upload_tables(pp_plan p) {
     }
     int maxl = 0;
     for (int c = 0; c < 4; ++c) maxl = std::max(maxl, int(lists[c].size()));
+    if constexpr (sizeof(T) == 8) {
+        if (p->use_f64) {  // the operators and the near-field table as fixed point
+            pp::f64_pack_m2l(tabT.data() + p->off_B, p->n_ops, P1, maxl, &p->f64sc);
+            p->f64sc.ln_root = std::log(double(p->n) * p->h);
+            pp::f64_pack_near(Kr.data(), p->Rk);
+        }
+    }
     p->il_stride = std::max(maxl, 1);
     std::vector<pp::M2LEntry> ilh(size_t(4) * p->il_stride, pp::M2LEntry{0, 0, 0, 0});
     for (int c = 0; c < 4; ++c) {
@@ -522,8 +532,10 @@ int alloc_tree(pp_plan p) {
         return PP_ERR_OOM;
     if (cudaMemset(p->moments_buf, 0, sizeof(double) * (pp::moments_partial_doubles() + 3)) != cudaSuccess)
         return PP_ERR_CUDA;
-    if (dalloc(p, (void**)&p->up_counter, sizeof(unsigned) * 4) != cudaSuccess) return PP_ERR_OOM;
-    if (cudaMemset(p->up_counter, 0, sizeof(unsigned) * 4) != cudaSuccess) return PP_ERR_CUDA;
+    p->use_f64 = sizeof(T) == 8 && pp::f64_ok(p->P1, p->Lleaf);
+    const size_t nc = p->use_f64 ? pp::f64_counter_words(p->Lleaf) : 4;
+    if (dalloc(p, (void**)&p->up_counter, sizeof(unsigned) * nc) != cudaSuccess) return PP_ERR_OOM;
+    if (cudaMemset(p->up_counter, 0, sizeof(unsigned) * nc) != cudaSuccess) return PP_ERR_CUDA;
     if (dalloc(p, (void**)&p->err, sizeof(int) * 4) != cudaSuccess) return PP_ERR_OOM;
     if (cudaMemset(p->err, 0, sizeof(int) * 4) != cudaSuccess) return PP_ERR_CUDA;
     if (sizeof(T) == 4 && dalloc(p, (void**)&p->Sf, sizeof(float2) * size_t(nbox)) != cudaSuccess)
@@ -547,6 +559,7 @@ int prepare_device(int device, int precision) {
     const int k = precision == PP_FP64 ? 0 : 1;
     if (done[device][k]) return PP_OK;
     cudaError_t e = precision == PP_FP64 ? pp::prepare_kernels<double>() : pp::prepare_kernels<float>();
+    if (e == cudaSuccess && precision == PP_FP64) e = pp::prepare_f64();
     if (e == cudaSuccess && precision == PP_MIXED) e = pp::prepare_near_tc();
     if (e == cudaSuccess && precision == PP_MIXED) e = pp::prepare_m2l_tc();
     if (e != cudaSuccess) {
@@ -576,7 +589,7 @@ int64_t plan_bytes(int n, int order, double theta, int precision, int tile, int 
     b += al(8 * 8);                                                // forces
     b += al(8 * (int64_t(pp::penal_partial_doubles()) + 4));       // penalisation partials
     b += al(8 * (int64_t(pp::moments_partial_doubles()) + 3));     // body-moment partials
-    b += al(4 * 4);                                                // upward arrival counter
+    b += al(4 * (precision == PP_FP64 && pp::f64_ok(int(P1), Lleaf) ? int64_t(pp::f64_counter_words(Lleaf)) : 4));
     if (precision == PP_MIXED && Lleaf >= 5) {                     // downward side buffers
         const int64_t na = pp::level_offset(Lleaf - 3);
         b += al(csz * na * P1) + al(8 * na);
@@ -698,7 +711,13 @@ int run_rhs(pp_plan p, const void* u, const void* v, const void* chi, const void
     p->near_forked = nullptr;  // new source weights: any pending near field is stale
     stage_begin(p, ST_RHS);
     int nk = 0;
-    if (pp::launch_rhs_p2m<T>(t, (const T*)u, (const T*)v, (const T*)chi, (const T*)usx, (const T*)usy,
+    if (p->use_f64) {
+        nk = 2;
+        if (pp::launch_rhs64(reinterpret_cast<const pp::Tree<double>&>(t), (const double*)u, (const double*)v,
+                             (const double*)chi, (const double*)usx, (const double*)usy, p->rho, lam, (double*)f_out,
+                             p->stream) != cudaSuccess)
+            return cuda_fail(p);
+    } else if (pp::launch_rhs_p2m<T>(t, (const T*)u, (const T*)v, (const T*)chi, (const T*)usx, (const T*)usy,
                               p->rho, lam, (T*)f_out, p->stream, &nk) != cudaSuccess)
         return cuda_fail(p);
     stage_end(p, ST_RHS);
@@ -713,9 +732,11 @@ int ensure_up(pp_plan p) {
     if (p->have_up) return PP_OK;
     pp::Tree<T> t = make_tree<T>(p);
     stage_begin(p, ST_UP);
-    if (pp::launch_upward<T>(t, p->stream) != cudaSuccess) return cuda_fail(p);
+    const cudaError_t eu = p->use_f64 ? pp::launch_up64(reinterpret_cast<const pp::Tree<double>&>(t), p->stream)
+                                      : pp::launch_upward<T>(t, p->stream);
+    if (eu != cudaSuccess) return cuda_fail(p);
     stage_end(p, ST_UP);
-    p->launches += pp::upward_launches<T>(t);
+    p->launches += p->use_f64 ? 1 : pp::upward_launches<T>(t);
     p->have_up = true;
     return PP_OK;
 }
@@ -732,7 +753,9 @@ int fork_near(pp_plan p, void* p_out) {
     // the tensor-core kernel stores 16-byte vectors: an output off that alignment takes the
     // FP32-core kernel
     const bool tc = p->use_tc && (reinterpret_cast<uintptr_t>(p_out) & 15) == 0;
-    const cudaError_t en = tc ? pp::launch_near_tc(p->tc_maps, static_cast<const float*>(p->q), p->ktc, p->near,
+    const cudaError_t en = p->use_f64
+                               ? pp::launch_near64(reinterpret_cast<const pp::Tree<double>&>(t), (double*)p_out, p->aux)
+                           : tc ? pp::launch_near_tc(p->tc_maps, static_cast<const float*>(p->q), p->ktc, p->near,
                                                    p->n_near, p->Dmax, p->n,
                                                           (float*)p_out, p->err + 1, p->aux)
                                      : pp::launch_near_only<T>(t, (T*)p_out, p->aux);
@@ -746,6 +769,26 @@ int fork_near(pp_plan p, void* p_out) {
 template <typename T>
 int run_solve(pp_plan p, void* p_out) {
     pp::Tree<T> t = make_tree<T>(p);
+    if (p->use_f64) {
+        // the near field on the integer pipe beside the expansion chain on the FP64 pipe
+        const pp::Tree<double>& td = reinterpret_cast<const pp::Tree<double>&>(t);
+        if (p_out && p->near_forked != p_out) {
+            const int sf = fork_near<T>(p, p_out);
+            if (sf != PP_OK) return sf;
+        }
+        p->near_forked = nullptr;
+        const int st = ensure_up<T>(p);
+        if (st != PP_OK) return st;
+        stage_begin(p, ST_DOWN);
+        if (pp::launch_m2l64(td, p->f64sc, p->stream) != cudaSuccess) return cuda_fail(p);
+        stage_end(p, ST_DOWN);
+        if (p_out && cudaStreamWaitEvent(p->stream, p->ev_join, 0) != cudaSuccess) return cuda_fail(p);
+        stage_begin(p, ST_LEAFM2L);
+        if (pp::launch_down64(td, (double*)p_out, p->stream) != cudaSuccess) return cuda_fail(p);
+        stage_end(p, ST_LEAFM2L);
+        p->launches += 1 + pp::f64_down_launches(td) + (p_out ? 1 : 0);
+        return PP_OK;
+    }
     if (p_out && pp::split_solve_ok<T>(t)) {
         if (p->near_forked != p_out) {
             const int sf = fork_near<T>(p, p_out);
@@ -1256,6 +1299,7 @@ int pp_step_graph_create(pp_plan p, const void* u, const void* v, const void* ch
     // the near field forks right after the source weights, ahead of the upward pass
     if (st == PP_OK && p_out && p->precision == PP_MIXED && pp::split_solve_ok<float>(make_tree<float>(p)))
         st = fork_near<float>(p, p_out);
+    if (st == PP_OK && p_out && p->use_f64) st = fork_near<double>(p, p_out);
     if (st == PP_OK) st = p->precision == PP_FP64 ? ensure_up<double>(p) : ensure_up<float>(p);
     if (st == PP_OK && npts > 0) {
         // the surface path needs only q and the multipoles: run it beside the solve

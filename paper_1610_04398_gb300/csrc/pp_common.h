@@ -180,6 +180,30 @@ cudaError_t launch_m2l_tc(const Tree<float>& t, const void* tables, int n_ops, i
                           unsigned* claim, int sms, int* err, cudaStream_t st);
 cudaError_t prepare_m2l_tc();
 
+// The FP64 path (orders up to 23, leaf level >= 2; pp_fp64.cuh): scales of its fixed-point
+// translation operators, the words of the plan's counter array (level exponents and arrival
+// counters), the packing of the operators and of the near-field table in place of their FP64
+// values, and the launches.  launch_near64 writes the near field (without its log h part, which
+// launch_down64 adds) to p_out; launch_down64 shifts the locals down and, with p_out, adds the
+// local expansions to it.
+struct F64Scales {
+    int wbits;       // fixed-point bits of the operators
+    int el[32];      // power-of-two scale of each row
+    double ln_root;  // log of the root box side
+};
+bool f64_ok(int P1, int Lleaf);
+size_t f64_counter_words(int Lleaf);
+void f64_pack_m2l(double2* B, int n_ops, int P1, int max_entries, F64Scales* sc);
+void f64_pack_near(double* K, int R);
+cudaError_t launch_rhs64(const Tree<double>& t, const double* u, const double* v, const double* chi, const double* usx,
+                         const double* usy, double rho, double lam, double* f_out, cudaStream_t st);
+cudaError_t launch_up64(const Tree<double>& t, cudaStream_t st);
+cudaError_t launch_near64(const Tree<double>& t, double* p_out, cudaStream_t st);
+cudaError_t launch_m2l64(const Tree<double>& t, const F64Scales& sc, cudaStream_t st);
+cudaError_t launch_down64(const Tree<double>& t, double* p_out, cudaStream_t st);
+int f64_down_launches(const Tree<double>& t);
+cudaError_t prepare_f64();
+
 struct SurfaceArgs {
     int npts;
     const double* pts;
@@ -257,6 +281,8 @@ cudaError_t launch_surface(const Tree<T>& t, const T* u, const T* v, const Surfa
 template <typename T>
 cudaError_t launch_export_expansion(const Tree<T>& t, int kind, int level, double* dst,
                                     cudaStream_t st);
+
+cudaError_t launch_treecode64(const Tree<double>& t, const SurfaceArgs& a, cudaStream_t st);
 
 constexpr int kSurfaceBlock = 64;
 // Surface scratch of a plan: a new plan holds it for kInitialSurfaceCap points and grows it

@@ -783,13 +783,16 @@ cudaError_t launch_rhs_p2m(const Tree<T>& t, const T* u, const T* v, const T* ch
     if (e != cudaSuccess) return e;
     const int64_t threads = int64_t(t.nL) * t.nL * 8;
     const unsigned blocks = unsigned((threads + 255) / 256);
-    switch (t.P1) {
+    if constexpr (sizeof(T) == 4) {
+        switch (t.P1) {
 #define PP_CASE(P) \
-    case P: k_p2m_reg<T, P><<<blocks, 256, 0, st>>>(t); break;
-        PP_FAST_ORDERS(PP_CASE)
+    case P: k_p2m_reg<T, P><<<blocks, 256, 0, st>>>(t); return cudaGetLastError();
+            PP_FAST_ORDERS(PP_CASE)
 #undef PP_CASE
-        default: k_p2m<T><<<blocks, 256, 0, st>>>(t); break;
+            default: break;
+        }
     }
+    k_p2m<T><<<blocks, 256, 0, st>>>(t);
     return cudaGetLastError();
 }
 
@@ -868,19 +871,15 @@ cudaError_t downward_fast(const Tree<T>& t, int l0, int l1, T* p_out, cudaStream
     return cudaSuccess;
 }
 
-// FP64 keeps the register kernels only where they fit without spilling.
-template <typename T>
-inline bool fast_order_ok(int P1) {
-    return sizeof(T) == 4 || P1 <= 21;
-}
-
+// FP64 plans have kernels of their own (pp_fp64.cuh) for orders up to 23, and the generic ones
+// beyond and on grids of fewer than 4 x 4 leaves.
 template <typename T>
 int upward_launches(const Tree<T>& t) {
     bool fast = false;
 #define PP_CASE(P) fast = fast || t.P1 == P;
     PP_FAST_ORDERS(PP_CASE)
 #undef PP_CASE
-    if (!fast || !fast_order_ok<T>(t.P1)) return t.Lleaf;
+    if (!fast || sizeof(T) != 4) return t.Lleaf;
     if (sizeof(T) == 4 && t.up_counter && t.Lleaf >= 1 && t.Lleaf <= 8) return 1;
     // levels Lleaf-1 .. 4 one launch each, levels <= 3 in one
     return (t.Lleaf - 1 > 3 ? t.Lleaf - 4 : 0) + (t.Lleaf >= 1 ? 1 : 0);
@@ -888,7 +887,7 @@ int upward_launches(const Tree<T>& t) {
 
 template <typename T>
 cudaError_t launch_upward(const Tree<T>& t, cudaStream_t st) {
-    switch (fast_order_ok<T>(t.P1) ? t.P1 : 0) {
+    if constexpr (sizeof(T) == 4) switch (t.P1) {
 #define PP_CASE(P) \
     case P: return upward_fast<T, P>(t, st);
         PP_FAST_ORDERS(PP_CASE)
@@ -908,7 +907,7 @@ cudaError_t launch_upward(const Tree<T>& t, cudaStream_t st) {
 // every cell to the near field already stored in p_out (register kernels only).
 template <typename T>
 cudaError_t launch_downward_levels(const Tree<T>& t, int l0, int l1, T* p_out, cudaStream_t st) {
-    switch (fast_order_ok<T>(t.P1) ? t.P1 : 0) {
+    if constexpr (sizeof(T) == 4) switch (t.P1) {
 #define PP_CASE(P) \
     case P: return downward_fast<T, P>(t, l0, l1, p_out, st);
         PP_FAST_ORDERS(PP_CASE)
@@ -1010,7 +1009,7 @@ cudaError_t launch_down_tree(const Tree<T>& t, T* p_out, cudaStream_t st) {
 
 template <typename T>
 cudaError_t launch_downward(const Tree<T>& t, cudaStream_t st) {
-    switch (fast_order_ok<T>(t.P1) ? t.P1 : 0) {
+    if constexpr (sizeof(T) == 4) switch (t.P1) {
 #define PP_CASE(P) \
     case P: return downward_fast<T, P>(t, 2, t.Lleaf, (T*)nullptr, st);
         PP_FAST_ORDERS(PP_CASE)
@@ -1120,9 +1119,17 @@ template <typename T>
 cudaError_t launch_surface(const Tree<T>& t, const T* u, const T* v, const SurfaceArgs& a,
                            cudaStream_t st) {
     const unsigned nb4 = unsigned((a.npts + 3) / 4);
-    switch (t.P1) {
+    bool done = false;
+    if constexpr (sizeof(T) == 8) {
+        if (f64_ok(t.P1, t.Lleaf)) {
+            done = true;
+            const cudaError_t e = launch_treecode64(t, a, st);
+            if (e != cudaSuccess) return e;
+        }
+    }
+    if (!done) switch (sizeof(T) == 4 ? t.P1 : 0) {
 #define PP_CASE(P) \
-    case P: k_treecode<T, P><<<nb4, 128, 0, st>>>(t, a); break;
+    case P: k_treecode<T, sizeof(T) == 4 ? P : 0><<<nb4, 128, 0, st>>>(t, a); break;
         PP_FAST_ORDERS(PP_CASE)
 #undef PP_CASE
         default: k_treecode<T, 0><<<nb4, 128, 0, st>>>(t, a); break;

@@ -1,6 +1,7 @@
 // Instantiation of the pressure-recovery kernels for T = double.
 #define PP_REAL double
 #include "pp_kernels.cuh"
+#include "pp_fp64.cuh"
 
 namespace pp {
 
