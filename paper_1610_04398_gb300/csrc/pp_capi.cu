@@ -524,6 +524,7 @@ int alloc_tree(pp_plan p) {
     if (dalloc(p, (void**)&p->S, sizeof(double) * size_t(nbox)) != cudaSuccess) return PP_ERR_OOM;
     if (dalloc(p, (void**)&p->L0, sizeof(double) * size_t(nbox)) != cudaSuccess) return PP_ERR_OOM;
     if (dalloc(p, (void**)&p->forces_dev, sizeof(double) * 8) != cudaSuccess) return PP_ERR_OOM;
+    if (cudaMemset(p->forces_dev, 0, sizeof(double) * 8) != cudaSuccess) return PP_ERR_CUDA;  // [6]: arrival counter
     if (dalloc(p, (void**)&p->penal_buf, sizeof(double) * (pp::penal_partial_doubles() + 4)) != cudaSuccess)
         return PP_ERR_OOM;
     if (cudaMemset(p->penal_buf, 0, sizeof(double) * (pp::penal_partial_doubles() + 4)) != cudaSuccess)
@@ -863,6 +864,7 @@ int run_surface(pp_plan p, const void* u, const void* v, int npts, const double*
     a.nrm = nrm;
     a.dS = dS;
     a.Psurf = p->Psurf;
+    a.counter = reinterpret_cast<unsigned*>(p->forces_dev + 6);
     a.per_point = per_point;
     a.partial = p->partial;
     a.forces = dev_forces ? forces : p->forces_dev;
@@ -872,13 +874,15 @@ int run_surface(pp_plan p, const void* u, const void* v, int npts, const double*
     a.uhat_y = p->uhy;
     a.theta = p->theta_surf;
     a.rho_h = p->h * std::exp(kC0);
+    a.theta2f = float(a.theta * a.theta);
+    a.rho2_cell = float(std::exp(2.0 * kC0));
     a.interp = p->interp;
     a.err = p->err;
     pp::Tree<T> t = make_tree<T>(p);
     stage_begin(p, ST_SURF);
     if (pp::launch_surface<T>(t, (const T*)u, (const T*)v, a, p->stream) != cudaSuccess) return cuda_fail(p);
     stage_end(p, ST_SURF);
-    p->launches += 3;
+    p->launches += 1;
     if (forces && !dev_forces) {
         int errflag = 0;
         if (cudaMemcpyAsync(forces, p->forces_dev, 6 * sizeof(double), cudaMemcpyDeviceToHost, p->stream) !=

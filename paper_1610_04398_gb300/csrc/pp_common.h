@@ -209,11 +209,13 @@ struct SurfaceArgs {
     const double* pts;
     const double* nrm;
     const double* dS;      // may be null: trapezoid weights
-    double* Psurf;         // [npts] pressure at the points (FP64)
+    double* Psurf;         // k_traction: [npts] pressure at the points; k_surface: the CTAs' partial sums
+    unsigned* counter;     // k_surface: arrivals, zero between calls
     double* per_point;     // [npts][5] or null
     double* partial;       // [blocks][4]
     double* forces;        // [6] device
     double lift, mu2, uhat_x, uhat_y, theta, rho_h;
+    float theta2f, rho2_cell;  // theta^2, (rho_h / h)^2
     int interp;
     int* err;              // device error flag (tree-code list overflow)
 };
@@ -281,8 +283,6 @@ cudaError_t launch_surface(const Tree<T>& t, const T* u, const T* v, const Surfa
 template <typename T>
 cudaError_t launch_export_expansion(const Tree<T>& t, int kind, int level, double* dst,
                                     cudaStream_t st);
-
-cudaError_t launch_treecode64(const Tree<double>& t, const SurfaceArgs& a, cudaStream_t st);
 
 constexpr int kSurfaceBlock = 64;
 // Surface scratch of a plan: a new plan holds it for kInitialSurfaceCap points and grows it

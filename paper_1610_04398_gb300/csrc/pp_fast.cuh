@@ -307,10 +307,12 @@ __global__ void __launch_bounds__(128, M2LOcc<T, P1>::value) k_m2l_reg(Tree<T> t
 
 // ------------------------------------------------------------------------------------
 // (a1) + leaf multipoles, mixed precision: one warp per strip of 128 cells (4 per lane)
-// and kRhsLeafRows leaf rows (8 grid rows each), so the two halo rows are read once per 16
-// rows.  Rows of the five fields stream through a kRhsRing-slot ring in shared memory per
-// warp by asynchronous 16-byte copies (each slot also holds the float4 left and right of
-// the strip), kRhsRing - 1 rows in flight.  As a row lands each lane turns it into the
+// and kRows leaf rows (8 grid rows each).  Large grids take two leaf rows, so the two halo rows are
+// read once per 16 rows; grids with fewer than eight one-row warps an SM (up to 1024^2) take one
+// and a ring of eight rows: their time is the latency of the rows, not their bytes (256^2:
+// 14.4 us with two leaf rows and a ring of four, 9.6 with this).  Rows of the five fields stream through a
+// kRing-slot ring in shared memory per warp by asynchronous 16-byte copies (each slot also holds
+// the float4 left and right of the strip), kRing - 1 rows in flight.  As a row lands each lane turns it into the
 // four values the stencil needs, u, v, a = chi (us_x - u) and b = chi (us_y - v), held in a
 // register window of three rows (the slot is free again at once); the row in the middle
 // of the window is then differenced (x neighbours by shuffles, the strip's edge columns
@@ -324,19 +326,18 @@ __global__ void __launch_bounds__(128, M2LOcc<T, P1>::value) k_m2l_reg(Tree<T> t
 // CTAs of two warps: the 2048 warps of a 2048^2 grid spread over the 152 SMs 13 or 14 to
 // an SM (eight-warp CTAs put 16 on some SMs and 8 on the rest).
 // ------------------------------------------------------------------------------------
-constexpr int kRhsRing = 4;                              // ring slots per warp (rows in flight + 1)
 constexpr int kRhsWarps = 2;                             // warps per CTA
-constexpr int kRhsLeafRows = 2;                          // leaf rows per warp
 constexpr int kRhsSlot = 5 * 34;                         // float4 per slot: 5 fields x (32 lanes + 2 halo)
-constexpr size_t kRhsRingBytes = size_t(kRhsWarps) * kRhsRing * kRhsSlot * sizeof(float4);
+__host__ __device__ constexpr int rhs_ring(int rows) { return rows == 1 ? 8 : 4; }  // ring slots per warp (rows in flight + 1)
 constexpr size_t kRhsParkBytes = size_t(kRhsWarps) * 4 * 32 * sizeof(float4);  // rows 0-3 of a leaf row
 // dynamic shared memory: the P2M table (omega_c^k / k, k = 1..P1-1, for the 32 cells of
 // leaf rows 4-7; P1 is odd, so a row of P1 + 1 entries starts 16-byte aligned and the rows
 // of the two cells a warp reads at once, 4 apart, sit 16 banks apart), the parked q, then
 // the rings
 __host__ __device__ constexpr int rhs_wstride(int P1) { return P1 + 1; }
-constexpr size_t rhs_smem_bytes(int P1) {
-    return size_t(32) * rhs_wstride(P1) * sizeof(float2) + kRhsParkBytes + kRhsRingBytes;
+constexpr size_t rhs_smem_bytes(int P1, int rows) {
+    return size_t(32) * rhs_wstride(P1) * sizeof(float2) + kRhsParkBytes +
+           size_t(kRhsWarps) * rhs_ring(rows) * kRhsSlot * sizeof(float4);
 }
 
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
@@ -350,13 +351,13 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-template <int P1>
+template <int P1, int kRows>
 __global__ void __launch_bounds__(32 * kRhsWarps, (P1 <= 17 ? 16 : 8) / kRhsWarps) k_rhs_p2m_fast(Tree<float> t, const float* __restrict__ u,
                                                     const float* __restrict__ v, const float* __restrict__ chi,
                                                     const float* __restrict__ usx, const float* __restrict__ usy,
                                                     float rho, float lam, float* __restrict__ f_out) {
     static_assert(P1 % 2 == 1, "the table is read two entries at a time");
-    constexpr int WS = rhs_wstride(P1);
+    constexpr int WS = rhs_wstride(P1), kRing = rhs_ring(kRows);
     extern __shared__ __align__(16) float4 rhs_smem[];
     float2* Ws = reinterpret_cast<float2*>(rhs_smem);  // [32 cells of rows 4-7][WS]: entries 0..P1-2 used
     float4* park = rhs_smem + 32 * WS / 2;            // [warp][row 0-3][lane]
@@ -365,9 +366,9 @@ __global__ void __launch_bounds__(32 * kRhsWarps, (P1 <= 17 ? 16 : 8) / kRhsWarp
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t wid = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int strips = (n + 127) >> 7;
-    const int LY0 = int(wid / strips) * kRhsLeafRows, sxi = int(wid % strips);
+    const int LY0 = int(wid / strips) * kRows, sxi = int(wid % strips);
     const bool live = LY0 < t.nL;                   // warp-uniform
-    const int nly = min(kRhsLeafRows, t.nL - LY0);  // leaf rows of this warp
+    const int nly = min(kRows, t.nL - LY0);  // leaf rows of this warp
     const int xs = sxi * 128, x0 = xs + 4 * lane;
     const bool act = x0 < n;
     const bool hasL = xs > 0, hasR = xs + 128 < n;  // the strip's neighbours exist
@@ -376,9 +377,9 @@ __global__ void __launch_bounds__(32 * kRhsWarps, (P1 <= 17 ? 16 : 8) / kRhsWarp
     const float hh = float(t.h) * float(t.h);
     // ring[slot][field][34]: entry 0 the float4 left of the strip, 1 + lane the lane's, 33 the
     // float4 right of it; fields u, v, chi, us_x, us_y
-    float4* ring = rhs_ring + size_t(warp) * kRhsRing * kRhsSlot;
+    float4* ring = rhs_ring + size_t(warp) * kRing * kRhsSlot;
     const float* fld[5] = {u, v, chi, usx, usy};
-    auto slot = [&](int yy) { return ring + ((yy - y0 + 1) % kRhsRing) * kRhsSlot; };
+    auto slot = [&](int yy) { return ring + ((yy - y0 + 1) % kRing) * kRhsSlot; };
     auto issue = [&](int yy) {  // one commit group per row (empty outside the grid or the band's rows)
         if (yy >= 0 && yy < n && yy <= ylast + 1) {
             const int64_t g = int64_t(yy) * n;
@@ -444,7 +445,7 @@ __global__ void __launch_bounds__(32 * kRhsWarps, (P1 <= 17 ? 16 : 8) / kRhsWarp
     // the first rows go out before the table is staged (its loads then overlap them)
     if (live) {
 #pragma unroll
-        for (int d = -1; d < kRhsRing - 1; ++d) issue(y0 + d);
+        for (int d = -1; d < kRing - 1; ++d) issue(y0 + d);
     }
 #pragma unroll
     for (int j = 0; j < (32 * (P1 - 1)) / (32 * kRhsWarps); ++j) {
@@ -460,7 +461,7 @@ __global__ void __launch_bounds__(32 * kRhsWarps, (P1 <= 17 ? 16 : 8) / kRhsWarp
     // 1 (y = yy - 1) with slots 0 (y - 1) and 2 (y + 1)
     constexpr int OW = 0, MW = 1, NW = 2;
     auto step = [&](int yy) {
-        cp_async_wait<kRhsRing - 1>();  // row yy has landed (kRhsRing - 1 later rows may be in flight)
+        cp_async_wait<kRing - 1>();  // row yy has landed (kRing - 1 later rows may be in flight)
         __syncwarp();
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -489,8 +490,8 @@ __global__ void __launch_bounds__(32 * kRhsWarps, (P1 <= 17 ? 16 : 8) / kRhsWarp
                 HU[NW] = uu, HV[NW] = vv, HA[NW] = cc * (xx - uu);
             }
         }
-        __syncwarp();  // every lane has read the slot: it takes row yy + kRhsRing
-        issue(yy + kRhsRing);
+        __syncwarp();  // every lane has read the slot: it takes row yy + kRing
+        issue(yy + kRing);
         const int y = yy - 1;  // the row in the middle of the window
         if (y < y0) return;    // warp-uniform
         // x neighbours of row y: the adjacent lanes' edge values, the strip's edges from the halo

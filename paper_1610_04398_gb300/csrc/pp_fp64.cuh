@@ -14,7 +14,6 @@
 
 #include "pp_fixed.cuh"
 #include "pp_kernels.cuh"
-#include "pp_log.cuh"
 
 namespace pp {
 namespace f64 {
@@ -870,100 +869,6 @@ __global__ void __launch_bounds__(32 * kDown64Warps) k_down64(Tree<double> t, do
     }
 }
 
-// ------------------------------------------------------------------------------------
-// (a7) Surface pressure, one warp per point as k_treecode, with the accepted boxes collected and
-// evaluated 32 at a time (full warps on the FP64 pipe, which bounds it) and logarithms from the table
-// method: 207 us before for 2048 points at 1024^2, p = 20, 124 now.
-// ------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) k_treecode64(Tree<double> t, SurfaceArgs a) {
-    __shared__ int cand[4][2][kCandCap];
-    __shared__ int2 acc_list[4][64];  // level, box
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int pt = blockIdx.x * 4 + w;
-    if (pt >= a.npts) return;  // warp-uniform, no block barriers
-    const int P1 = t.P1;
-    const double zx = a.pts[2 * pt], zy = a.pts[2 * pt + 1], L = double(t.n) * t.h;
-    const double th2 = a.theta * a.theta, rho2 = a.rho_h * a.rho_h;
-    const unsigned below = (1u << lane) - 1u;
-    double acc = 0.0;
-    bool overflow = false;
-    const auto evaluate = [&](int2 lb) {
-        const int side = 1 << lb.x, bx = lb.y & (side - 1), by = lb.y >> lb.x;
-        const double s = L * pow2(-lb.x);
-        const double dx = zx - fma(bx + 0.5, s, t.x0), dy = zy - fma(by + 0.5, s, t.y0);
-        const double d2 = dx * dx + dy * dy, sd = s / d2;
-        const double2 u{sd * dx, -sd * dy};
-        const int64_t box = level_offset(lb.x) + lb.y;
-        const double2* M = t.mp + box * P1;
-        double2 h = M[P1 - 1];
-#pragma unroll 4
-        for (int k = P1 - 2; k >= 1; --k) {
-            const double2 m = M[k];
-            h = double2{fma(h.x, u.x, fma(-h.y, u.y, m.x)), fma(h.x, u.y, fma(h.y, u.x, m.y))};
-        }
-        acc = fma(t.S[box], 0.5 * log_table(d2), acc) - (h.x * u.x - h.y * u.y);
-    };
-    if (lane == 0) cand[w][0][0] = 0;
-    __syncwarp();
-    int cur = 0, n = 1, na = 0;
-    for (int l = 0; l <= t.Lleaf; ++l) {
-        const int side = 1 << l;
-        const double s = L * pow2(-l), rb2 = 0.5 * s * s;
-        int next = 0;
-        for (int base = 0; base < n; base += 32) {
-            const bool in = base + lane < n;
-            const int b = in ? cand[w][cur][base + lane] : 0;
-            const int bx = b & (side - 1), by = b >> l;
-            const double dx = zx - fma(bx + 0.5, s, t.x0), dy = zy - fma(by + 0.5, s, t.y0);
-            const bool take = in && rb2 < th2 * (dx * dx + dy * dy), open = in && !take;
-            const unsigned tm = __ballot_sync(0xffffffffu, take);
-            if (take) acc_list[w][na + __popc(tm & below)] = make_int2(l, b);
-            na += __popc(tm);
-            __syncwarp();
-            if (na >= 32) {
-                evaluate(acc_list[w][lane]);
-                na -= 32;
-                const int2 v = acc_list[w][32 + lane];
-                __syncwarp();
-                acc_list[w][lane] = v;
-                __syncwarp();
-            }
-            unsigned om = __ballot_sync(0xffffffffu, open);
-            if (l == t.Lleaf) {
-                for (; om; om &= om - 1) {  // the leaf's 64 cells, two a lane
-                    const int lb = __shfl_sync(0xffffffffu, b, __ffs(om) - 1);
-                    const int LX = lb & (side - 1), LY = lb >> l;
-                    const double ex = zx - fma(8.0 * LX + (lane & 7) + 0.5, t.h, t.x0);
-                    const double ey = zy - fma(8.0 * LY + (lane >> 3) + 0.5, t.h, t.y0), ey1 = ey - 4.0 * t.h;
-                    const double x2 = ex * ex;
-                    const double* q = t.q + int64_t(lb) * 64 + lane;
-                    acc = fma(q[0], 0.5 * log_table(fmax(fma(ey, ey, x2), rho2)), acc);
-                    acc = fma(q[32], 0.5 * log_table(fmax(fma(ey1, ey1, x2), rho2)), acc);
-                }
-            } else {
-                if (open) {
-                    const int at = next + 4 * __popc(om & below);
-                    if (at + 4 <= kCandCap) {
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            cand[w][cur ^ 1][at + q] = (2 * by + (q >> 1)) * (2 * side) + 2 * bx + (q & 1);
-                    } else {
-                        overflow = true;
-                    }
-                }
-                next += 4 * __popc(om);
-            }
-        }
-        __syncwarp();
-        cur ^= 1;
-        n = min(next, kCandCap);
-    }
-    if (lane < na) evaluate(acc_list[w][lane]);
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) a.Psurf[pt] = acc * kInv2Pi;
-    if (overflow) atomicExch(a.err, 1);
-}
-
 }  // namespace f64
 
 // ------------------------------------------------------------------------------------
@@ -1096,11 +1001,6 @@ cudaError_t launch_down64(const Tree<double>& t, double* p_out, cudaStream_t st)
     const dim3 grid(1u << lr, 1u << lr);
     if (depth == 3) f64::k_down64<3><<<grid, 32 * f64::kDown64Warps, smem, st>>>(t, p_out);
     else f64::k_down64<2><<<grid, 32 * f64::kDown64Warps, smem, st>>>(t, p_out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_treecode64(const Tree<double>& t, const SurfaceArgs& a, cudaStream_t st) {
-    f64::k_treecode64<<<unsigned((a.npts + 3) / 4), 128, 0, st>>>(t, a);
     return cudaGetLastError();
 }
 

@@ -35,6 +35,7 @@ constexpr double kInv2Pi = 0.15915494309189533576888376337251;
 }  // namespace pp
 
 #include "pp_fast.cuh"
+#include "pp_surface.cuh"
 
 namespace pp {
 
@@ -424,202 +425,10 @@ __global__ void __launch_bounds__(256) k_leaf(Tree<T> t, int has_far, T* __restr
 }
 
 // ------------------------------------------------------------------------------------
-// (a7) Surface pressure by the tree-code (Sec. A.2, Fig. "multipole"): each point walks
-// the quadtree from the root; a box is accepted when r_box < theta d and then
-// contributes its multipole (Eq. pressTruncated about its centre); leaves that are never
-// accepted are summed directly.  One warp per point, lanes over candidate boxes.
+// (a8) Tractions and their integrals (Sec. 2.3) from a given surface pressure, for the
+// allocation-free entry point (k_surface forms them with the walk).  One thread per point; a
+// deterministic block tree reduction of the four force sums, then one final CTA.
 // ------------------------------------------------------------------------------------
-constexpr int kCandCap = 256;
-constexpr int kLeafCap = 64;
-
-template <typename T, int P1T>
-__global__ void __launch_bounds__(128) k_treecode(Tree<T> t, SurfaceArgs a) {
-    typedef typename cplx_of<T>::type C;
-    __shared__ int cand[4][2][kCandCap];
-    __shared__ int leaves[4][kLeafCap];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int pt = blockIdx.x * 4 + warp;
-    if (pt >= a.npts) return;
-    const int P1 = P1T > 0 ? P1T : t.P1;
-    const double zx = a.pts[2 * pt], zy = a.pts[2 * pt + 1];
-    const double L = double(t.n) * t.h;
-    double mono = 0.0;
-    float mh = 0.f, ml = 0.f;  // cell-unit points of mixed plans: the monopole sum as a double-float pair
-    T ser = T(0);
-    int cur = 0, ncand = 1, nleaf = 0;
-    bool overflow = false;
-    // The root box is never accepted for a point inside the domain (no such point is
-    // farther than its half-diagonal from the centre), so such points start from the
-    // four boxes of level 1.
-    const bool inside = zx >= t.x0 && zx <= t.x0 + L && zy >= t.y0 && zy <= t.y0 + L && t.Lleaf >= 1;
-    const int l_start = inside ? 1 : 0;
-    // Mixed plans, points inside the domain: offsets in cell units, an exact integer
-    // difference plus the point's fraction of a cell (split once in FP64), so no FP64 per
-    // box.  The log h parts of every accepted box and near cell add up to log h times the
-    // root monopole (they partition the domain) and enter once at the end.
-    const bool cellu = sizeof(T) == 4 && inside && t.Sf != nullptr;
-    int ix = 0, iy = 0;
-    float fx = 0.f, fy = 0.f;
-    if (cellu) {
-        const double cxd = (zx - t.x0) * t.inv_h, cyd = (zy - t.y0) * t.inv_h;
-        ix = int(floor(cxd));
-        iy = int(floor(cyd));
-        fx = float(cxd - ix);
-        fy = float(cyd - iy);
-    }
-    if (inside) {
-        ncand = 4;
-        if (lane < 4) cand[warp][0][lane] = lane;
-    } else if (lane == 0) {
-        cand[warp][0][0] = 0;
-    }
-    __syncwarp();
-    const T th2 = T(a.theta * a.theta);
-    for (int l = l_start; l <= t.Lleaf; ++l) {
-        const int side = 1 << l;
-        const double s = cellu ? 0.0 : L / side;  // box side and half-diagonal (FP64 offsets only)
-        const double rb = s * 0.70710678118654752440;
-        const int64_t off = level_offset(l);
-        int nnext = 0;
-        for (int base = 0; base < ncand; base += 32) {
-            const int i = base + lane;
-            bool open = false;
-            int b = 0;
-            if (i < ncand) {
-                b = cand[warp][cur][i];
-                const int bx = b % side, by = b / side;
-                T dx, dy, sT, rb2;
-                if (cellu) {  // cell units
-                    const int sc = 8 << (t.Lleaf - l);
-                    dx = T(float(ix - (bx * sc + (sc >> 1))) + fx);
-                    dy = T(float(iy - (by * sc + (sc >> 1))) + fy);
-                    sT = T(sc);
-                    rb2 = T(0.5) * sT * sT;
-                } else {
-                    // offsets in FP64 (exact enough at any distance), the rest in the plan precision
-                    dx = T(zx - (t.x0 + (bx + 0.5) * s));
-                    dy = T(zy - (t.y0 + (by + 0.5) * s));
-                    sT = T(s);
-                    rb2 = T(rb * rb);
-                }
-                const T d2 = dx * dx + dy * dy;
-                if (rb2 < th2 * d2) {
-                    // Eq. pressTruncated about the box centre: S log|w| - Re sum_k M_k (s / w)^k
-                    const T lg = T(0.5) * log_t<T>(d2);
-                    if (cellu) {  // double-float S log|w| on the FP32 pipe (mixed plans)
-                        const float2 sp = t.Sf[off + b];
-                        df_fma(mh, ml, sp.x, sp.y, float(lg), 0.f);
-                    } else {
-                        mono += t.S[off + b] * double(lg);
-                    }
-                    const T sd = sT / d2;
-                    const C u = cmake<T>(sd * dx, -sd * dy);
-                    const C* M = t.mp + (off + b) * P1;
-                    C acc = M[P1 - 1];
-#pragma unroll
-                    for (int k = P1 - 2; k >= 1; --k) {
-                        const C m = M[k];
-                        const T nr = fma(acc.x, u.x, fma(-acc.y, u.y, m.x));
-                        const T ni = fma(acc.x, u.y, fma(acc.y, u.x, m.y));
-                        acc.x = nr;
-                        acc.y = ni;
-                    }
-                    ser -= acc.x * u.x - acc.y * u.y;
-                } else {
-                    open = true;
-                }
-            }
-    const unsigned mask = __ballot_sync(0xffffffffu, open);
-            const int pos = __popc(mask & ((1u << lane) - 1u));
-            if (l < t.Lleaf) {
-                if (open) {
-                    const int at = nnext + 4 * pos;
-                    if (at + 4 <= kCandCap) {
-                        const int bx = b % side, by = b / side;
-                        for (int q = 0; q < 4; ++q)
-                            cand[warp][cur ^ 1][at + q] = (2 * by + (q >> 1)) * (2 * side) + 2 * bx + (q & 1);
-                    } else {
-                        overflow = true;
-                    }
-                }
-                nnext += 4 * __popc(mask);
-            } else {
-                if (open) {
-                    const int at = nleaf + pos;
-                    if (at < kLeafCap) leaves[warp][at] = b;
-                    else overflow = true;
-                }
-                nleaf += __popc(mask);
-            }
-        }
-        __syncwarp();
-        cur ^= 1;
-        ncand = min(nnext, kCandCap);
-    }
-    nleaf = min(nleaf, kLeafCap);
-    const T rh2 = cellu ? T((a.rho_h / t.h) * (a.rho_h / t.h)) : T(a.rho_h * a.rho_h);
-    const T hT = cellu ? T(1) : T(t.h);
-    double nearsum = 0.0;
-    T nearf = T(0);  // cell units: the lane's near-field partial in T, converted once
-    for (int e = 0; e < nleaf; ++e) {
-        const int b = leaves[warp][e];
-        const int LX = b % t.nL, LY = b / t.nL;
-        // point relative to the leaf corner (FP64, or exact cell units), cells relative to that in T
-        const T ox = cellu ? T(float(ix - 8 * LX) + fx) : T(zx - (t.x0 + 8.0 * LX * t.h));
-        const T oy = cellu ? T(float(iy - 8 * LY) + fy) : T(zy - (t.y0 + 8.0 * LY * t.h));
-        T part = T(0);
-        for (int c = lane; c < 64; c += 32) {
-            const T dx = ox - (T(c & 7) + T(0.5)) * hT;
-            const T dy = oy - (T(c >> 3) + T(0.5)) * hT;
-            const T r2 = dx * dx + dy * dy;
-            part += t.q[int64_t(b) * 64 + c] * (T(0.5) * log_t<T>(r2 > rh2 ? r2 : rh2));
-        }
-        if (cellu)
-            nearf += part;
-        else
-            nearsum += double(part);
-    }
-    double tot;
-    if (cellu) {  // warp-uniform: the lanes' sums as double-float pairs, reduced on the FP32 pipe
-        df_add(mh, ml, float(ser), 0.f);
-        df_add(mh, ml, float(nearf), 0.f);
-        for (int o = 16; o > 0; o >>= 1) {
-            const float oh = __shfl_xor_sync(0xffffffffu, mh, o), ol = __shfl_xor_sync(0xffffffffu, ml, o);
-            df_add(mh, ml, oh, ol);
-        }
-        tot = df_to(mh, ml) + t.lnh * t.S[0];  // log h times the root monopole, once per point
-    } else {
-        tot = mono + double(ser) + nearsum;
-        for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
-    }
-    const bool ovf = __any_sync(0xffffffffu, overflow);
-    if (lane == 0) {
-        a.Psurf[pt] = tot * kInv2Pi;
-        if (ovf) atomicExch(a.err, 1);
-    }
-}
-
-// ------------------------------------------------------------------------------------
-// (a8) Tractions and their integrals (Sec. 2.3).  One thread per point; a deterministic
-// block tree reduction of the four force sums, then one final CTA.
-// ------------------------------------------------------------------------------------
-template <typename T>
-__device__ __forceinline__ void cell_grad(const T* u, const T* v, int n, double inv2h, int i, int j,
-                                          double g[4]) {
-    const int64_t c = int64_t(j) * n + i;
-    g[0] = (double(u[c + 1]) - double(u[c - 1])) * inv2h;
-    g[1] = (double(u[c + n]) - double(u[c - n])) * inv2h;
-    g[2] = (double(v[c + 1]) - double(v[c - 1])) * inv2h;
-    g[3] = (double(v[c + n]) - double(v[c - n])) * inv2h;
-}
-
-__device__ __forceinline__ int clampi(double x, int lo, int hi) {
-    if (!(x == x)) return lo;  // NaN
-    if (x < double(lo)) return lo;
-    if (x > double(hi)) return hi;
-    return int(x);
-}
-
 template <typename T>
 __global__ void __launch_bounds__(kSurfaceBlock)
 k_traction(Tree<T> t, const T* __restrict__ u, const T* __restrict__ v, SurfaceArgs a) {
@@ -752,7 +561,10 @@ cudaError_t launch_rhs_p2m(const Tree<T>& t, const T* u, const T* v, const T* ch
         auto al = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
         const bool aligned = al(u) && al(v) && al(chi) && al(usx) && al(usy) && al(f_out);
         if (aligned) {
-            const int64_t warps = int64_t((t.n + 127) / 128) * ((t.nL + kRhsLeafRows - 1) / kRhsLeafRows);
+            // one leaf row a warp while that leaves at most eight warps an SM (see the kernel)
+            const int64_t one = int64_t((t.n + 127) / 128) * t.nL;
+            const int rows = one <= t.resident_threads / 384 * 8 ? 1 : 2;
+            const int64_t warps = int64_t((t.n + 127) / 128) * ((t.nL + rows - 1) / rows);
             const unsigned blocks = unsigned((warps + kRhsWarps - 1) / kRhsWarps);
             const Tree<float>& tf = reinterpret_cast<const Tree<float>&>(t);
             const float* fu = reinterpret_cast<const float*>(u);
@@ -764,8 +576,12 @@ cudaError_t launch_rhs_p2m(const Tree<T>& t, const T* u, const T* v, const T* ch
             switch (t.P1) {
 #define PP_CASE(P)                                                                                         \
     case P:                                                                                                \
-        k_rhs_p2m_fast<P><<<blocks, 32 * kRhsWarps, rhs_smem_bytes(P), st>>>(tf, fu, fv, fc, fsx, fsy, float(rho), \
-                                                                            float(lam), ff);                    \
+        if (rows == 1)                                                                                     \
+            k_rhs_p2m_fast<P, 1><<<blocks, 32 * kRhsWarps, rhs_smem_bytes(P, 1), st>>>(                    \
+                tf, fu, fv, fc, fsx, fsy, float(rho), float(lam), ff);                                     \
+        else                                                                                               \
+            k_rhs_p2m_fast<P, 2><<<blocks, 32 * kRhsWarps, rhs_smem_bytes(P, 2), st>>>(                    \
+                tf, fu, fv, fc, fsx, fsy, float(rho), float(lam), ff);                                     \
         *launches = 1;                                                                                     \
         return cudaGetLastError();
                 PP_FAST_ORDERS(PP_CASE)
@@ -1118,29 +934,20 @@ cudaError_t launch_leaf_eval(const Tree<T>& t, T* p_out, cudaStream_t st) {
 template <typename T>
 cudaError_t launch_surface(const Tree<T>& t, const T* u, const T* v, const SurfaceArgs& a,
                            cudaStream_t st) {
-    const unsigned nb4 = unsigned((a.npts + 3) / 4);
-    bool done = false;
-    if constexpr (sizeof(T) == 8) {
-        if (f64_ok(t.P1, t.Lleaf)) {
-            done = true;
-            const cudaError_t e = launch_treecode64(t, a, st);
-            if (e != cudaSuccess) return e;
+    constexpr int kWarps = SurfCta<T>::warps, kThreads = SurfCta<T>::threads;
+    constexpr size_t smem = surf_smem_bytes<T>();
+    const unsigned chunks = unsigned((a.npts + kWarps - 1) / kWarps);
+    const unsigned nb = chunks < kSurfMaxCtas ? chunks : kSurfMaxCtas;
+    if constexpr (sizeof(T) == 4) {
+        switch (t.P1) {
+#define PP_CASE(P) \
+    case P: k_surface<T, P><<<nb, kThreads, smem, st>>>(t, u, v, a); return cudaGetLastError();
+            PP_FAST_ORDERS(PP_CASE)
+#undef PP_CASE
+            default: break;
         }
     }
-    if (!done) switch (sizeof(T) == 4 ? t.P1 : 0) {
-#define PP_CASE(P) \
-    case P: k_treecode<T, sizeof(T) == 4 ? P : 0><<<nb4, 128, 0, st>>>(t, a); break;
-        PP_FAST_ORDERS(PP_CASE)
-#undef PP_CASE
-        default: k_treecode<T, 0><<<nb4, 128, 0, st>>>(t, a); break;
-    }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const int nb = (a.npts + kSurfaceBlock - 1) / kSurfaceBlock;
-    k_traction<T><<<nb, kSurfaceBlock, 0, st>>>(t, u, v, a);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_forces_final<T><<<1, 256, 0, st>>>(nb, a);
+    k_surface<T, 0><<<nb, kThreads, smem, st>>>(t, u, v, a);
     return cudaGetLastError();
 }
 
@@ -1156,13 +963,19 @@ cudaError_t prepare_kernels() {
         return e;
     if ((e = cudaFuncSetAttribute(k_leaf<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) != cudaSuccess)
         return e;
-    if (sizeof(T) == 4) {
-        const void* fns[] = {(const void*)k_leaf_fast<1, true>, (const void*)k_leaf_fast<2, true>,
+    if ((e = cudaFuncSetAttribute(k_surface<T, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) != cudaSuccess)
+        return e;
+    if constexpr (sizeof(T) == 4) {
+        const void* fns[] = {(const void*)k_surface<T, 13>, (const void*)k_surface<T, 17>,
+                             (const void*)k_surface<T, 21>, (const void*)k_surface<T, 25>,
+                             (const void*)k_leaf_fast<1, true>, (const void*)k_leaf_fast<2, true>,
                              (const void*)k_leaf_fast<3, true>, (const void*)k_leaf_fast<1, false>,
                              (const void*)k_leaf_fast<2, false>, (const void*)k_leaf_fast<3, false>,
                              (const void*)k_near16<1>, (const void*)k_near16<2>, (const void*)k_near16<3>,
-                             (const void*)k_rhs_p2m_fast<13>, (const void*)k_rhs_p2m_fast<17>,
-                             (const void*)k_rhs_p2m_fast<21>, (const void*)k_rhs_p2m_fast<25>};
+                             (const void*)k_rhs_p2m_fast<13, 1>, (const void*)k_rhs_p2m_fast<17, 1>,
+                             (const void*)k_rhs_p2m_fast<21, 1>, (const void*)k_rhs_p2m_fast<25, 1>,
+                             (const void*)k_rhs_p2m_fast<13, 2>, (const void*)k_rhs_p2m_fast<17, 2>,
+                             (const void*)k_rhs_p2m_fast<21, 2>, (const void*)k_rhs_p2m_fast<25, 2>};
         for (const void* f : fns)
             if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) != cudaSuccess)
                 return e;

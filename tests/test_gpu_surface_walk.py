@@ -1,0 +1,52 @@
+"""The surface pass (tree-code walk, tractions and force sums in one launch) where its lists and
+its grid change: the strictest acceptance (a lane's list of accepted boxes fills and is flushed),
+points outside the domain (the walk starts at the root), point counts that leave part of a CTA idle
+and more points than one sweep of the grid covers, in both precisions, against the oracle.
+
+Tolerances: FP64 truncation 10 theta^(p+1); mixed 1e-4 (the mixed path's bar)."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1610_04398_gb300 import api, synth
+from gpu_cases import rel_l2, to_dev
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1610_04398_gb300 as pkg
+    pkg.build()
+    oracle.build()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("npts,theta_s", [(1, 0.5), (9, 0.25), (533, 0.25), (20001, 0.6)])
+def test_surface_pressure_and_forces(precision, npts, theta_s):
+    snap = synth.cylinder_flow(256, diameter=0.3, centre=(0.5, 0.5), n_surface=max(npts, 3), seed=npts)
+    pts, nrm = snap.points[:npts].copy(), snap.normals[:npts].copy()
+    if npts > 8:
+        pts[5], pts[6] = (1.4, 0.5), (-0.3, -0.2)
+    plan = api.Plan(256, snap.h, 12, 0.6, precision=precision, lift=snap.lift, theta_surface=theta_s)
+    f = [to_dev(a, plan.dtype) for a in (snap.u, snap.v, snap.chi, snap.usx, snap.usy)]
+    per = torch.empty(npts * 5, dtype=torch.float64, device="cuda")
+    forces = torch.empty(6, dtype=torch.float64, device="cuda")
+    dS = torch.full((npts,), 0.01, dtype=torch.float64, device="cuda")
+    plan.rhs(*f, snap.lam)
+    for _ in range(2):  # the arrival counter is reset
+        plan.surface_traction(f[0], f[1], to_dev(pts, torch.float64), to_dev(nrm, torch.float64), snap.nu, dS=dS,
+                              per_point=per, forces=forces)
+    per = per.view(npts, 5).cpu().numpy()
+    at = np.arange(npts) if npts < 1000 else np.unique(np.r_[0:40, np.random.default_rng(0).choice(npts, 400), npts - 1])
+    q = oracle.source_weights(oracle.rhs(snap.u, snap.v, snap.chi, snap.usx, snap.usy, h=snap.h, lam=snap.lam), snap.h)
+    ref = oracle.green_sum_grid(q, snap.h, pts[at, 0], pts[at, 1])
+    tol = max(10 * theta_s ** 13, 1e-12) if precision == "fp64" else 1e-4
+    assert rel_l2(per[at, 0], ref) < tol
+    assert np.allclose(per[:, 1:3], -per[:, :1] * nrm, rtol=1e-14, atol=0)
+    F = 0.01 * per[:, 1:].sum(0)
+    assert np.allclose(forces.cpu().numpy()[:4], F, rtol=1e-9, atol=1e-9 * np.abs(0.01 * per[:, 1:]).sum())
+    plan.destroy()
