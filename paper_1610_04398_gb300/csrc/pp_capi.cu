@@ -131,6 +131,8 @@ struct pp_plan_s {
     float2* lnTauF = nullptr;  // mixed plans: log|tau| as double-float pairs
     float2* Sf = nullptr;      // mixed plans: box monopoles as double-float pairs
     pp::M2LEntry* il = nullptr;
+    pp::M2LGroup* ig = nullptr;
+    int ig_groups[4] = {0, 0, 0, 0}, ig_count[4] = {0, 0, 0, 0};
     void* Ktab = nullptr;
     void* Krel = nullptr;
     int2* near = nullptr;
@@ -232,7 +234,7 @@ pp::Tree<T> make_tree(const pp_plan p) {
     t.x0 = p->x0;
     t.y0 = p->y0;
     t.q = static_cast<T*>(p->q);
-    t.mp = static_cast<C*>(p->mp);
+    t.mp = static_cast<C*>(p->mp) + (sizeof(T) == 4 ? 1 : 0);  // mixed: pairs of coefficients on 16 bytes
     t.S = p->S;
     t.loc = static_cast<C*>(p->loc);
     t.L0 = p->L0;
@@ -250,7 +252,12 @@ pp::Tree<T> make_tree(const pp_plan p) {
     t.lnTauF = p->lnTauF;
     t.Sf = p->Sf;
     t.il = p->il;
-    for (int c = 0; c < 4; ++c) t.il_count[c] = p->il_count[c];
+    t.ig = p->ig;
+    for (int c = 0; c < 4; ++c) {
+        t.il_count[c] = p->il_count[c];
+        t.ig_groups[c] = p->ig_groups[c];
+        t.ig_count[c] = p->ig_count[c];
+    }
     t.il_stride = p->il_stride;
     t.Ktab = static_cast<const T*>(p->Ktab);
     t.Krel = static_cast<const T*>(p->Krel);
@@ -405,6 +412,37 @@ int upload_tables(pp_plan p) {
         for (size_t i = 0; i < lists[c].size(); ++i) ilh[size_t(c) * p->il_stride + i] = lists[c][i];
     }
     p->il_host = ilh;
+    // the same lists with the sources at 90 degree rotations of one offset grouped, groups first
+    std::vector<pp::M2LGroup> igh;
+    if (sizeof(T) == 4) {
+        igh.assign(size_t(4) * p->il_stride, pp::M2LGroup{{-1, -1, -1, -1}, 0, {0, 0, 0}});
+        for (int c = 0; c < 4; ++c) {
+            const auto& lst = lists[c];
+            std::vector<char> used(lst.size(), 0);
+            std::vector<pp::M2LGroup> single;
+            int n = 0;
+            for (size_t i = 0; i < lst.size(); ++i) {
+                if (used[i]) continue;
+                pp::M2LGroup g{{-1, -1, -1, -1}, lst[i].op, {0, 0, 0}};
+                Op o = ops[lst[i].op];
+                int members = 0;
+                for (int j = 0; j < 4; ++j) {
+                    for (size_t k = i; k < lst.size(); ++k)
+                        if (!used[k] && ops[lst[k].op] == o) {
+                            used[k] = 1;
+                            g.m[j] = (lst[k].dx + 128) | (lst[k].dy + 128) << 8 | lst[k].pad << 16;
+                            ++members;
+                        }
+                    o = Op{-o.ty2, o.tx2, o.ratio};  // i tau
+                }
+                if (members > 1) igh[size_t(c) * p->il_stride + n++] = g;
+                else single.push_back(g);
+            }
+            p->ig_groups[c] = n;
+            for (auto& g : single) igh[size_t(c) * p->il_stride + n++] = g;
+            p->ig_count[c] = n;
+        }
+    }
     std::vector<int2> nh;
     for (auto& o : nearl) nh.push_back(make_int2(o.first, o.second));
     p->n_near = int(nh.size());
@@ -426,6 +464,11 @@ int upload_tables(pp_plan p) {
             return PP_ERR_CUDA;
     }
     if ((e = dalloc(p, (void**)&p->il, sizeof(pp::M2LEntry) * ilh.size())) != cudaSuccess) return PP_ERR_OOM;
+    if (!igh.empty()) {
+        if (dalloc(p, (void**)&p->ig, sizeof(pp::M2LGroup) * igh.size()) != cudaSuccess) return PP_ERR_OOM;
+        if (cudaMemcpy(p->ig, igh.data(), sizeof(pp::M2LGroup) * igh.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+            return PP_ERR_CUDA;
+    }
     if ((e = dalloc(p, &p->Ktab, sizeof(T) * K.size())) != cudaSuccess) return PP_ERR_OOM;
     if ((e = dalloc(p, &p->Krel, sizeof(T) * Kr.size())) != cudaSuccess) return PP_ERR_OOM;
     if ((e = dalloc(p, (void**)&p->near, sizeof(int2) * nh.size())) != cudaSuccess) return PP_ERR_OOM;
@@ -519,7 +562,8 @@ int alloc_tree(pp_plan p) {
     typedef typename pp::cplx_of<T>::type C;
     const int64_t nbox = pp::level_offset(p->Lleaf + 1);
     if (dalloc(p, &p->q, sizeof(T) * size_t(p->n) * p->n) != cudaSuccess) return PP_ERR_OOM;
-    if (dalloc(p, &p->mp, sizeof(C) * size_t(nbox) * p->P1) != cudaSuccess) return PP_ERR_OOM;
+    if (dalloc(p, &p->mp, sizeof(C) * (size_t(nbox) * p->P1 + (sizeof(T) == 4 ? 1 : 0))) != cudaSuccess)
+        return PP_ERR_OOM;
     if (dalloc(p, &p->loc, sizeof(C) * size_t(nbox) * p->P1) != cudaSuccess) return PP_ERR_OOM;
     if (dalloc(p, (void**)&p->S, sizeof(double) * size_t(nbox)) != cudaSuccess) return PP_ERR_OOM;
     if (dalloc(p, (void**)&p->L0, sizeof(double) * size_t(nbox)) != cudaSuccess) return PP_ERR_OOM;
@@ -585,7 +629,7 @@ int64_t plan_bytes(int n, int order, double theta, int precision, int tile, int 
     const int64_t nbox = pp::level_offset(Lleaf + 1);
     int64_t b = 0;
     b += al(sz * int64_t(n) * n);                                  // q
-    b += 2 * al(csz * nbox * P1);                                  // multipoles, locals
+    b += 2 * al(csz * nbox * P1) + (precision == PP_MIXED ? csz : 0);  // multipoles, locals
     b += 2 * al(8 * nbox);                                         // S, L0
     b += al(8 * 8);                                                // forces
     b += al(8 * (int64_t(pp::penal_partial_doubles()) + 4));       // penalisation partials
@@ -622,6 +666,7 @@ int64_t plan_bytes(int n, int order, double theta, int precision, int tile, int 
     b += al(8 * std::max<int64_t>(n_ops, 1));                      // log|tau|
     if (precision == PP_MIXED) b += al(8 * std::max<int64_t>(n_ops, 1)) + al(8 * nbox);  // pairs: log|tau|, S
     b += al(int64_t(sizeof(pp::M2LEntry)) * 4 * il_stride);        // interaction lists
+    if (precision == PP_MIXED) b += al(int64_t(sizeof(pp::M2LGroup)) * 4 * il_stride);  // grouped
     const auto nearl = near_offsets(theta);
     int Dmax = 0;
     for (auto& o : nearl) Dmax = std::max(Dmax, std::max(std::abs(o.first), std::abs(o.second)));

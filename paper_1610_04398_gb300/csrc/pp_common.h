@@ -36,6 +36,14 @@ struct M2LEntry {
     int dx, dy, op, pad;
 };
 
+// An item of the grouped interaction list (mixed plans): up to four sources at offsets i^j tau_0
+// (member j, -1 where the list has none; the same side ratio), op the operator of tau_0.  A
+// member packs its entry: dx + 128, dy + 128 (8 bits each), pad.
+struct M2LGroup {
+    int m[4];
+    int op, unused[3];
+};
+
 // Device-resident data of one plan, shared by all kernels of one precision.
 template <typename T>
 struct Tree {
@@ -68,6 +76,9 @@ struct Tree {
     const M2LEntry* il;    // [4][il_stride] interaction lists per child position
     int il_count[4];
     int il_stride;
+    const M2LGroup* ig;    // mixed plans: [4][il_stride] the same lists, sources at rotated offsets grouped;
+    int ig_groups[4];      // the groups of two to four first,
+    int ig_count[4];       // then the single sources
     const T* Ktab;         // [(2 Rk + 1)^2]: log max(h |Delta|, rho_h) for integer cell offsets
     const T* Krel;         // same offsets, log max(|Delta|, rho_h / h) = Ktab - log h (split solve: the
                            // log h part is added exactly from the near leaves' monopoles)
@@ -84,6 +95,34 @@ struct Tree {
     float2* Sf;                    // mixed plans: S per box as a double-float pair (hi, lo), else null
     const float2* lnTauF;          // mixed plans: log|tau| per operator as a double-float pair, else null
 };
+
+// The multipole coefficients of box b (row-major) of level l.  FP64 plans keep a box's coefficients
+// together.  Mixed plans keep a level's as planes over its boxes: coefficient 0, then pairs (1, 2),
+// (3, 4), ... of 16 bytes a box (a last unpaired one alone), so that a warp whose lanes take
+// neighbouring boxes reads and writes whole lines.  With a box's P1 coefficients together every
+// such access touched 26 lines, and the translations depended on all of them staying in L1, most of
+// which is shared memory while the near field runs beside them.  Pairs sit on 16 bytes for levels >= 1
+// (the array starts one element past a 16-byte boundary, and level_offset(l) P1 is odd there for odd P1).
+template <typename T>
+struct Multipole {
+    typedef typename cplx_of<T>::type C;
+    C* p;
+    int box, nb, P1;  // mixed: the box, the boxes of the level, the coefficients of a box
+    __device__ __forceinline__ C& operator[](int k) const {
+        if constexpr (sizeof(T) == 8) return p[k];
+        const int j = k - 1;
+        if (k == 0 || (k == P1 - 1 && !(j & 1))) return p[int64_t(nb) * k + box];  // a plane of its own
+        return p[int64_t(nb) * (1 + (j & ~1)) + 2 * box + (j & 1)];
+    }
+    // mixed plans, odd P1, levels >= 1: the pair (k, k + 1), k odd, as one 16-byte value
+    __device__ __forceinline__ float4* pair(int k) const {
+        return reinterpret_cast<float4*>(p + int64_t(nb) * k + 2 * box);
+    }
+};
+template <typename T>
+__device__ __forceinline__ Multipole<T> multipole(const Tree<T>& t, int l, int64_t b) {
+    return {t.mp + (sizeof(T) == 4 ? level_offset(l) * t.P1 : (level_offset(l) + b) * t.P1), int(b), 1 << (2 * l), t.P1};
+}
 
 // ------------------------------------------------------------------------------------
 // Double-float arithmetic: a value hi + lo held in two floats (|lo| <= ulp(hi) / 2), about

@@ -72,17 +72,19 @@ __device__ __forceinline__ void m2l_list(const Tree<T>& t, int l, int bx, int by
     for (int e = e0; e < cnt; e += stride) {
         const M2LEntry en = lst[e];
         int64_t src;
+        Multipole<T> M;
         if (en.pad == 0) {  // same-level source box
             const int sx = bx + en.dx, sy = by + en.dy;
             if (sx < 0 || sy < 0 || sx >= side || sy >= side) continue;
             src = off + int64_t(sy) * side + sx;
+            M = multipole(t, l, int64_t(sy) * side + sx);
         } else {  // parent-level source box standing for four separated children
             const int hs = side >> 1;
             const int sx = (bx >> 1) + en.dx, sy = (by >> 1) + en.dy;
             if (sx < 0 || sy < 0 || sx >= hs || sy >= hs) continue;
             src = level_offset(l - 1) + int64_t(sy) * hs + sx;
+            M = multipole(t, l - 1, int64_t(sy) * hs + sx);
         }
-        const C* M = t.mp + src * P1;
         const C* tp = t.Tpow + int64_t(en.op) * P1;
         const C* tl = t.TpowL + int64_t(en.op) * P1;
         const double Sd = t.S[src];
@@ -121,67 +123,188 @@ __device__ __forceinline__ void m2l_list(const Tree<T>& t, int l, int bx, int by
     }
 }
 
-// The same translations with the constant-term parts accumulated in double-float on the
-// FP32 pipe: (ah, al) = sum S log|tau|, (sh, sl) = sum S, from the pairs Sf and lnTauF.
+// Two-warp CTAs on 8 x 8 boxes: the 1366 of a 2048^2 grid put nine on every SM (683 of four warps put
+// five on some SMs and four on the others), and the sources of a square tile are half those of a row.
+constexpr int kFarThreads = 64;
+
+// The translations of k_m2l_far: items of the child position's grouped list, the constant-term
+// parts accumulated in double-float on the FP32 pipe, (ah, al) = sum S log|tau| and (sh, sl) =
+// sum S, from the pairs Sf and lnTauF.
+//
+// Sources whose offsets are 90 degree rotations of one another about the target's centre, tau_j =
+// i^j tau_0 (same side ratio), share one real product: with
+//   G_r[k] = sum_j i^(-j r) M_k of source j   (a 4-point transform: 16 additions),
+//   L_l += tau_0^-l sum_k R[l][k] (r / tau_0)^k G_(l+k)[k]   (index of G mod 4),
+// 748 FP32 operations for up to four sources at p = 12 in place of 412 each (1612 for 1168 at p = 20).
+// The lists hold 4 to 15 such groups of two to four sources; the flops of a list fall to 0.74 (p =
+// 12, theta 0.75) and 0.70 (p = 20, theta 0.5) of one product per source.
+// The sources of a column pair (k, k + 1) are one 16-byte load; for P1 > 13 the sums L sit in shared
+// memory (a column a thread, touched once an item), so the registers hold the pair's loads instead.
+// FP32-bound.  Alone, before (a product per source, a box's coefficients together) and now: 46.7 and
+// 45.7 us at 2048^2, p = 12, theta 0.75; 201 and 174 at p = 20, theta 0.5.  What the steps gain beside
+// the near field is more (4096^2 704 to 654 us): the loads no longer live off L1.
+struct M2LSource {
+    int base, nb;  // pair (k, k + 1), k odd, at mp[base + k nb]; base < 0: outside the grid
+    int box;       // flat box index (S arrays)
+};
+__device__ __forceinline__ M2LSource m2l_source(int packed, int P1, int l, int bx, int by) {
+    M2LSource s{-1, 0, 0};
+    if (packed < 0) return s;
+    const int lv = l - (packed >> 16);  // parent-level sources are one level up
+    const int side = 1 << lv;
+    const int sx = (bx >> (l - lv)) + (packed & 255) - 128, sy = (by >> (l - lv)) + ((packed >> 8) & 255) - 128;
+    if (sx < 0 || sy < 0 || sx >= side || sy >= side) return s;
+    const int off = int(level_offset(lv)), b = sy * side + sx;
+    s.base = off * P1 + 2 * b;
+    s.nb = 1 << (2 * lv);
+    s.box = off + b;
+    return s;
+}
+
+// The sums L of a thread: in registers, or (large orders) in its column of shared memory.
 template <int P1>
-__device__ __forceinline__ void m2l_list_df(const Tree<float>& t, int l, int bx, int by, int e0, int stride,
-                                            float (&Lr)[P1], float (&Li)[P1], float& ah, float& al, float& sh,
-                                            float& sl) {
-    typedef float2 C;
-    typedef float T;
-    const int side = 1 << l;
-    const int64_t off = level_offset(l);
+struct M2LSums {
+    static constexpr bool kShared = P1 > 13;
+    float2 reg[kShared ? 1 : P1];
+    float2 (*col)[kFarThreads];
+    __device__ __forceinline__ float2 get(int i) const { return kShared ? col[i][threadIdx.x] : reg[kShared ? 0 : i]; }
+    __device__ __forceinline__ void set(int i, float2 v) {
+        if (kShared) col[i][threadIdx.x] = v;
+        else reg[kShared ? 0 : i] = v;
+    }
+};
+
+template <int P1>
+__device__ __forceinline__ void m2l_finish(const float2* tl, const float (&yr)[P1], const float (&yi)[P1], M2LSums<P1>& L) {
+    const float2 v0 = L.get(0);
+    L.set(0, make_float2(v0.x + yr[0], 0.f));
+#pragma unroll
+    for (int ll = 1; ll < P1; ++ll) {
+        const float2 w = tl[ll], v = L.get(ll);
+        L.set(ll, make_float2(fma(yr[ll], w.x, fma(-yi[ll], w.y, v.x)), fma(yr[ll], w.y, fma(yi[ll], w.x, v.y))));
+    }
+}
+
+// kGroups: the grouped list; otherwise every source by itself (threads that share a box and its list:
+// groups would leave most of them idle).
+template <int P1, bool kGroups>
+__device__ __forceinline__ void m2l_items_df(const Tree<float>& t, int l, int bx, int by, int e0, int stride,
+                                             M2LSums<P1>& L, float& ah, float& al, float& sh, float& sl) {
+    static_assert(P1 % 2 == 1, "columns 1 .. P1 - 1 in pairs");
     const int par = (bx & 1) + 2 * (by & 1);
-    const int cnt = t.il_count[par];
-    const M2LEntry* lst = t.il + int64_t(par) * t.il_stride;
-    for (int e = e0; e < cnt; e += stride) {
-        const M2LEntry en = lst[e];
-        int64_t src;
-        if (en.pad == 0) {  // same-level source box
-            const int sx = bx + en.dx, sy = by + en.dy;
-            if (sx < 0 || sy < 0 || sx >= side || sy >= side) continue;
-            src = off + int64_t(sy) * side + sx;
-        } else {  // parent-level source box standing for four separated children
-            const int hs = side >> 1;
-            const int sx = (bx >> 1) + en.dx, sy = (by >> 1) + en.dy;
-            if (sx < 0 || sy < 0 || sx >= hs || sy >= hs) continue;
-            src = level_offset(l - 1) + int64_t(sy) * hs + sx;
+    const M2LGroup* lst = t.ig + int64_t(par) * t.il_stride;
+    const int ng = kGroups ? t.ig_groups[par] : 0, cnt = kGroups ? t.ig_count[par] : t.il_count[par];
+    if constexpr (kGroups) {
+#pragma unroll 1
+        for (int e = e0; e < ng; e += stride) {
+            const M2LGroup en = lst[e];
+            int base[4];
+            float s[4];
+            float gh = 0.f, gl = 0.f;  // sum of the group's S
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const M2LSource src = m2l_source(en.m[j], P1, l, bx, by);
+                base[j] = src.base;
+                const float2 S = src.base >= 0 ? t.Sf[src.box] : make_float2(0.f, 0.f);
+                s[j] = S.x;
+                df_add(gh, gl, S.x, S.y);
+            }
+            const int nb = 1 << (2 * (l - (en.m[0] >> 16)));  // of the members' level (member 0 is always there)
+            const float2* tp = t.Tpow + int64_t(en.op) * P1;
+            float yr[P1], yi[P1];
+            yr[0] = 0.f;
+            yi[0] = 0.f;
+            {
+                const float e2 = s[0] + s[2], f2 = s[1] + s[3], g2 = s[0] - s[2], h2 = s[1] - s[3];
+#pragma unroll
+                for (int ll = 1; ll < P1; ++ll) {
+                    const float c = c_ops.m2l[ll][0];
+                    yr[ll] = c * ((ll & 3) == 0 ? e2 + f2 : (ll & 3) == 2 ? e2 - f2 : g2);
+                    yi[ll] = (ll & 3) == 1 ? -c * h2 : (ll & 3) == 3 ? c * h2 : 0.f;
+                }
+            }
+#pragma unroll
+            for (int kp = 1; kp < P1; kp += 2) {
+                float4 m4[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    m4[j] = base[j] >= 0 ? *reinterpret_cast<const float4*>(t.mp + base[j] + kp * nb)
+                                         : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int k = kp + u;
+                    float2 m[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) m[j] = u ? make_float2(m4[j].z, m4[j].w) : make_float2(m4[j].x, m4[j].y);
+                    const float2 w = tp[k];
+                    const float2 ee = make_float2(m[0].x + m[2].x, m[0].y + m[2].y);
+                    const float2 ff = make_float2(m[1].x + m[3].x, m[1].y + m[3].y);
+                    const float2 gg = make_float2(m[0].x - m[2].x, m[0].y - m[2].y);
+                    const float2 hh = make_float2(m[1].x - m[3].x, m[1].y - m[3].y);
+                    const float2 G[4] = {make_float2(ee.x + ff.x, ee.y + ff.y), make_float2(gg.x + hh.y, gg.y - hh.x),
+                                         make_float2(ee.x - ff.x, ee.y - ff.y), make_float2(gg.x - hh.y, gg.y + hh.x)};
+                    float2 x[4];
+#pragma unroll
+                    for (int r = 0; r < 4; ++r)
+                        x[r] = make_float2(G[r].x * w.x - G[r].y * w.y, G[r].x * w.y + G[r].y * w.x);
+                    yr[0] = fma(c_ops.m2l[0][k], x[k & 3].x, yr[0]);
+#pragma unroll
+                    for (int ll = 1; ll < P1; ++ll) {
+                        yr[ll] = fma(c_ops.m2l[ll][k], x[(ll + k) & 3].x, yr[ll]);
+                        yi[ll] = fma(c_ops.m2l[ll][k], x[(ll + k) & 3].y, yi[ll]);
+                    }
+                }
+            }
+            m2l_finish<P1>(t.TpowL + int64_t(en.op) * P1, yr, yi, L);
+            const float2 lt = t.lnTauF[en.op];
+            df_fma(ah, al, gh, gl, lt.x, lt.y);
+            df_add(sh, sl, gh, gl);
         }
-        const C* M = t.mp + src * P1;
-        const C* tp = t.Tpow + int64_t(en.op) * P1;
-        const C* tl = t.TpowL + int64_t(en.op) * P1;
-        const float2 Sd = t.Sf[src];
-        const T St = Sd.x;
+    }
+#pragma unroll 1
+    for (int e = ng + e0; e < cnt; e += stride) {
+        int packed, op;
+        if constexpr (kGroups) {
+            packed = lst[e].m[0];
+            op = lst[e].op;
+        } else {
+            const M2LEntry en = t.il[int64_t(par) * t.il_stride + e];
+            packed = (en.dx + 128) | (en.dy + 128) << 8 | en.pad << 16;
+            op = en.op;
+        }
+        const M2LSource src = m2l_source(packed, P1, l, bx, by);
+        if (src.base < 0) continue;
+        const float2* tp = t.Tpow + int64_t(op) * P1;
+        const float2 Sd = t.Sf[src.box];
         // y = R x, accumulated column by column: 2 P1 - 1 independent FMA chains
-        T yr[P1], yi[P1];
-        yr[0] = T(0);
-        yi[0] = T(0);
+        float yr[P1], yi[P1];
+        yr[0] = 0.f;
+        yi[0] = 0.f;
 #pragma unroll
         for (int ll = 1; ll < P1; ++ll) {
-            yr[ll] = c_ops.m2l[ll][0] * St;
-            yi[ll] = T(0);
+            yr[ll] = c_ops.m2l[ll][0] * Sd.x;
+            yi[ll] = 0.f;
         }
 #pragma unroll
-        for (int k = 1; k < P1; ++k) {
-            const C m = M[k];
-            const C w = tp[k];
-            const T xr = m.x * w.x - m.y * w.y;
-            const T xi = m.x * w.y + m.y * w.x;
-            yr[0] = fma(c_ops.m2l[0][k], xr, yr[0]);
+        for (int kp = 1; kp < P1; kp += 2) {
+            const float4 m4 = *reinterpret_cast<const float4*>(t.mp + src.base + kp * src.nb);
 #pragma unroll
-            for (int ll = 1; ll < P1; ++ll) {
-                yr[ll] = fma(c_ops.m2l[ll][k], xr, yr[ll]);
-                yi[ll] = fma(c_ops.m2l[ll][k], xi, yi[ll]);
+            for (int u = 0; u < 2; ++u) {
+                const int k = kp + u;
+                const float2 m = u ? make_float2(m4.z, m4.w) : make_float2(m4.x, m4.y);
+                const float2 w = tp[k];
+                const float xr = m.x * w.x - m.y * w.y;
+                const float xi = m.x * w.y + m.y * w.x;
+                yr[0] = fma(c_ops.m2l[0][k], xr, yr[0]);
+#pragma unroll
+                for (int ll = 1; ll < P1; ++ll) {
+                    yr[ll] = fma(c_ops.m2l[ll][k], xr, yr[ll]);
+                    yi[ll] = fma(c_ops.m2l[ll][k], xi, yi[ll]);
+                }
             }
         }
-        Lr[0] += yr[0];
-#pragma unroll
-        for (int ll = 1; ll < P1; ++ll) {
-            const C w = tl[ll];
-            Lr[ll] = fma(yr[ll], w.x, fma(-yi[ll], w.y, Lr[ll]));
-            Li[ll] = fma(yr[ll], w.y, fma(yi[ll], w.x, Li[ll]));
-        }
-        const float2 lt = t.lnTauF[en.op];
+        m2l_finish<P1>(t.TpowL + int64_t(op) * P1, yr, yi, L);
+        const float2 lt = t.lnTauF[op];
         df_fma(ah, al, Sd.x, Sd.y, lt.x, lt.y);
         df_add(sh, sl, Sd.x, Sd.y);
     }
@@ -580,10 +703,10 @@ __global__ void __launch_bounds__(32 * kRhsWarps, (P1 <= 17 ? 16 : 8) / kRhsWarp
             if (act && !(lane & 1)) {
                 const int64_t box = level_offset(t.Lleaf) + int64_t(LY) * t.nL + (x0 >> 3);
                 store_S_leaf(t, box, ar[0]);
-                float2* M = t.mp + box * P1;
+                const Multipole<float> M = multipole(t, t.Lleaf, int64_t(LY) * t.nL + (x0 >> 3));
                 M[0] = make_float2(ar[0], 0.f);
 #pragma unroll
-                for (int k = 1; k < P1; ++k) M[k] = make_float2(ar[k], ai[k]);
+                for (int k = 1; k < P1; k += 2) *M.pair(k) = make_float4(ar[k], ai[k], ar[k + 1], ai[k + 1]);
             }
 #pragma unroll
             for (int k = 0; k < P1; ++k) {
@@ -788,8 +911,8 @@ __global__ void __launch_bounds__(128) k_m2l_chain(Tree<float> t, int lt, LevelL
 // its box and the 84 boxes below it.
 // ------------------------------------------------------------------------------------
 template <int P1>
-struct FarOcc {  // resident 128-thread CTAs per SM of k_m2l_far (register budget without spills)
-    static constexpr int value = P1 <= 13 ? 5 : P1 <= 17 ? 4 : 3;
+struct FarOcc {  // resident kFarThreads-thread CTAs per SM of k_m2l_far (register budget without spills)
+    static constexpr int value = P1 <= 13 ? 9 : P1 <= 21 ? 8 : 6;
 };
 constexpr int kDownAnc = 12;     // ancestor levels 2..lr-1 a CTA of k_down_tree can hold (L <= 17)
 constexpr int kDownSub = 85;     // boxes of a subtree: 1 + 4 + 16 + 64
@@ -808,8 +931,8 @@ constexpr int kDownRoom = 4096;
 // a0 + log(box side) sum S + Re part (lnRoot: log of the root box side); it and the coefficients go to loc/L0 for levels >= lr and
 // to the side buffers locA/L0A for the shared ancestor levels below lr, which k_down_tree
 // reads from every CTA while it writes the complete locals to loc/L0.
-template <int P1>
-__global__ void __launch_bounds__(128, FarOcc<P1>::value) k_m2l_far(Tree<float> t, int lr, int S, double lnRoot) {
+template <int P1, bool kGroups>
+__global__ void __launch_bounds__(kFarThreads, FarOcc<P1>::value) k_m2l_far(Tree<float> t, int lr, int S, double lnRoot) {
     const int64_t g = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     int64_t b = g / S;
     const int sub = int(g % S);
@@ -819,16 +942,29 @@ __global__ void __launch_bounds__(128, FarOcc<P1>::value) k_m2l_far(Tree<float> 
         --l;
     }
     const bool act = l >= 2;
+    int bx = 0, by = 0;
+    if (l >= 3) {  // tiles of 8 x 8 boxes
+        const int tiles = 1 << (l - 3), tile = int(b >> 6);
+        bx = (tile & (tiles - 1)) * 8 + int(b & 7);
+        by = (tile >> (l - 3)) * 8 + int((b >> 3) & 7);
+        b = (int64_t(by) << l) + bx;
+    } else if (act) {
+        bx = int(b & 3);
+        by = int(b >> 2);
+    }
+    __shared__ float2 Ls[M2LSums<P1>::kShared ? P1 : 1][kFarThreads];
+    M2LSums<P1> sums;
+    sums.col = Ls;
+#pragma unroll
+    for (int i = 0; i < P1; ++i) sums.set(i, make_float2(0.f, 0.f));
+    float ah = 0.f, al = 0.f, sh = 0.f, sl = 0.f;  // double-float sum S log|tau|, sum S
+    if (act) m2l_items_df<P1, kGroups>(t, l, bx, by, sub, S, sums, ah, al, sh, sl);
     float Lr[P1], Li[P1];
 #pragma unroll
     for (int i = 0; i < P1; ++i) {
-        Lr[i] = 0.f;
-        Li[i] = 0.f;
-    }
-    float ah = 0.f, al = 0.f, sh = 0.f, sl = 0.f;  // double-float sum S log|tau|, sum S
-    if (act) {
-        const int side = 1 << l;
-        m2l_list_df<P1>(t, l, int(b % side), int(b / side), sub, S, Lr, Li, ah, al, sh, sl);
+        const float2 v = sums.get(i);
+        Lr[i] = v.x;
+        Li[i] = v.y;
     }
     for (int o = 1; o < S; o <<= 1) {
 #pragma unroll
@@ -1087,8 +1223,8 @@ __device__ __forceinline__ float m2m_parent(const Tree<T>& t, int l, int64_t b, 
         const int bx = int(b % side), by = int(b / side);
         const int cs = 2 * side;
         for (int q = sub; q < 4; q += G) {
-            const int64_t child = coff + int64_t(2 * by + (q >> 1)) * cs + 2 * bx + (q & 1);
-            const C* M = t.mp + child * P1;
+            const int64_t cb = int64_t(2 * by + (q >> 1)) * cs + 2 * bx + (q & 1), child = coff + cb;
+            const Multipole<T> M = multipole(t, l + 1, cb);
             const C* zi = t.Ziq + q * P1;
             const C* z = t.Zq + q * P1;
             const double Sd = ld_child(t.S + child, kCg);
@@ -1101,17 +1237,23 @@ __device__ __forceinline__ float m2m_parent(const Tree<T>& t, int l, int64_t b, 
                 yr[k] = c_ops.m2m[k][0] * St;
                 yi[k] = T(0);
             }
+            static_assert(sizeof(T) == 4 && P1 % 2 == 1, "columns 1 .. P1 - 1 in pairs");
 #pragma unroll
-            for (int j = 1; j < P1; ++j) {
-                const C m = ld_child(M + j, kCg);
-                if constexpr (kMax) mx = fmaxf(mx, fmaxf(fabsf(float(m.x)), fabsf(float(m.y))));
-                const C w = zi[j];
-                const T wr = m.x * w.x - m.y * w.y;
-                const T wi = m.x * w.y + m.y * w.x;
+            for (int jp = 1; jp < P1; jp += 2) {
+                const float4 m4 = kCg ? __ldcg(M.pair(jp)) : *M.pair(jp);
 #pragma unroll
-                for (int k = j; k < P1; ++k) {
-                    yr[k] = fma(c_ops.m2m[k][j], wr, yr[k]);
-                    yi[k] = fma(c_ops.m2m[k][j], wi, yi[k]);
+                for (int u = 0; u < 2; ++u) {
+                    const int j = jp + u;
+                    const C m = u ? cmake<T>(m4.z, m4.w) : cmake<T>(m4.x, m4.y);
+                    if constexpr (kMax) mx = fmaxf(mx, fmaxf(fabsf(float(m.x)), fabsf(float(m.y))));
+                    const C w = zi[j];
+                    const T wr = m.x * w.x - m.y * w.y;
+                    const T wi = m.x * w.y + m.y * w.x;
+#pragma unroll
+                    for (int k = j; k < P1; ++k) {
+                        yr[k] = fma(c_ops.m2m[k][j], wr, yr[k]);
+                        yi[k] = fma(c_ops.m2m[k][j], wi, yi[k]);
+                    }
                 }
             }
 #pragma unroll
@@ -1131,14 +1273,20 @@ __device__ __forceinline__ float m2m_parent(const Tree<T>& t, int l, int64_t b, 
         S += __shfl_xor_sync(0xffffffffu, S, o);
     }
     if (act && sub == 0) {
-        C* out = t.mp + (poff + b) * P1;
+        const Multipole<T> out = multipole(t, l, b);
         store_S(t, poff + b, S);
         out[0] = cmake<T>(T(S), T(0));
         if constexpr (kMax) mx = fmaxf(mx, fabsf(float(S)));
 #pragma unroll
-        for (int k = 1; k < P1; ++k) {
-            out[k] = cmake<T>(Br[k], Bi[k]);
-            if constexpr (kMax) mx = fmaxf(mx, fmaxf(fabsf(float(Br[k])), fabsf(float(Bi[k]))));
+        for (int k = 1; k < P1; k += 2) {
+            const float4 v = make_float4(Br[k], Bi[k], Br[k + 1], Bi[k + 1]);
+            if (l > 0) {
+                *out.pair(k) = v;
+            } else {  // the root's pairs are not aligned
+                out[k] = cmake<T>(v.x, v.y);
+                out[k + 1] = cmake<T>(v.z, v.w);
+            }
+            if constexpr (kMax) mx = fmaxf(mx, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
         }
     }
     return mx;

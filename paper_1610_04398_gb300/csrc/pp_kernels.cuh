@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(256) k_p2m(Tree<T> t) {
     if (act && row == 0) {
         // FP64 monopole of the leaf (sum of the eight FP32/FP64 row sums)
         store_S_leaf(t, off + leaf, s0);
-        t.mp[(off + leaf) * P1] = cmake<T>(s0, T(0));
+        multipole(t, t.Lleaf, leaf)[0] = cmake<T>(s0, T(0));
     }
     for (int k = 1; k < P1; ++k) {
         T ar = T(0), ai = T(0);
@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(256) k_p2m(Tree<T> t) {
         }
         if (act && row == (k & 7)) {
             const T ik = T(1) / T(k);
-            t.mp[(off + leaf) * P1 + k] = cmake<T>(ar * ik, ai * ik);
+            multipole(t, t.Lleaf, leaf)[k] = cmake<T>(ar * ik, ai * ik);
         }
     }
 }
@@ -211,11 +211,11 @@ __global__ void __launch_bounds__(256) k_p2m_reg(Tree<T> t) {
             ai[k] += __shfl_xor_sync(0xffffffffu, ai[k], o);
         }
     if (!act) return;
-    const int64_t base = (level_offset(t.Lleaf) + leaf) * P1;
+    const auto M = multipole(t, t.Lleaf, leaf);
     if (row == 0) store_S_leaf(t, level_offset(t.Lleaf) + leaf, ar[0]);
 #pragma unroll
     for (int k = 0; k < P1; ++k)
-        if ((k & 7) == row) t.mp[base + k] = k == 0 ? cmake<T>(ar[0], T(0)) : cmake<T>(ar[k] / T(k), ai[k] / T(k));
+        if ((k & 7) == row) M[k] = k == 0 ? cmake<T>(ar[0], T(0)) : cmake<T>(ar[k] / T(k), ai[k] / T(k));
 }
 
 // ------------------------------------------------------------------------------------
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(128) k_m2m(Tree<T> t, int l) {
     for (int idx = lane; idx < 4 * P1; idx += 32) {
         const int q = idx / P1, k = idx % P1;
         const int64_t child = int64_t(2 * by + (q >> 1)) * cs + 2 * bx + (q & 1);
-        cb[idx] = t.mp[(coff + child) * P1 + k];
+        cb[idx] = multipole(t, l + 1, child)[k];
     }
     __syncwarp();
     for (int k = 1 + lane; k < P1; k += 32) {
@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(128) k_m2m(Tree<T> t, int l) {
             const C* A = t.Am2m + int64_t(q) * P1 * P1;
             for (int j = 0; j <= k; ++j) cfma(acc, A[j * P1 + k], cb[q * P1 + j]);
         }
-        t.mp[(poff + b) * P1 + k] = acc;
+        multipole(t, l, b)[k] = acc;
     }
     if (lane == 0) {
         double S = 0.0;
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(128) k_m2m(Tree<T> t, int l) {
             S += t.S[coff + child];
         }
         store_S(t, poff + b, S);
-        t.mp[(poff + b) * P1] = cmake<T>(T(S), T(0));
+        multipole(t, l, b)[0] = cmake<T>(T(S), T(0));
     }
 }
 
@@ -302,18 +302,21 @@ __global__ void __launch_bounds__(128) k_m2l(Tree<T> t, int l) {
     for (int e = 0; e < cnt; ++e) {
         const M2LEntry en = lst[e];
         int64_t src;
+        Multipole<T> M;
         if (en.pad == 0) {
             const int sx = bx + en.dx, sy = by + en.dy;
             if (sx < 0 || sy < 0 || sx >= side || sy >= side) continue;
             src = off + int64_t(sy) * side + sx;
+            M = multipole(t, l, int64_t(sy) * side + sx);
         } else {
             const int hs = side >> 1;
             const int sx = (bx >> 1) + en.dx, sy = (by >> 1) + en.dy;
             if (sx < 0 || sy < 0 || sx >= hs || sy >= hs) continue;
             src = level_offset(l - 1) + int64_t(sy) * hs + sx;
+            M = multipole(t, l - 1, int64_t(sy) * hs + sx);
         }
         __syncwarp();
-        for (int k = lane; k < P1; k += 32) sb[k] = t.mp[src * P1 + k];
+        for (int k = lane; k < P1; k += 32) sb[k] = M[k];
         __syncwarp();
         const C* B = t.Bm2l + int64_t(en.op) * P1 * P1;
         for (int r = 0; r < 2; ++r) {
@@ -536,7 +539,7 @@ __global__ void k_export(Tree<T> t, int kind, int level, double* dst) {
         const int k = int(idx % t.P1);
         double re, im;
         if (kind == 0) {
-            const typename cplx_of<T>::type c = t.mp[(off + b) * t.P1 + k];
+            const typename cplx_of<T>::type c = multipole(t, level, b)[k];
             re = (k == 0) ? t.S[off + b] : double(c.x);
             im = (k == 0) ? 0.0 : double(c.y);
         } else {
@@ -789,11 +792,14 @@ cudaError_t launch_m2l_far(const Tree<T>& t, cudaStream_t st) {
         switch (t.P1) {
 #define PP_CASE(P)                                                                      \
     case P: {                                                                           \
-        const int64_t slots = t.resident_threads / 384 * 128 * FarOcc<P>::value;        \
+        const int64_t slots = t.resident_threads / 384 * kFarThreads * FarOcc<P>::value; \
         int S = 1;                                                                      \
         while (S < 32 && 4 * boxes * S < 3 * slots) S <<= 1;                            \
-        const unsigned blocks = unsigned((boxes * S + 127) / 128);                      \
-        k_m2l_far<P><<<blocks, 128, 0, st>>>(tf, t.Lleaf - 3, S, lnRoot);               \
+        const unsigned blocks = unsigned((boxes * S + kFarThreads - 1) / kFarThreads);  \
+        if (S == 1)                                                                     \
+            k_m2l_far<P, true><<<blocks, kFarThreads, 0, st>>>(tf, t.Lleaf - 3, S, lnRoot); \
+        else                                                                            \
+            k_m2l_far<P, false><<<blocks, kFarThreads, 0, st>>>(tf, t.Lleaf - 3, S, lnRoot); \
         return cudaGetLastError();                                                      \
     }
             PP_FAST_ORDERS(PP_CASE)

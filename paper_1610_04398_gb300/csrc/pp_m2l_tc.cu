@@ -360,8 +360,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 if (slane && q < G::NREC) {
                     int64_t box = 0;
                     const bool in = record_box<MG>(T, r, q % G::HX, q / G::HX, box);
-                    const float2* m = t.mp + box * kP1 + kk;
-                    const float2* second = kk + 1 < kP1 ? m + 1 : t.Sf + box;
+                    const int bl = r < 4 ? T.l : T.l - 1;
+                    const Multipole<float> M = multipole(t, bl, in ? box - level_offset(bl) : 0);
+                    const float2* m = &M[kk];
+                    const float2* second = kk + 1 < kP1 ? &M[kk + 1] : t.Sf + box;
                     uint8_t* d = sb + (uint32_t(kRecPerStep * s + rl) * (kP1 + 1) + uint32_t(kk)) * 8u;
                     cp_async8z(d, in ? m : t.Sf, in);
                     cp_async8z(d + 8, in ? second : t.Sf, in);
