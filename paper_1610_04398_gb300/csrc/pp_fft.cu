@@ -9,7 +9,7 @@
 //
 // Three launches per solve, every line transform held whole in shared memory:
 //   1. rows: two real rows packed as one complex line (a + i b), forward transform, the half
-//      spectra of both rows untangled from Z(k) and Z(M - k) and stored, k in [0, M/2];
+//      spectra of both rows untangled from Z(k) and Z(M - k) and stored as pairs, k in [0, M/2];
 //   2. columns: each column k_x of the half spectrum (n values, zero padded to M) forward
 //      transformed, multiplied by the real transformed kernel, inverse transformed, and its
 //      first n values stored back in place;
@@ -283,8 +283,14 @@ __device__ __forceinline__ void fft_middle_group(C* line, const R* __restrict__ 
     for (int j = 0; j < RR; ++j) line[p0 + j] = v[j];
 }
 
+// The half spectra lie as pairs of rows: H[y / 2][k_x] holds (row y, row y + 1) side by side, 16 or
+// 32 bytes.  A row kernel's thread moves a pair in one access, and the column kernel, which was bound
+// by the 4096 lines a column's 8-byte loads and stores touched (one L1 lookup each, a quarter of
+// every 32-byte sector used), touches half as many per column, shared by two columns: 65.4 to 56 us a
+// launch at n = 2048, FP32 (139 to 137 a step with two columns a CTA).  What bounds it now: half the
+// issue slots, half the shared-memory pipe, and the barriers between the phases that use them.
 template <typename C>
-struct CPair {
+struct alignas(16) CPair {
     C a, b;
 };
 
@@ -308,7 +314,7 @@ __device__ __forceinline__ void batched_copy(int total, Load load, Store store) 
 
 // Launch 1.  CTA b transforms rows 2 NL b .. 2 NL b + 2 NL - 1 of q (leaf-major: cell (x, y)
 // at ((y/8) nL + x/8) 64 + (y mod 8) 8 + x mod 8) and writes their half spectra, k in
-// [0, M/2], to rows of H (row stride W; columns M/2 + 1 .. W - 1 are set to zero).
+// [0, M/2], to H (W pairs per two rows; columns M/2 + 1 .. W - 1 are set to zero).
 template <typename R, int NL>
 __global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 ? 3 : 1)
     k_fft_rows_fwd(const R* __restrict__ q, int n, int nL, int M, int m, int W, int ls,
@@ -342,9 +348,7 @@ __global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 ? 3 : 1)
             A = C{R(0.5) * (zk.x + zm.x), R(0.5) * (zk.y - zm.y)};
             B = C{R(0.5) * (zk.y + zm.y), R(0.5) * (zm.x - zk.x)};
         }
-        C* h0 = H + int64_t(y0 + 2 * l) * W + k;
-        h0[0] = A;
-        h0[W] = B;
+        reinterpret_cast<CPair<C>*>(H)[int64_t((y0 >> 1) + l) * W + k] = CPair<C>{A, B};
     }
 }
 
@@ -363,9 +367,14 @@ __global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 ? 3 : 1)
     const int ns = fft_nsteps(m);
     if (ns == 1)  // the single step reads the zero padding y in [n, M)
         for (int i = threadIdx.x; i < NL * n; i += blockDim.x) lines[(i % NL) * ls + fpad(n + i / NL)] = C{0, 0};
-    batched_copy<8>(
-        NL * n, [&](int i) { return H[int64_t(i / NL) * W + kx0 + i % NL]; },
-        [&](int i, C v) { lines[(i % NL) * ls + fpad(i / NL)] = v; });
+    CPair<C>* Hp = reinterpret_cast<CPair<C>*>(H) + kx0;
+    batched_copy<4>(
+        NL * (n >> 1), [&](int i) { return Hp[int64_t(i / NL) * W + i % NL]; },
+        [&](int i, CPair<C> v) {
+            C* x = lines + (i % NL) * ls + fpad(2 * (i / NL));  // no pad slot between 2 j and 2 j + 1
+            x[0] = v.a;
+            x[1] = v.b;
+        });
     __syncthreads();
     // forward steps but the last (the first one skips the zero half)
     if (ns > 1) {
@@ -394,9 +403,10 @@ __global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 ? 3 : 1)
     if (ns == 1) {
         // nothing left: the middle was the whole transform
     }
-    for (int i = threadIdx.x; i < NL * n; i += blockDim.x) {
-        const int y = i / NL, l = i - y * NL;
-        if (kx0 + l <= half) H[int64_t(y) * W + kx0 + l] = lines[l * ls + fpad(y)];
+    for (int i = threadIdx.x; i < NL * (n >> 1); i += blockDim.x) {
+        const int j = i / NL, l = i - j * NL;
+        const C* x = lines + l * ls + fpad(2 * j);
+        if (kx0 + l <= half) Hp[int64_t(j) * W + l] = CPair<C>{x[0], x[1]};
     }
 }
 
@@ -416,8 +426,7 @@ __global__ void __launch_bounds__(kFftThreads, sizeof(R) == 4 ? 3 : 1)
         NL * nk,
         [&](int i) {
             const int l = i / nk, k = i - l * nk;
-            const C* h0 = H + int64_t(y0 + 2 * l) * W + k;
-            return CPair<C>{h0[0], h0[W]};
+            return reinterpret_cast<const CPair<C>*>(H)[int64_t((y0 >> 1) + l) * W + k];
         },
         [&](int i, CPair<C> ab) {
             const int l = i / nk, k = i - l * nk;
@@ -521,16 +530,22 @@ int log2i(int M) {
 // lines a CTA interleaves in its column loads and stores fall in different bank halves.
 int line_stride(int M) { return M + M / 16 + M / 256 + 8; }
 
-// Lines per CTA (three CTAs per SM either way in FP32): two up to M = 2048, one above, where
-// the finer grain balances the waves better (2n = 4096: 0.116 against 0.122 ms a solve).
+// Lines per CTA (three CTAs per SM either way in FP32).  Rows: two up to M = 2048, one above, where
+// the finer grain balances the waves better (M = 4096: 0.116 against 0.122 ms a solve).  Columns: two
+// as long as three CTAs of two lines fit an SM, since two neighbouring columns fill the 32-byte
+// sectors of H (M = 4096: step 137.0 against 139.2 us with one).
 template <typename R>
 int lines_per_cta(int M) {
     return sizeof(R) == 4 && M <= 2048 ? 2 : 1;
 }
+template <typename R>
+int cols_per_cta(int M) {
+    return sizeof(R) == 4 && M <= 4096 ? 2 : 1;
+}
 
 template <typename R>
-size_t fft_smem(int M) {
-    return size_t(lines_per_cta<R>(M)) * size_t(line_stride(M)) * sizeof(typename Cplx<R>::type);
+size_t fft_smem(int M, int lines) {
+    return size_t(lines) * size_t(line_stride(M)) * sizeof(typename Cplx<R>::type);
 }
 
 int twiddle_entries(int M, int m) {
@@ -561,7 +576,7 @@ cudaError_t set_smem_attrs() {
 bool fft_size_ok(int n, bool fp64) {
     if (n < 8 || n > 4096 || (n & (n - 1))) return false;
     const int M = 2 * n;
-    return (fp64 ? fft_smem<double>(M) : fft_smem<float>(M)) <= size_t(kFftSmemLimit) &&
+    return (fp64 ? fft_smem<double>(M, 1) : fft_smem<float>(M, cols_per_cta<float>(M))) <= size_t(kFftSmemLimit) &&
            size_t(M) * 16 <= size_t(kFftSmemLimit);  // one FP64 line of the spectrum transform
 }
 
@@ -617,16 +632,16 @@ cudaError_t fft_prepare_spectrum(int n, double h, double rh, bool fp64, void* Kp
 
 // One solve: q (leaf-major weights f h^2) -> p_out (row-major n x n).  H: fft_work_bytes;
 // Kp: the spectrum buffer fft_prepare_spectrum formed.
-template <typename R, int NL>
+template <typename R, int NL, int NC>
 cudaError_t launch_fft_lines(const R* q, int n, int nL, const void* Kp, void* H, R* p_out, cudaStream_t st) {
     typedef typename Cplx<R>::type C;
     const int M = 2 * n, m = log2i(M), W = n + 4, ls = line_stride(M);
-    const size_t sm = fft_smem<R>(M);
+    const size_t sm = fft_smem<R>(M, NL), smc = fft_smem<R>(M, NC);
     const R* K = static_cast<const R*>(Kp);
     const C* tab = reinterpret_cast<const C*>(static_cast<const unsigned char*>(Kp) + kp_bytes(M, sizeof(R)));
     C* Hc = static_cast<C*>(H);
     k_fft_rows_fwd<R, NL><<<n / (2 * NL), kFftThreads, sm, st>>>(q, n, nL, M, m, W, ls, tab, Hc);
-    k_fft_cols<R, NL><<<(M / 2 + NL) / NL, kFftThreads, sm, st>>>(Hc, K, n, M, m, W, ls, tab);
+    k_fft_cols<R, NC><<<(M / 2 + NC) / NC, kFftThreads, smc, st>>>(Hc, K, n, M, m, W, ls, tab);
     k_fft_rows_inv<R, NL><<<n / (2 * NL), kFftThreads, sm, st>>>(Hc, n, M, m, W, ls, tab, p_out);
     return cudaGetLastError();
 }
@@ -634,9 +649,10 @@ cudaError_t launch_fft_lines(const R* q, int n, int nL, const void* Kp, void* H,
 template <typename R>
 cudaError_t launch_fft_solve(const R* q, int n, int nL, const void* Kp, void* H, R* p_out, cudaStream_t st) {
     if constexpr (sizeof(R) == 4) {
-        if (lines_per_cta<R>(2 * n) == 2) return launch_fft_lines<R, 2>(q, n, nL, Kp, H, p_out, st);
+        if (lines_per_cta<R>(2 * n) == 2) return launch_fft_lines<R, 2, 2>(q, n, nL, Kp, H, p_out, st);
+        if (cols_per_cta<R>(2 * n) == 2) return launch_fft_lines<R, 1, 2>(q, n, nL, Kp, H, p_out, st);
     }
-    return launch_fft_lines<R, 1>(q, n, nL, Kp, H, p_out, st);
+    return launch_fft_lines<R, 1, 1>(q, n, nL, Kp, H, p_out, st);
 }
 
 template cudaError_t launch_fft_solve<float>(const float*, int, int, const void*, void*, float*, cudaStream_t);
