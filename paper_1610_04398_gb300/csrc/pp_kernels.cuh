@@ -937,24 +937,34 @@ cudaError_t launch_leaf_eval(const Tree<T>& t, T* p_out, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t launch_surface(const Tree<T>& t, const T* u, const T* v, const SurfaceArgs& a,
-                           cudaStream_t st) {
-    constexpr int kWarps = SurfCta<T>::warps, kThreads = SurfCta<T>::threads;
-    constexpr size_t smem = surf_smem_bytes<T>();
+template <typename T, bool kMany>
+cudaError_t launch_surface_form(const Tree<T>& t, const T* u, const T* v, const SurfaceArgs& a, cudaStream_t st) {
+    constexpr int kWarps = SurfCta<T, kMany>::warps, kThreads = SurfCta<T, kMany>::threads;
+    constexpr size_t smem = sizeof(SurfWalk) * kWarps;
     const unsigned chunks = unsigned((a.npts + kWarps - 1) / kWarps);
     const unsigned nb = chunks < kSurfMaxCtas ? chunks : kSurfMaxCtas;
     if constexpr (sizeof(T) == 4) {
         switch (t.P1) {
 #define PP_CASE(P) \
-    case P: k_surface<T, P><<<nb, kThreads, smem, st>>>(t, u, v, a); return cudaGetLastError();
+    case P: k_surface<T, P, kMany><<<nb, kThreads, smem, st>>>(t, u, v, a); return cudaGetLastError();
             PP_FAST_ORDERS(PP_CASE)
 #undef PP_CASE
             default: break;
         }
     }
-    k_surface<T, 0><<<nb, kThreads, smem, st>>>(t, u, v, a);
+    k_surface<T, 0, kMany><<<nb, kThreads, smem, st>>>(t, u, v, a);
     return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_surface(const Tree<T>& t, const T* u, const T* v, const SurfaceArgs& a,
+                           cudaStream_t st) {
+    if constexpr (sizeof(T) == 4) {
+        // more points than one wave of the 8-point CTAs (resident_threads counts 384 per SM)
+        if (a.npts > t.resident_threads / 384 * SurfCta<T>::ctas * SurfCta<T>::warps)
+            return launch_surface_form<T, true>(t, u, v, a, st);
+    }
+    return launch_surface_form<T, false>(t, u, v, a, st);
 }
 
 // Opt every kernel with dynamic shared memory into the same generous limit, once per
@@ -969,11 +979,14 @@ cudaError_t prepare_kernels() {
         return e;
     if ((e = cudaFuncSetAttribute(k_leaf<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) != cudaSuccess)
         return e;
-    if ((e = cudaFuncSetAttribute(k_surface<T, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) != cudaSuccess)
+    if ((e = cudaFuncSetAttribute(k_surface<T, 0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) != cudaSuccess)
         return e;
     if constexpr (sizeof(T) == 4) {
-        const void* fns[] = {(const void*)k_surface<T, 13>, (const void*)k_surface<T, 17>,
-                             (const void*)k_surface<T, 21>, (const void*)k_surface<T, 25>,
+        const void* fns[] = {(const void*)k_surface<T, 13, false>, (const void*)k_surface<T, 17, false>,
+                             (const void*)k_surface<T, 21, false>, (const void*)k_surface<T, 25, false>,
+                             (const void*)k_surface<T, 13, true>, (const void*)k_surface<T, 17, true>,
+                             (const void*)k_surface<T, 21, true>, (const void*)k_surface<T, 25, true>,
+                             (const void*)k_surface<T, 0, true>,
                              (const void*)k_leaf_fast<1, true>, (const void*)k_leaf_fast<2, true>,
                              (const void*)k_leaf_fast<3, true>, (const void*)k_leaf_fast<1, false>,
                              (const void*)k_leaf_fast<2, false>, (const void*)k_leaf_fast<3, false>,

@@ -11,9 +11,14 @@ namespace pp {
 // Points a CTA walks at once, a warp each; one more warp forms their tractions, a lane each.  The
 // FP64 walk is bound by its SM's FP64 pipe: few points a CTA, so that few points still spread over
 // the SMs.  The mixed walk has no FP64: as many points as fill the traction warp's instructions.
-template <typename T>
+// kMany (mixed, more points than one wave of the other form holds, 24 an SM): 64 registers instead
+// of 72, so that an SM holds 28 points.  The 4096 points of a 256^2 step were 1.12 waves and every
+// warp's chain ran twice: 25.9 us, now 22.7 (in the step, 51.1 to 47.2).  Up to one wave the 72 registers
+// are better: 2048 points at 2048^2 take 21.0 against 22.0 us (146.0 against 147.4 in the step).
+template <typename T, bool kMany = false>
 struct SurfCta {
-    static constexpr int warps = sizeof(T) == 8 ? 4 : 8;
+    static constexpr int warps = sizeof(T) == 8 ? 4 : kMany ? 7 : 8;
+    static constexpr int ctas = kMany ? 4 : 3;  // per SM
     static constexpr int threads = 32 * (warps + 1);
 };
 constexpr int kSurfCap = 256;         // candidates of a level; accepted boxes a warp holds at once (FP64)
@@ -272,11 +277,11 @@ __device__ __forceinline__ void cell_grad(const T* u, const T* v, int n, double 
 // lifted point, the dS), then the tractions and their sums.  The CTA that finishes last (a counter it
 // resets; no CTA waits) adds the CTAs' sums in a fixed order and forms drag and lift.  Before, the
 // walk, the tractions (8.5 us, a chain of FP64 latencies) and the final sum (4.8 us) ran one after the
-// other: 39 us for 2048 points at 2048^2, p = 12, theta 0.5, 20 now (4096 points: 37, 24 now).
-template <typename T, int P1T>
-__global__ void __launch_bounds__(SurfCta<T>::threads, 3)
+// other: 39 us for 2048 points at 2048^2, p = 12, theta 0.5, 21 now (4096 points at 256^2: 37, 23 now).
+template <typename T, int P1T, bool kMany>
+__global__ void __launch_bounds__((SurfCta<T, kMany>::threads), (SurfCta<T, kMany>::ctas))
 k_surface(Tree<T> t, const T* __restrict__ u, const T* __restrict__ v, SurfaceArgs a) {
-    constexpr int kWarps = SurfCta<T>::warps, kThreads = SurfCta<T>::threads;
+    constexpr int kWarps = SurfCta<T, kMany>::warps, kThreads = SurfCta<T, kMany>::threads;
     extern __shared__ __align__(16) unsigned char surf_smem[];
     SurfWalk* walk = reinterpret_cast<SurfWalk*>(surf_smem);  // [kWarps]
     __shared__ SurfPoint pts[kWarps];
@@ -381,9 +386,10 @@ k_surface(Tree<T> t, const T* __restrict__ u, const T* __restrict__ v, SurfaceAr
     }
     // the CTA's partial sums (the traction warp's lanes), kept in the plan's surface scratch
     if (warp == kWarps) {
+        static_assert(kWarps <= 8, "points of a CTA in lanes 0 .. 7");
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-            for (int o = kWarps / 2; o > 0; o >>= 1) sum[k] += __shfl_xor_sync(0xffffffffu, sum[k], o);
+            for (int o = 4; o > 0; o >>= 1) sum[k] += __shfl_xor_sync(0xffffffffu, sum[k], o);
         if (lane == 0) {
             for (int k = 0; k < 4; ++k) a.Psurf[4 * int64_t(blockIdx.x) + k] = sum[k];
             __threadfence();
@@ -416,8 +422,5 @@ k_surface(Tree<T> t, const T* __restrict__ u, const T* __restrict__ v, SurfaceAr
         *a.counter = 0u;
     }
 }
-
-template <typename T>
-constexpr size_t surf_smem_bytes() { return sizeof(SurfWalk) * SurfCta<T>::warps; }
 
 }  // namespace pp

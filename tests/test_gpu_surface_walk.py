@@ -50,3 +50,23 @@ def test_surface_pressure_and_forces(precision, npts, theta_s):
     F = 0.01 * per[:, 1:].sum(0)
     assert np.allclose(forces.cpu().numpy()[:4], F, rtol=1e-9, atol=1e-9 * np.abs(0.01 * per[:, 1:]).sum())
     plan.destroy()
+
+
+@pytest.mark.parametrize("order", [10, 12, 16, 20, 24])
+def test_more_points_than_one_wave(order):
+    """The form for more points than a wave holds (from 3649 on 152 SMs) against the other on the
+    first points: the same FP32 operations, so rounding of the contracted ones at most (1e-6)."""
+    npts = 24 * torch.cuda.get_device_properties(0).multi_processor_count + 1
+    snap = synth.cylinder_flow(128, diameter=0.3, centre=(0.5, 0.5), n_surface=npts, seed=order)
+    plan = api.Plan(128, snap.h, order, 0.6, precision="mixed", lift=snap.lift)
+    f = [to_dev(a, plan.dtype) for a in (snap.u, snap.v, snap.chi, snap.usx, snap.usy)]
+    plan.rhs(*f, snap.lam)
+    out = []
+    for m in (npts, npts - 1):
+        per = torch.full((m * 5,), float("nan"), dtype=torch.float64, device="cuda")
+        plan.surface_traction(f[0], f[1], to_dev(snap.points[:m], torch.float64), to_dev(snap.normals[:m], torch.float64),
+                              snap.nu, per_point=per)
+        out.append(per.view(m, 5).cpu().numpy())
+    assert np.isfinite(out[0]).all()
+    assert rel_l2(out[0][:-1], out[1]) < 1e-6
+    plan.destroy()
