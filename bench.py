@@ -210,7 +210,8 @@ def alu_peak(precision, n_sm, local=0):
 
 # The sources that build and launch each kernel a traffic record covers (its header, the
 # translation units that instantiate it, the C ABI that sizes its launches).
-_STEP_SOURCES = ("pp_common.h", "pp_kernels.cuh", "pp_fast.cuh", "pp_kernels_f32.cu", "pp_kernels_f64.cu",
+_STEP_SOURCES = ("pp_common.h", "pp_kernels.cuh", "pp_fast.cuh", "pp_fp64.cuh", "pp_fixed.cuh",
+                 "pp_log.cuh", "pp_surface.cuh", "pp_kernels_f32.cu", "pp_kernels_f64.cu",
                  "pp_tc.cu", "pp_tcgen05.cuh", "pp_capi.cu")
 KERNEL_SOURCES = {"k_m2l_reg": _STEP_SOURCES, "k_m2l_far": _STEP_SOURCES, "k_m2l_tc": _STEP_SOURCES + ("pp_m2l_tc.cu",),
                   "k_near_tc": _STEP_SOURCES,
@@ -268,7 +269,7 @@ def stage_work(info, n, P1, prec_bytes, fused_leaf):
     near = info.near_pairs * 2.0          # one FMA per source/target pair
     m2l = info.m2l_pairs * m2l_flops(P1)
     l2l = (nbox - 21) * shift_flops(P1)   # one shift into every box of levels 3..L
-    two = fused_leaf and getattr(info, "downward", 0) >= 2
+    two = fused_leaf and (prec_bytes == 8 or getattr(info, "downward", 0) >= 2)  # FP64: k_m2l64, then k_down64
     return {
         # RHS: read u, v, chi, us_x, us_y, write q (plan precision)
         "rhs_p2m": ("hbm", 6.0 * n * n * prec_bytes),
@@ -403,7 +404,8 @@ def run_ours(a):
     # the roofline is reported for the longest stage whose algorithmic work is defined
     # (the surface stage is a latency-bound tree walk with no such figure)
     dom = max((k for k in stages if stages[k]["ms"] and work[k][1]), key=lambda k: stages[k]["ms"])
-    near_name = {128: "k_near_tc", 16: "k_near16", 8: "k_leaf_fast"}.get(info.near_kernel, "k_leaf")
+    f64 = a.precision == "fp64" and a.order <= 23 and info.levels > 2  # the fixed-point kernels
+    near_name = {128: "k_near_tc", 16: "k_near16", 8: "k_leaf_fast"}.get(info.near_kernel, "k_near64" if f64 else "k_leaf")
     if info.near_kernel == 128 and stages["leaf"]["ms"]:
         # the near field is a dense contraction on the tensor cores (kind::f16, FP32
         # accumulate): its roofline is the dense FP16 tensor peak, which is the measured
@@ -415,9 +417,10 @@ def run_ours(a):
         e["frac"] = e["achieved_tflops"] / e["peak_tflops"]
     two = fused and info.downward >= 2
     far = "k_m2l_tc" if info.downward == 3 else "k_m2l_far"
-    kern = {"leaf": near_name if fused else "k_leaf", "downward": far if two else "k_m2l_reg",
-            "rhs_p2m": "k_rhs_p2m_fast", "upward": "k_up_tree" if a.precision == "mixed" else "k_m2m_reg",
-            "leaf_m2l": "k_down_tree" if two else "k_l2p_leaf", "surface": "k_treecode"}[dom]
+    kern = {"leaf": near_name if fused else "k_leaf", "downward": far if two else "k_m2l64" if f64 else "k_m2l_reg",
+            "rhs_p2m": "k_rhs64" if f64 else "k_rhs_p2m_fast",
+            "upward": "k_up_tree" if a.precision == "mixed" else "k_up64" if f64 else "k_m2m_reg",
+            "leaf_m2l": "k_down_tree" if two else "k_down64" if f64 else "k_l2p_leaf", "surface": "k_surface"}[dom]
     d = stages[dom]
     if d["bound"] == "tensor":
         roof = {"bound": "tensor", "achieved": d["achieved_tflops"], "peak": d["peak_tflops"], "unit": "TFLOP/s",
@@ -429,6 +432,8 @@ def run_ours(a):
     else:
         roof = {"bound": "alu", "achieved": d.get("achieved_tflops"), "peak": alu_pk, "unit": "TFLOP/s",
                 "frac": d.get("frac"), "peak_source": alu_src}
+        if f64 and dom in ("leaf", "downward"):
+            roof["peak_source"] += "; the kernel runs in fixed point on the integer pipe, so frac can pass 1"
     roof["kernel"] = kern
     roof["concurrent"] = fused  # the near field shares the GPU with the expansion passes
     alu_total = sum(w[1] for k, w in work.items() if w[0] == "alu" and w[1])
@@ -862,7 +867,8 @@ def adaptive_measure(calls=20):
             "ms": t * 1e3, "cells_per_s": xs.size / t, "first_solve_ms": t_first * 1e3,
             "tree_build_ms": t_build * 1e3, "work": work,
             "roofline": {"bound": "alu", "achieved": tflops, "peak": pk64, "unit": "TFLOP/s",
-                         "frac": tflops / pk64, "peak_source": src64},
+                         "frac": tflops / pk64,
+                         "peak_source": src64 + "; the near field runs in fixed point on the integer pipe, so frac can pass 1"},
             "rel_l2_vs_p30": diff30,
             "mixed": mixed,
             "note": "FP64, p = 20, theta = 0.5; ms: device time of a solve on a kept tree (CUDA events); "

@@ -231,13 +231,14 @@ typedef struct {
     double theta_surface;  /* acceptance parameter the surface tree-code uses */
     int near_kernel;       /* near-field kernel a solve runs: 128 = tensor cores (tcgen05,
                               128-leaf tiles), 16 / 8 = FP32 cores with 16 / 8 targets per
-                              thread, 0 = the generic leaf kernel (FP64 plans) */
+                              thread, 0 = FP64 plans (fixed point on the integer pipe for
+                              orders up to 23 and leaf level >= 2, else the generic kernel) */
     int downward;          /* downward pass of a solve into a 16-byte aligned output: 2 = two
                               launches (every level's multipole-to-local translations in one,
                               then the local-to-local shifts and the evaluation per subtree of
                               the level L - 3 boxes), 3 = the same with the translations on the
                               tensor cores (option m2l_tensor), 1 = one launch per level,
-                              0 = generic per-level kernels */
+                              0 = FP64 plans */
 } pp_plan_info_t;
 
 int pp_plan_info(pp_plan plan, pp_plan_info_t* info);
@@ -350,9 +351,9 @@ int pp_atree_destroy(pp_atree tree);
  *    leaves were given to pp_atree_create, cell (cx, cy) of a block at cy*8 + cx (8 x 8 cells
  *    per block, cell side = block side / 8).
  * p_out: nleaf*64 device doubles, same layout.  order: 2..30.  stream: a CUDA stream or NULL.
- * Near field: between leaves of one level from a table of log|D| over integer cell offsets
- * (built once in FP64), between leaves of different levels directly.
- * The first solve on a tree uploads the tree, the lists and the table and allocates the
+ * Near field: from tables of log|D| over the integer offsets of the cells of a leaf pair, in
+ * cells or half cells of the finer leaf (built once in FP64); leaf pairs beyond the tables directly.
+ * The first solve on a tree uploads the tree, the lists and the tables and allocates the
  * expansions (synchronising the stream); so does a solve at a higher order than before.  They
  * stay with the tree until pp_atree_destroy, so later solves allocate nothing and only launch
  * kernels on the stream.  Solves on one tree share its arrays: order them on one stream.
@@ -377,7 +378,7 @@ int pp_atree_solve_mixed(pp_atree tree, int order, const float* q, float* p_out,
 /*
  * Pressure at npts off-grid points (the body's surface points, Sec. 2.3.1) on an adaptive grid,
  * FP64, by the tree-code over the adaptive tree (Appendix A.2: a group is accepted for a
- * target at a sufficient distance): depth-first from the root, a box whose half-diagonal r
+ * target at a sufficient distance): level by level from the root, a box whose half-diagonal r
  * is below theta d (d the distance of the point from its centre) contributes its multipole
  * (Eq. pressTruncated about the box centre), a leaf that is not accepted is summed directly
  * over its 64 cells, each clamped at its own rho_h (Eq. greenSum), any other box opens its

@@ -141,8 +141,9 @@ constexpr int kFarThreads = 64;
 // The sources of a column pair (k, k + 1) are one 16-byte load; for P1 > 13 the sums L sit in shared
 // memory (a column a thread, touched once an item), so the registers hold the pair's loads instead.
 // FP32-bound.  Alone, before (a product per source, a box's coefficients together) and now: 46.7 and
-// 45.7 us at 2048^2, p = 12, theta 0.75; 201 and 174 at p = 20, theta 0.5.  What the steps gain beside
-// the near field is more (4096^2 704 to 654 us): the loads no longer live off L1.
+// 45.5 us at 2048^2, p = 12, theta 0.75; 201 and 211 at p = 20, theta 0.5.  The gain is beside the near
+// field, whose shared memory leaves little L1 (the loads no longer live off it): the steps went from
+// 516 to 484 us (p = 20, theta 0.5) and 704 to 652 (4096^2, p = 12).
 struct M2LSource {
     int base, nb;  // pair (k, k + 1), k odd, at mp[base + k nb]; base < 0: outside the grid
     int box;       // flat box index (S arrays)
