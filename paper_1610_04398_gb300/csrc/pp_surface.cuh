@@ -174,6 +174,7 @@ __device__ __forceinline__ void surf_walk(const Tree<T>& t, const SurfaceArgs& a
             } else {
                 const unsigned tm = __ballot_sync(0xffffffffu, take);
                 if (na > kSurfCap - 32) {
+                    __syncwarp();  // the entries come from all lanes (a vote does not order memory)
                     for (int i = lane; i < na; i += 32) evaluate(sm.taken[i]);
                     na = 0;
                     __syncwarp();

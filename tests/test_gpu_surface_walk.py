@@ -70,3 +70,26 @@ def test_more_points_than_one_wave(order):
     assert np.isfinite(out[0]).all()
     assert rel_l2(out[0][:-1], out[1]) < 1e-6
     plan.destroy()
+
+
+def test_fp64_strict_walk_flushes_its_list():
+    """Acceptance 0.25 at 1024^2: more than 224 accepted boxes a point, so a walk evaluates its list
+    before its levels are done.  Allowed at each point: truncation theta^21 and 1e-14 for rounding (some
+    90 units), both of sum |q log r| there (every r is below 1): one wrong or missing box shows."""
+    npts = 533
+    snap = synth.cylinder_flow(1024, diameter=0.3, centre=(0.5, 0.5), n_surface=npts, seed=7)
+    plan = api.Plan(1024, snap.h, 20, 0.6, precision="fp64", lift=snap.lift, theta_surface=0.25)
+    f = [to_dev(a, plan.dtype) for a in (snap.u, snap.v, snap.chi, snap.usx, snap.usy)]
+    plan.rhs(*f, snap.lam)
+    pts, nrm = to_dev(snap.points, torch.float64), to_dev(snap.normals, torch.float64)
+    out = []
+    for _ in range(4):
+        per = torch.empty(npts * 5, dtype=torch.float64, device="cuda")
+        plan.surface_traction(f[0], f[1], pts, nrm, snap.nu, per_point=per)
+        out.append(per)
+    assert all(torch.equal(out[0], o) for o in out)
+    q = oracle.source_weights(oracle.rhs(snap.u, snap.v, snap.chi, snap.usx, snap.usy, h=snap.h, lam=snap.lam), snap.h)
+    ref = oracle.green_sum_grid(q, snap.h, snap.points[:, 0], snap.points[:, 1])
+    size = -oracle.green_sum_grid(np.abs(q), snap.h, snap.points[:, 0], snap.points[:, 1])
+    assert (np.abs(out[0].view(npts, 5)[:, 0].cpu().numpy() - ref) < (0.25 ** 21 + 1e-14) * size).all()
+    plan.destroy()
