@@ -142,8 +142,7 @@ struct pp_plan_s {
     size_t off_T = 0, off_TL = 0, off_Z = 0, off_ZI = 0;
     // surface scratch
     int surf_cap = 0;
-    double* Psurf = nullptr;
-    double* partial = nullptr;
+    double* Psurf = nullptr;  // the first block: k_surface's CTA sums
     double* forces_dev = nullptr;
     double* penal_buf = nullptr;  // penalisation force: block partials, then 4 results
     double* moments_buf = nullptr;  // body moments: block partials and counter, then 3 results
@@ -692,25 +691,15 @@ int64_t plan_bytes(int n, int order, double theta, int precision, int tile, int 
     return b;
 }
 
+// The scratch grows by an added block and never moves: k_surface keeps its CTA sums in the first
+// block, whose address the captured steps hold.  (Growing by reallocation freed it under them.)
 int ensure_surface(pp_plan p, int npts) {
     if (npts <= p->surf_cap) return PP_OK;
     const int cap = pp::surface_cap_after(p->surf_cap, npts);
-    // release the old buffers (stream-ordered work must not still use them)
-    if (p->Psurf) {
-        if (cudaStreamSynchronize(p->stream) != cudaSuccess) return PP_ERR_CUDA;
-        p->workspace -= pp::surface_scratch_bytes(p->surf_cap);
-        for (void* ptr : {(void*)p->Psurf, (void*)p->partial}) {
-            for (size_t i = 0; i < p->allocs.size(); ++i)
-                if (p->allocs[i] == ptr) {
-                    cudaFree(ptr);
-                    p->allocs.erase(p->allocs.begin() + long(i));
-                    break;
-                }
-        }
-    }
-    const int nb = (cap + pp::kSurfaceBlock - 1) / pp::kSurfaceBlock;
-    if (dalloc(p, (void**)&p->Psurf, sizeof(double) * size_t(cap)) != cudaSuccess) return PP_ERR_OOM;
-    if (dalloc(p, (void**)&p->partial, sizeof(double) * 4 * size_t(nb)) != cudaSuccess) return PP_ERR_OOM;
+    const int64_t held = p->surf_cap ? pp::surface_scratch_bytes(p->surf_cap) : 0;
+    void* block = nullptr;
+    if (dalloc(p, &block, size_t(pp::surface_scratch_bytes(cap) - held)) != cudaSuccess) return PP_ERR_OOM;
+    if (!p->Psurf) p->Psurf = static_cast<double*>(block);
     p->surf_cap = cap;
     return PP_OK;
 }
@@ -911,7 +900,7 @@ int run_surface(pp_plan p, const void* u, const void* v, int npts, const double*
     a.Psurf = p->Psurf;
     a.counter = reinterpret_cast<unsigned*>(p->forces_dev + 6);
     a.per_point = per_point;
-    a.partial = p->partial;
+    a.partial = nullptr;
     a.forces = dev_forces ? forces : p->forces_dev;
     a.lift = p->lift < 0 ? 2.0 * p->h : p->lift;
     a.mu2 = 2.0 * p->rho * nu;

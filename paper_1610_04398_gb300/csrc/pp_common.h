@@ -326,8 +326,12 @@ cudaError_t launch_export_expansion(const Tree<T>& t, int kind, int level, doubl
 constexpr int kSurfaceBlock = 64;
 // Surface scratch of a plan: a new plan holds it for kInitialSurfaceCap points and grows it
 // to surface_cap_after(cap, npts) points when a call brings more; surface_scratch_bytes is
-// what `cap` points take (the pressure per point and 4 partial sums per block).
+// what `cap` points take (a double per point and 4 per block), the figure pp_plan_bytes states.
+// k_surface uses the first kInitialSurfaceCap doubles only: four sums for each of at most
+// kSurfMaxCtas CTAs.
 constexpr int kInitialSurfaceCap = 4096;
+constexpr unsigned kSurfMaxCtas = 1024;
+static_assert(4 * kSurfMaxCtas <= kInitialSurfaceCap, "the CTA sums fit the first block of the scratch");
 int64_t surface_scratch_bytes(int cap);
 int surface_cap_after(int cap, int npts);
 constexpr int kDynSmemLimit = 200 * 1024;  // dynamic shared memory any launch may use

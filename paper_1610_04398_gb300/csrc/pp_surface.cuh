@@ -24,7 +24,6 @@ struct SurfCta {
 constexpr int kSurfCap = 256;         // candidates of a level; accepted boxes a warp holds at once (FP64)
 constexpr int kSurfLane = 16;         // accepted boxes a lane holds at once (mixed)
 constexpr int kSurfLeaves = 64;       // leaves summed directly, per point
-constexpr unsigned kSurfMaxCtas = 1024;  // four partial sums each: they fit the smallest surface scratch
 
 struct SurfWalk {  // a warp's lists
     int cand[2][kSurfCap];

@@ -93,3 +93,30 @@ def test_fp64_strict_walk_flushes_its_list():
     size = -oracle.green_sum_grid(np.abs(q), snap.h, snap.points[:, 0], snap.points[:, 1])
     assert (np.abs(out[0].view(npts, 5)[:, 0].cpu().numpy() - ref) < (0.25 ** 21 + 1e-14) * size).all()
     plan.destroy()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_captured_step_outlives_a_larger_call(precision):
+    """A step captured with few points, a call with more than the plan's scratch held so far, a replay:
+    the scratch grows without moving, so the replay gives the first launch's values bit for bit."""
+    snap = synth.cylinder_flow(128, diameter=0.3, centre=(0.5, 0.5), n_surface=20001, seed=3)
+    plan = api.Plan(128, snap.h, 12, 0.6, precision=precision, lift=snap.lift)
+    f = [to_dev(a, plan.dtype) for a in (snap.u, snap.v, snap.chi, snap.usx, snap.usy)]
+    pts, nrm = to_dev(snap.points, torch.float64), to_dev(snap.normals, torch.float64)
+    per = torch.empty(5 * 400, dtype=torch.float64, device="cuda")
+    forces = torch.zeros(6, dtype=torch.float64, device="cuda")
+    step = plan.capture_step(*f, snap.lam, p_out=torch.empty(128 * 128, dtype=plan.dtype, device="cuda"),
+                             points=pts[:400].contiguous(), normals=nrm[:400].contiguous(), nu=snap.nu,
+                             per_point=per, forces=forces)
+    step.launch()
+    first = per.clone(), forces.clone()
+    before = plan.info().workspace_bytes
+    plan.surface_traction(f[0], f[1], pts, nrm, snap.nu)
+    assert plan.info().workspace_bytes > before  # it did grow
+    spoil = torch.full((1 << 16,), float("nan"), dtype=torch.float64, device="cuda")
+    per.zero_(), forces.zero_()
+    step.launch()
+    torch.cuda.synchronize()
+    assert torch.equal(per, first[0]) and torch.equal(forces, first[1]) and torch.isnan(spoil).all()
+    step.destroy()
+    plan.destroy()
