@@ -272,6 +272,13 @@ __device__ __forceinline__ void cell_grad(const T* u, const T* v, int n, double 
     g[3] = (double(v[c + n]) - double(v[c - n])) * inv2h;
 }
 
+// "P is there", a barrier that the walking warps and the traction warp reach in different code:
+// a named one, since __syncthreads() has to be the same for all threads of a block.
+template <int kThreads>
+__device__ __forceinline__ void surf_barrier() {
+    asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory");
+}
+
 // The walks, the tractions and the force sums in one launch.  The traction warp splits the CTA's points,
 // then, while they are walked, forms what the tractions need besides P (the velocity gradient at the
 // lifted point, the dS), then the tractions and their sums.  The CTA that finishes last (a counter it
@@ -325,7 +332,7 @@ k_surface(Tree<T> t, const T* __restrict__ u, const T* __restrict__ v, SurfaceAr
                     surf_walk<T, P1T, false>(t, a, pts[warp], walk[warp], lane, overflow, phi[warp]);
                 if (__any_sync(0xffffffffu, overflow) && lane == 0) atomicExch(a.err, 1);
             }
-            __syncthreads();  // P is there
+            surf_barrier<kThreads>();  // P is there
         } else {
             double nx = 0.0, ny = 0.0, dS = 0.0, tnx = 0.0, tny = 0.0, s0 = 0.0;
             if (act) {
@@ -363,7 +370,7 @@ k_surface(Tree<T> t, const T* __restrict__ u, const T* __restrict__ v, SurfaceAr
                 tnx = a.mu2 * (g[0] * nx + dxy * ny);
                 tny = a.mu2 * (dxy * nx + g[3] * ny);
             }
-            __syncthreads();  // P is there
+            surf_barrier<kThreads>();  // P is there
             if (act) {
                 const SurfPhi f = phi[lane];
                 const double P = (f.pair ? df_to(f.hi, f.lo) + s0 : f.phi) * 0.15915494309189533576888376337251;
