@@ -273,9 +273,11 @@ __device__ __forceinline__ void cell_grad(const T* u, const T* v, int n, double 
 }
 
 // "P is there", a barrier that the walking warps and the traction warp reach in different code:
-// a named one, since __syncthreads() has to be the same for all threads of a block.
+// a named one, since __syncthreads() has to be the same for all threads of a block (bar.sync wants
+// whole warps: the lanes join first).
 template <int kThreads>
 __device__ __forceinline__ void surf_barrier() {
+    __syncwarp();
     asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory");
 }
 
