@@ -103,11 +103,12 @@ def test_captured_step_outlives_a_larger_call(precision):
     plan = api.Plan(128, snap.h, 12, 0.6, precision=precision, lift=snap.lift)
     f = [to_dev(a, plan.dtype) for a in (snap.u, snap.v, snap.chi, snap.usx, snap.usy)]
     pts, nrm = to_dev(snap.points, torch.float64), to_dev(snap.normals, torch.float64)
+    few, few_nrm = pts[:400].clone(), nrm[:400].clone()  # held while the step exists
     per = torch.empty(5 * 400, dtype=torch.float64, device="cuda")
     forces = torch.zeros(6, dtype=torch.float64, device="cuda")
-    step = plan.capture_step(*f, snap.lam, p_out=torch.empty(128 * 128, dtype=plan.dtype, device="cuda"),
-                             points=pts[:400].contiguous(), normals=nrm[:400].contiguous(), nu=snap.nu,
-                             per_point=per, forces=forces)
+    P = torch.empty(128 * 128, dtype=plan.dtype, device="cuda")
+    step = plan.capture_step(*f, snap.lam, p_out=P, points=few, normals=few_nrm, nu=snap.nu, per_point=per,
+                             forces=forces)
     step.launch()
     first = per.clone(), forces.clone()
     before = plan.info().workspace_bytes
