@@ -97,32 +97,54 @@ struct Tree {
 };
 
 // The multipole coefficients of box b (row-major) of level l.  FP64 plans keep a box's coefficients
-// together.  Mixed plans keep a level's as planes over its boxes: coefficient 0, then pairs (1, 2),
+// together.  Mixed plans keep a row of boxes as planes: coefficient 0, then pairs (1, 2),
 // (3, 4), ... of 16 bytes a box (a last unpaired one alone), so that a warp whose lanes take
 // neighbouring boxes reads and writes whole lines.  With a box's P1 coefficients together every
 // such access touched 26 lines, and the translations depended on all of them staying in L1, most of
-// which is shared memory while the near field runs beside them.  Pairs sit on 16 bytes for levels >= 1
-// (the array starts one element past a 16-byte boundary, and level_offset(l) P1 is odd there for odd P1).
+// which is shared memory while the near field runs beside them.  Planes over a row and not over a
+// level: a tile of boxes then lies in a few MB, where the planes of a large level put each
+// coefficient pair of it into memory pages of its own.  Pairs of odd P1 sit on 16 bytes (the array
+// starts one element past a 16-byte boundary; level_offset(l) P1 is odd and the side even for l >= 1,
+// and both are trivial at the root).
 template <typename T>
 struct Multipole {
     typedef typename cplx_of<T>::type C;
-    C* p;
-    int box, nb, P1;  // mixed: the box, the boxes of the level, the coefficients of a box
+    C* p;                // FP64: the box's coefficients; mixed: its row of boxes
+    int x, side, P1;     // mixed: the box in the row, the row's boxes, the coefficients of a box
     __device__ __forceinline__ C& operator[](int k) const {
         if constexpr (sizeof(T) == 8) return p[k];
         const int j = k - 1;
-        if (k == 0 || (k == P1 - 1 && !(j & 1))) return p[int64_t(nb) * k + box];  // a plane of its own
-        return p[int64_t(nb) * (1 + (j & ~1)) + 2 * box + (j & 1)];
+        if (k == 0 || (k == P1 - 1 && !(j & 1))) return p[side * k + x];  // a plane of its own
+        return p[side * (1 + (j & ~1)) + 2 * x + (j & 1)];
     }
-    // mixed plans, odd P1, levels >= 1: the pair (k, k + 1), k odd, as one 16-byte value
-    __device__ __forceinline__ float4* pair(int k) const {
-        return reinterpret_cast<float4*>(p + int64_t(nb) * k + 2 * box);
-    }
+    // mixed plans, odd P1: the pair (k, k + 1), k odd, as one 16-byte value
+    __device__ __forceinline__ float4* pair(int k) const { return reinterpret_cast<float4*>(p + side * k + 2 * x); }
 };
 template <typename T>
-__device__ __forceinline__ Multipole<T> multipole(const Tree<T>& t, int l, int64_t b) {
-    return {t.mp + (sizeof(T) == 4 ? level_offset(l) * t.P1 : (level_offset(l) + b) * t.P1), int(b), 1 << (2 * l), t.P1};
+__device__ __forceinline__ Multipole<T> multipole(const Tree<T>& t, int l, int x, int y) {
+    const int64_t row = level_offset(l) + (int64_t(y) << l);
+    return {t.mp + (sizeof(T) == 4 ? row : row + x) * t.P1, x, 1 << l, t.P1};
 }
+template <typename T>
+__device__ __forceinline__ Multipole<T> multipole(const Tree<T>& t, int l, int64_t b) {
+    return multipole(t, l, int(b) & ((1 << l) - 1), int(b >> l));
+}
+
+// Coefficient k of any box, for the kernels whose lanes take one coefficient each: element a side + m x
+// + c of the P1 side ones of the box's row (both layouts), so that a box costs a lane two
+// multiply-adds.
+template <typename T>
+struct CoefIndex {
+    int a, m, c;
+    __device__ __forceinline__ CoefIndex(int k, int P1) {
+        const int j = k - 1;
+        if (sizeof(T) == 8) a = 0, m = P1, c = k;
+        else if (k == 0 || (k == P1 - 1 && !(j & 1))) a = k, m = 1, c = 0;
+        else a = 1 + (j & ~1), m = 2, c = j & 1;
+    }
+    // row: level_offset + y side of the box's row (times P1 below 2^31 up to the largest grid and order)
+    __device__ __forceinline__ int at(int row, int side, int x, int P1) const { return row * P1 + a * side + m * x + c; }
+};
 
 // ------------------------------------------------------------------------------------
 // Double-float arithmetic: a value hi + lo held in two floats (|lo| <= ulp(hi) / 2), about

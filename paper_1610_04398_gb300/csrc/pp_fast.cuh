@@ -77,13 +77,13 @@ __device__ __forceinline__ void m2l_list(const Tree<T>& t, int l, int bx, int by
             const int sx = bx + en.dx, sy = by + en.dy;
             if (sx < 0 || sy < 0 || sx >= side || sy >= side) continue;
             src = off + int64_t(sy) * side + sx;
-            M = multipole(t, l, int64_t(sy) * side + sx);
+            M = multipole(t, l, sx, sy);
         } else {  // parent-level source box standing for four separated children
             const int hs = side >> 1;
             const int sx = (bx >> 1) + en.dx, sy = (by >> 1) + en.dy;
             if (sx < 0 || sy < 0 || sx >= hs || sy >= hs) continue;
             src = level_offset(l - 1) + int64_t(sy) * hs + sx;
-            M = multipole(t, l - 1, int64_t(sy) * hs + sx);
+            M = multipole(t, l - 1, sx, sy);
         }
         const C* tp = t.Tpow + int64_t(en.op) * P1;
         const C* tl = t.TpowL + int64_t(en.op) * P1;
@@ -145,8 +145,8 @@ constexpr int kFarThreads = 64;
 // field, whose shared memory leaves little L1 (the loads no longer live off it): the steps went from
 // 516 to 484 us (p = 20, theta 0.5) and 704 to 652 (4096^2, p = 12).
 struct M2LSource {
-    int base, nb;  // pair (k, k + 1), k odd, at mp[base + k nb]; base < 0: outside the grid
-    int box;       // flat box index (S arrays)
+    int base, side;  // pair (k, k + 1), k odd, at mp[base + k side]; base < 0: outside the grid
+    int box;         // flat box index (S arrays)
 };
 __device__ __forceinline__ M2LSource m2l_source(int packed, int P1, int l, int bx, int by) {
     M2LSource s{-1, 0, 0};
@@ -155,10 +155,10 @@ __device__ __forceinline__ M2LSource m2l_source(int packed, int P1, int l, int b
     const int side = 1 << lv;
     const int sx = (bx >> (l - lv)) + (packed & 255) - 128, sy = (by >> (l - lv)) + ((packed >> 8) & 255) - 128;
     if (sx < 0 || sy < 0 || sx >= side || sy >= side) return s;
-    const int off = int(level_offset(lv)), b = sy * side + sx;
-    s.base = off * P1 + 2 * b;
-    s.nb = 1 << (2 * lv);
-    s.box = off + b;
+    const int row = int(level_offset(lv)) + sy * side;
+    s.base = row * P1 + 2 * sx;
+    s.side = side;
+    s.box = row + sx;
     return s;
 }
 
@@ -210,7 +210,7 @@ __device__ __forceinline__ void m2l_items_df(const Tree<float>& t, int l, int bx
                 s[j] = S.x;
                 df_add(gh, gl, S.x, S.y);
             }
-            const int nb = 1 << (2 * (l - (en.m[0] >> 16)));  // of the members' level (member 0 is always there)
+            const int ms = 1 << (l - (en.m[0] >> 16));  // the side of the members' level (member 0 is always there)
             const float2* tp = t.Tpow + int64_t(en.op) * P1;
             float yr[P1], yi[P1];
             yr[0] = 0.f;
@@ -229,7 +229,7 @@ __device__ __forceinline__ void m2l_items_df(const Tree<float>& t, int l, int bx
                 float4 m4[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
-                    m4[j] = base[j] >= 0 ? *reinterpret_cast<const float4*>(t.mp + base[j] + kp * nb)
+                    m4[j] = base[j] >= 0 ? *reinterpret_cast<const float4*>(t.mp + base[j] + kp * ms)
                                          : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
@@ -288,7 +288,7 @@ __device__ __forceinline__ void m2l_items_df(const Tree<float>& t, int l, int bx
         }
 #pragma unroll
         for (int kp = 1; kp < P1; kp += 2) {
-            const float4 m4 = *reinterpret_cast<const float4*>(t.mp + src.base + kp * src.nb);
+            const float4 m4 = *reinterpret_cast<const float4*>(t.mp + src.base + kp * src.side);
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
                 const int k = kp + u;
@@ -704,7 +704,7 @@ __global__ void __launch_bounds__(32 * kRhsWarps, (P1 <= 17 ? 16 : 8) / kRhsWarp
             if (act && !(lane & 1)) {
                 const int64_t box = level_offset(t.Lleaf) + int64_t(LY) * t.nL + (x0 >> 3);
                 store_S_leaf(t, box, ar[0]);
-                const Multipole<float> M = multipole(t, t.Lleaf, int64_t(LY) * t.nL + (x0 >> 3));
+                const Multipole<float> M = multipole(t, t.Lleaf, x0 >> 3, LY);
                 M[0] = make_float2(ar[0], 0.f);
 #pragma unroll
                 for (int k = 1; k < P1; k += 2) *M.pair(k) = make_float4(ar[k], ai[k], ar[k + 1], ai[k + 1]);

@@ -146,6 +146,10 @@ __global__ void __launch_bounds__(256) k_p2m(Tree<T> t) {
         store_S_leaf(t, off + leaf, s0);
         multipole(t, t.Lleaf, leaf)[0] = cmake<T>(s0, T(0));
     }
+    // Mixed plans collect the four leaves of a warp and store them as planes; FP64 ones store at once.
+    __shared__ C stage[sizeof(T) == 4 ? 8 : 1][sizeof(T) == 4 ? 4 : 1][kMaxP1 + 1];
+    const int lane = threadIdx.x & 31, w = sizeof(T) == 4 ? threadIdx.x >> 5 : 0;
+    C* rec = sizeof(T) == 4 ? stage[w][(lane >> 3) & (sizeof(T) == 4 ? 3 : 0)] : t.mp + (off + leaf) * P1;
     for (int k = 1; k < P1; ++k) {
         T ar = T(0), ai = T(0);
 #pragma unroll
@@ -161,9 +165,20 @@ __global__ void __launch_bounds__(256) k_p2m(Tree<T> t) {
             ar += __shfl_xor_sync(0xffffffffu, ar, o);
             ai += __shfl_xor_sync(0xffffffffu, ai, o);
         }
-        if (act && row == (k & 7)) {
+        if ((sizeof(T) == 4 || act) && row == (k & 7)) {
             const T ik = T(1) / T(k);
-            multipole(t, t.Lleaf, leaf)[k] = cmake<T>(ar * ik, ai * ik);
+            rec[k] = cmake<T>(ar * ik, ai * ik);
+        }
+    }
+    if constexpr (sizeof(T) == 4) {
+        __syncwarp();
+        const int lf = lane & 3;
+        const int64_t mine = leaf - (lane >> 3) + lf;
+        if (mine >= nleaf) return;
+        const Multipole<T> M = multipole(t, t.Lleaf, mine);
+        for (int k = 1 + 2 * (lane >> 2); k < P1; k += 16) {  // a pair a lane, the last one perhaps alone
+            M[k] = stage[w][lf][k];
+            if (k + 1 < P1) M[k + 1] = stage[w][lf][k + 1];
         }
     }
 }
@@ -237,8 +252,7 @@ __global__ void __launch_bounds__(128) k_m2m(Tree<T> t, int l) {
     C* cb = buf[warp];
     for (int idx = lane; idx < 4 * P1; idx += 32) {
         const int q = idx / P1, k = idx % P1;
-        const int64_t child = int64_t(2 * by + (q >> 1)) * cs + 2 * bx + (q & 1);
-        cb[idx] = multipole(t, l + 1, child)[k];
+        cb[idx] = t.mp[CoefIndex<T>(k, P1).at(int(coff) + (2 * by + (q >> 1)) * cs, cs, 2 * bx + (q & 1), P1)];
     }
     __syncwarp();
     for (int k = 1 + lane; k < P1; k += 32) {
@@ -247,7 +261,7 @@ __global__ void __launch_bounds__(128) k_m2m(Tree<T> t, int l) {
             const C* A = t.Am2m + int64_t(q) * P1 * P1;
             for (int j = 0; j <= k; ++j) cfma(acc, A[j * P1 + k], cb[q * P1 + j]);
         }
-        multipole(t, l, b)[k] = acc;
+        t.mp[CoefIndex<T>(k, P1).at(int(poff) + by * side, side, bx, P1)] = acc;
     }
     if (lane == 0) {
         double S = 0.0;
@@ -307,16 +321,20 @@ __global__ void __launch_bounds__(128) k_m2l(Tree<T> t, int l) {
             const int sx = bx + en.dx, sy = by + en.dy;
             if (sx < 0 || sy < 0 || sx >= side || sy >= side) continue;
             src = off + int64_t(sy) * side + sx;
-            M = multipole(t, l, int64_t(sy) * side + sx);
+            if constexpr (sizeof(T) == 4) M = multipole(t, l, int64_t(sy) * side + sx);
         } else {
             const int hs = side >> 1;
             const int sx = (bx >> 1) + en.dx, sy = (by >> 1) + en.dy;
             if (sx < 0 || sy < 0 || sx >= hs || sy >= hs) continue;
             src = level_offset(l - 1) + int64_t(sy) * hs + sx;
-            M = multipole(t, l - 1, int64_t(sy) * hs + sx);
+            if constexpr (sizeof(T) == 4) M = multipole(t, l - 1, int64_t(sy) * hs + sx);
         }
         __syncwarp();
-        for (int k = lane; k < P1; k += 32) sb[k] = M[k];
+        if constexpr (sizeof(T) == 4) {
+            for (int k = lane; k < P1; k += 32) sb[k] = M[k];
+        } else {
+            for (int k = lane; k < P1; k += 32) sb[k] = t.mp[src * P1 + k];
+        }
         __syncwarp();
         const C* B = t.Bm2l + int64_t(en.op) * P1 * P1;
         for (int r = 0; r < 2; ++r) {
