@@ -139,11 +139,20 @@ constexpr int kFarThreads = 64;
 // The lists hold 4 to 15 such groups of two to four sources; the flops of a list fall to 0.74 (p =
 // 12, theta 0.75) and 0.70 (p = 20, theta 0.5) of one product per source.
 // The sources of a column pair (k, k + 1) are one 16-byte load; for P1 > 13 the sums L sit in shared
-// memory (a column a thread, touched once an item), so the registers hold the pair's loads instead.
-// FP32-bound.  Alone, before (a product per source, a box's coefficients together) and now: 46.7 and
-// 45.5 us at 2048^2, p = 12, theta 0.75; 201 and 211 at p = 20, theta 0.5.  The gain is beside the near
-// field, whose shared memory leaves little L1 (the loads no longer live off it): the steps went from
-// 516 to 484 us (p = 20, theta 0.5) and 704 to 652 (4096^2, p = 12).
+// memory (a column a thread, touched once an item), so the registers hold the pair's loads instead,
+// and for P1 > 13 the next column pair is read before this pair's products (at 13 the registers
+// do not hold it: 16 to 30 us more in 2 ms at 8192^2).
+// Waits for its loads: at 2048^2, p = 12, theta 0.75 it issues in 53% of the cycles, the FMA pipe is busy
+// in 31% and long scoreboard is the largest stall.  The gain over a product per source from
+// whole records is beside the near field, whose shared memory leaves little L1: captured steps went
+// from 516 to 480 us (2048^2, p = 20, theta 0.5), 712 to 650 (4096^2, p = 12, theta 0.6) and 1189 to 1105
+// (4096^2, p = 20, theta 0.6).  Alone, as in separate calls where the near field has finished before, both
+// take the same time within 1.5% (2048^2, p = 20, theta 0.5: the calls 523 and 527 us).
+// Up to four sources at once want four times the lines in L1.  Beyond the L2 (leaf multipoles over
+// kGroupedBytes) that costs more than the shared products save and every source goes by itself:
+// 8192^2, p = 20, theta 0.7: step 3628 us grouped, 3375 not, 3913 from records (the calls 3431, 3365
+// and 3312); what stays slower than records there are separate calls at p = 16 and 24 (3 and 10%).
+constexpr int64_t kGroupedBytes = int64_t(1) << 27;
 struct M2LSource {
     int base, side;  // pair (k, k + 1), k odd, at mp[base + k side]; base < 0: outside the grid
     int box;         // flat box index (S arrays)
@@ -192,6 +201,7 @@ template <int P1, bool kGroups>
 __device__ __forceinline__ void m2l_items_df(const Tree<float>& t, int l, int bx, int by, int e0, int stride,
                                              M2LSums<P1>& L, float& ah, float& al, float& sh, float& sl) {
     static_assert(P1 % 2 == 1, "columns 1 .. P1 - 1 in pairs");
+    constexpr bool kAhead = M2LSums<P1>::kShared;  // the next pair of columns is read before this one's products
     const int par = (bx & 1) + 2 * (by & 1);
     const M2LGroup* lst = t.ig + int64_t(par) * t.il_stride;
     const int ng = kGroups ? t.ig_groups[par] : 0, cnt = kGroups ? t.ig_count[par] : t.il_count[par];
@@ -224,13 +234,25 @@ __device__ __forceinline__ void m2l_items_df(const Tree<float>& t, int l, int bx
                     yi[ll] = (ll & 3) == 1 ? -c * h2 : (ll & 3) == 3 ? c * h2 : 0.f;
                 }
             }
+            const auto fetch = [&](int kp, float4 (&v)[4]) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    v[j] = base[j] >= 0 ? *reinterpret_cast<const float4*>(t.mp + base[j] + kp * ms)
+                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+            };
+            float4 ahead[4];
+            if constexpr (kAhead) fetch(1, ahead);
 #pragma unroll
             for (int kp = 1; kp < P1; kp += 2) {
                 float4 m4[4];
+                if constexpr (kAhead) {
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    m4[j] = base[j] >= 0 ? *reinterpret_cast<const float4*>(t.mp + base[j] + kp * ms)
-                                         : make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int j = 0; j < 4; ++j) m4[j] = ahead[j];
+                    if (kp + 2 < P1) fetch(kp + 2, ahead);
+                    asm volatile("" ::: "memory");  // the loads stay ahead of this pair's products
+                } else {
+                    fetch(kp, m4);
+                }
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
                     const int k = kp + u;
@@ -286,9 +308,18 @@ __device__ __forceinline__ void m2l_items_df(const Tree<float>& t, int l, int bx
             yr[ll] = c_ops.m2l[ll][0] * Sd.x;
             yi[ll] = 0.f;
         }
+        float4 ahead = make_float4(0.f, 0.f, 0.f, 0.f);
+        if constexpr (kAhead) ahead = *reinterpret_cast<const float4*>(t.mp + src.base + src.side);
 #pragma unroll
         for (int kp = 1; kp < P1; kp += 2) {
-            const float4 m4 = *reinterpret_cast<const float4*>(t.mp + src.base + kp * src.side);
+            float4 m4;
+            if constexpr (kAhead) {
+                m4 = ahead;
+                if (kp + 2 < P1) ahead = *reinterpret_cast<const float4*>(t.mp + src.base + (kp + 2) * src.side);
+                asm volatile("" ::: "memory");
+            } else {
+                m4 = *reinterpret_cast<const float4*>(t.mp + src.base + kp * src.side);
+            }
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
                 const int k = kp + u;
@@ -912,7 +943,7 @@ __global__ void __launch_bounds__(128) k_m2l_chain(Tree<float> t, int lt, LevelL
 // its box and the 84 boxes below it.
 // ------------------------------------------------------------------------------------
 template <int P1>
-struct FarOcc {  // resident kFarThreads-thread CTAs per SM of k_m2l_far (register budget without spills)
+struct FarOcc {  // resident kFarThreads-thread CTAs per SM of k_m2l_far (grouped forms spill 16 bytes at P1 = 13, 104 at 21)
     static constexpr int value = P1 <= 13 ? 9 : P1 <= 21 ? 8 : 6;
 };
 constexpr int kDownAnc = 12;     // ancestor levels 2..lr-1 a CTA of k_down_tree can hold (L <= 17)

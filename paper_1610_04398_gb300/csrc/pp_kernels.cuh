@@ -804,6 +804,7 @@ cudaError_t launch_m2l_far(const Tree<T>& t, cudaStream_t st) {
         const Tree<float>& tf = reinterpret_cast<const Tree<float>&>(t);
         int64_t boxes = 0;
         for (int l = 2; l <= t.Lleaf; ++l) boxes += int64_t(1) << (2 * l);
+        // Sources are grouped where a thread has a box to itself and the leaf multipoles fit the L2 (k_m2l_far).
         // S threads per box so that the grid fills at least three quarters of the resident
         // threads of k_m2l_far (resident_threads counts 384 per SM for mixed plans)
         const double lnRoot = std::log(double(t.n) * t.h);
@@ -814,7 +815,7 @@ cudaError_t launch_m2l_far(const Tree<T>& t, cudaStream_t st) {
         int S = 1;                                                                      \
         while (S < 32 && 4 * boxes * S < 3 * slots) S <<= 1;                            \
         const unsigned blocks = unsigned((boxes * S + kFarThreads - 1) / kFarThreads);  \
-        if (S == 1)                                                                     \
+        if (S == 1 && int64_t(8 * P) << (2 * t.Lleaf) <= kGroupedBytes)                 \
             k_m2l_far<P, true><<<blocks, kFarThreads, 0, st>>>(tf, t.Lleaf - 3, S, lnRoot); \
         else                                                                            \
             k_m2l_far<P, false><<<blocks, kFarThreads, 0, st>>>(tf, t.Lleaf - 3, S, lnRoot); \
