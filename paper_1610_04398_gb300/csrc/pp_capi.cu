@@ -166,6 +166,8 @@ struct pp_plan_s {
     // FP64 plans of the fixed-point path (pp_fp64.cuh)
     bool use_f64 = false;
     pp::F64Scales f64sc = {};
+    double near_ln = 0.0;
+    int near_q = 0, near_k = 0;
     std::vector<double> op_geo;            // [op][tau_x, tau_y, side ratio]
     std::vector<pp::M2LEntry> il_host;     // the interaction lists as uploaded
     void* ktc = nullptr;
@@ -229,6 +231,9 @@ pp::Tree<T> make_tree(const pp_plan p) {
     t.P1 = p->P1;
     t.h = p->h;
     t.lnh = std::log(p->h);
+    t.near_ln = p->near_ln;
+    t.near_q = p->near_q;
+    t.near_k = p->near_k;
     t.inv_h = 1.0 / p->h;
     t.x0 = p->x0;
     t.y0 = p->y0;
@@ -397,13 +402,6 @@ int upload_tables(pp_plan p) {
     }
     int maxl = 0;
     for (int c = 0; c < 4; ++c) maxl = std::max(maxl, int(lists[c].size()));
-    if constexpr (sizeof(T) == 8) {
-        if (p->use_f64) {  // the operators and the near-field table as fixed point
-            pp::f64_pack_m2l(tabT.data() + p->off_B, p->n_ops, P1, maxl, &p->f64sc);
-            p->f64sc.ln_root = std::log(double(p->n) * p->h);
-            pp::f64_pack_near(Kr.data(), p->Rk);
-        }
-    }
     p->il_stride = std::max(maxl, 1);
     std::vector<pp::M2LEntry> ilh(size_t(4) * p->il_stride, pp::M2LEntry{0, 0, 0, 0});
     for (int c = 0; c < 4; ++c) {
@@ -411,6 +409,13 @@ int upload_tables(pp_plan p) {
         for (size_t i = 0; i < lists[c].size(); ++i) ilh[size_t(c) * p->il_stride + i] = lists[c][i];
     }
     p->il_host = ilh;
+    if constexpr (sizeof(T) == 8) {
+        if (p->use_f64) {  // the operators and the near-field table as fixed point
+            pp::f64_pack_m2l(tabT.data() + p->off_B, p->n_ops, P1, ilh.data(), p->il_count, p->il_stride, &p->f64sc);
+            p->f64sc.ln_root = std::log(double(p->n) * p->h);
+            pp::f64_pack_near(Kr.data(), p->Rk, p->h, &p->near_ln, &p->near_q, &p->near_k);
+        }
+    }
     // the same lists with the sources at 90 degree rotations of one offset grouped, groups first
     std::vector<pp::M2LGroup> igh;
     if (sizeof(T) == 4) {

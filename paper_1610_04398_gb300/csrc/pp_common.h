@@ -80,6 +80,8 @@ struct Tree {
     int ig_groups[4];      // the groups of two to four first,
     int ig_count[4];       // then the single sources
     const T* Ktab;         // [(2 Rk + 1)^2]: log max(h |Delta|, rho_h) for integer cell offsets
+    double near_ln;        // fixed-point FP64 plans: the part of log h that is not in the near-field table,
+    int near_q, near_k;    // and the bits of its weights and kernel values
     const T* Krel;         // same offsets, log max(|Delta|, rho_h / h) = Ktab - log h (split solve: the
                            // log h part is added exactly from the near leaves' monopoles)
     int Rk;                // largest |Delta| component in the near field (8 Dmax + 7)
@@ -244,18 +246,18 @@ cudaError_t prepare_m2l_tc();
 // The FP64 path (orders up to 23, leaf level >= 2; pp_fp64.cuh): scales of its fixed-point
 // translation operators, the words of the plan's counter array (level exponents and arrival
 // counters), the packing of the operators and of the near-field table in place of their FP64
-// values, and the launches.  launch_near64 writes the near field (without its log h part, which
-// launch_down64 adds) to p_out; launch_down64 shifts the locals down and, with p_out, adds the
-// local expansions to it.
+// values, and the launches.  launch_near64 writes the near field's 2 pi P to p_out; launch_down64 shifts the
+// locals down and, with p_out, adds the local expansions to it and divides by 2 pi.
 struct F64Scales {
     int wbits;       // fixed-point bits of the operators
+    int fold_mask;   // list entries between two carries of the cross terms, less one
     int el[32];      // power-of-two scale of each row
     double ln_root;  // log of the root box side
 };
 bool f64_ok(int P1, int Lleaf);
 size_t f64_counter_words(int Lleaf);
-void f64_pack_m2l(double2* B, int n_ops, int P1, int max_entries, F64Scales* sc);
-void f64_pack_near(double* K, int R);
+void f64_pack_m2l(double2* B, int n_ops, int P1, const M2LEntry* il, const int* il_count, int il_stride, F64Scales* sc);
+void f64_pack_near(double* K, int R, double h, double* near_ln, int* near_q, int* near_k);
 cudaError_t launch_rhs64(const Tree<double>& t, const double* u, const double* v, const double* chi, const double* usx,
                          const double* usy, double rho, double lam, double* f_out, cudaStream_t st);
 cudaError_t launch_up64(const Tree<double>& t, cudaStream_t st);

@@ -12,6 +12,8 @@
 // Times at the kernels: one GB300, 1024^2, p = 20, theta = 0.5.
 #pragma once
 
+#include <vector>
+
 #include "pp_fixed.cuh"
 #include "pp_kernels.cuh"
 
@@ -315,14 +317,19 @@ __global__ void __launch_bounds__(128) k_up64(Tree<double> t) {
 
 // ------------------------------------------------------------------------------------
 // Near field in fixed point.  One CTA of 256 threads per 2 x 2 leaves: the source weights of the
-// (2 + 2D)^2 leaves around them, relative to their largest exponent (53 bits), and a quadrant of
-// the kernel table log max(|(mx, my)|, rho_h / h) (2^-52 units) sit in shared memory; log h enters
-// through the near leaves' monopoles in k_down64.  A thread owns a row of 8 target cells and one
-// source row of every near leaf: 15 kernel values and 8 weights for 64 cell pairs, three mad_wide
-// each.  The eight source rows (lanes of a target row) are added in integers, one lane a target.
+// (2 + 2D)^2 leaves around them, 55 or 56 bits relative to their largest exponent (what FP64 holds of
+// weights within two or three bits of it), and a quadrant of the kernel table log(h max(|(mx, my)|, rho_h /
+// h)) (2^-52 or 2^-53 units; h clamped to e^-11 .. e^11, what is left of log h entering through the near
+// leaves' monopoles in k_down64) sit in shared memory.  A thread owns a row of 8 target cells and one
+// source row of every near leaf: 15 kernel values and 8 weights for 64 cell pairs, an exact product each
+// (FixedSum).  The eight source rows (lanes of a target row) are added in integers, one lane a target.
+// Before, with 53 bits, the products' low digits dropped and all of log h in the monopoles, whose product
+// cancels most of the table's sum, the near field's error was 1.5 to 20 times that of FP64
+// multiply-adds; now 0.4 to 1.1 times (64^2, p = 20, theta = 0.5: relative l2 of the field 3.5 and 6.0e-16).
 // Bound by the integer multiply-adds: 1600 pairs a cell at theta = 0.5, 570 us at 1024^2 at the
-// measured rate; 2818 us before on the FP64 pipe (evaluation included).
+// measured rate; 2818 us on the FP64 pipe (evaluation included), 713 with the low digits dropped, 770 now.
 // ------------------------------------------------------------------------------------
+constexpr double kNearLn = 11.0;  // |log h| in the table: with log 66 below 16
 constexpr int kNearRow = 10;  // int2 per source row (8 used): rows on distinct banks
 
 __host__ __device__ constexpr int near64_halo(int D) { return (2 + 2 * D) * (2 + 2 * D); }
@@ -355,37 +362,38 @@ __global__ void __launch_bounds__(256, 2) k_near64(Tree<double> t, double* __res
     const bool bad = e == kExpBad;
     e = max(e, -900);
     for (int i = tid; i < H * H * 64; i += 256)
-        qs[(i >> 3) * kNearRow + (i & 7)] = bad ? int2{0, 0} : split28(to_fixed(weight(i), e, 53));
+        qs[(i >> 3) * kNearRow + (i & 7)] = bad ? int2{0, 0} : split28(to_fixed(weight(i), e, t.near_q));
     __syncthreads();
 
     const int lx = (warp >> 1) & 1, ly = warp >> 2, ty = (lane >> 3) + 4 * (warp & 1), sy = lane & 7;
     const int LX = LX0 + lx, LY = LY0 + ly;
     double acc = 0.0;  // this lane's target, column sy of row ty
-    long long hh[8], mid[8];
+    FixedSum sum[8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) hh[j] = mid[j] = 0;
-    // the eight lanes of a row: lane sy ends with target sy's sum (butterfly, in integers)
+    for (int j = 0; j < 8; ++j) sum[j].clear();
+    // the eight lanes of a row: lane sy ends with target sy's sum (butterfly, in integers), as v1 2^68 + v0 2^28
     const auto drain = [&]() {
-        int lo[8];
+        long long v1[8], v0[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {  // mid's upper part into hh, 28 bits left
-            hh[j] += mid[j] >> 28;
-            lo[j] = int(mid[j]) & 0x0fffffff;
+        for (int j = 0; j < 8; ++j) {
+            long long hi;
+            int lo;
+            sum[j].digits(hi, lo);
+            v1[j] = hi >> 12;
+            v0[j] = (hi & 4095) << 28 | lo;
+            sum[j].clear();
         }
 #pragma unroll
         for (int o = 4; o >= 1; o >>= 1)
 #pragma unroll
             for (int j = 0; j < o; ++j) {
                 const bool up = (sy & o) != 0;
-                const long long sh = up ? hh[j] : hh[j + o];
-                const int sl = up ? lo[j] : lo[j + o];
-                hh[j] = (up ? hh[j + o] : hh[j]) + __shfl_xor_sync(0xffffffffu, sh, o);
-                lo[j] = (up ? lo[j + o] : lo[j]) + __shfl_xor_sync(0xffffffffu, sl, o);
+                const long long s1 = up ? v1[j] : v1[j + o], s0 = up ? v0[j] : v0[j + o];
+                v1[j] = (up ? v1[j + o] : v1[j]) + __shfl_xor_sync(0xffffffffu, s1, o);
+                v0[j] = (up ? v0[j + o] : v0[j]) + __shfl_xor_sync(0xffffffffu, s0, o);
             }
-        // units: 2^(e - 53) 2^-52
-        acc = fma(double(hh[0]), pow2(56 + e - 105), fma(double(lo[0]), pow2(28 + e - 105), acc));
-#pragma unroll
-        for (int j = 0; j < 8; ++j) hh[j] = mid[j] = 0;
+        const int unit = e - t.near_q - t.near_k;
+        acc += fma(double(v1[0]), pow2(68 + unit), double(v0[0]) * pow2(28 + unit));
     };
     int n = 0;
     for (int i = 0; i < t.n_near; ++i) {
@@ -393,27 +401,34 @@ __global__ void __launch_bounds__(256, 2) k_near64(Tree<double> t, double* __res
         if (LX + o.x < 0 || LY + o.y < 0 || LX + o.x >= nL || LY + o.y >= nL) continue;  // warp-uniform
         const int4* q4 = reinterpret_cast<const int4*>(qs + (((ly + D + o.y) * H + lx + D + o.x) * 8 + sy) * kNearRow);
         const int2* kr = tab + abs(8 * o.y + sy - ty) * W;
-        int2 kc[15];
+        int2 kc[15];  // source column r and target column j: kc[r - j + 7]
+        int ks[15];
+        const auto kernel = [&](int m) {
+            kc[m] = kr[abs(8 * o.x - 7 + m)];
+            ks[m] = kc[m].x + kc[m].y;
+        };
 #pragma unroll
-        for (int m = 0; m < 15; ++m) kc[m] = kr[abs(8 * o.x - 7 + m)];
+        for (int m = 0; m < 7; ++m) kernel(m);
 #pragma unroll
         for (int r2 = 0; r2 < 4; ++r2) {
             const int4 a = q4[r2];
-            const int qh[2] = {a.x, a.z}, ql[2] = {a.y, a.w};
+            const int2 q[2] = {int2{a.x, a.y}, int2{a.z, a.w}};
 #pragma unroll
-            for (int u = 0; u < 2; ++u)
+            for (int u = 0; u < 2; ++u) {
+                kernel(2 * r2 + u + 7);
+                const int qsum = q[u].x + q[u].y;
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    const int2 kv = kc[2 * r2 + u - j + 7];
-                    mad_wide(hh[j], qh[u], kv.x);
-                    mad_wide(mid[j], qh[u], kv.y);
-                    mad_wide(mid[j], ql[u], kv.x);
+                    const int m = 2 * r2 + u - j + 7;
+                    sum[j].add(q[u], qsum, kc[m], ks[m]);
                 }
+            }
         }
-        if ((++n & 31) == 0) drain();  // 32 leaves: 2048 terms a target stay below 2^63
+        // 16 leaves, 128 terms a thread: the sums stay below 2^63 (f64_pack_near), v1 then adds eight lanes
+        if ((++n & 15) == 0) drain();
     }
     drain();
-    const double out = bad ? __longlong_as_double(0x7ff8000000000000ll) : acc * kInv2Pi;
+    const double out = bad ? __longlong_as_double(0x7ff8000000000000ll) : acc;
     p_out[int64_t(LY * 8 + ty) * t.n + LX * 8 + sy] = out;
 }
 
@@ -421,24 +436,30 @@ __global__ void __launch_bounds__(256, 2) k_near64(Tree<double> t, double* __res
 // Multipole-to-local translations of every level in fixed point.  Per list entry the operator is
 // one complex P1 x P1 matrix B (the same for all targets of a child position); a row l of B is
 // scaled by a power of two that makes its largest entry below 1 (with column k carrying the
-// 2^-floor(k/2) the multipoles are scaled by), wbits fixed-point bits; the multipoles have 52 bits
+// 2^-floor(k/2) the multipoles are scaled by), wbits fixed-point bits; the multipoles have kM2LBits
 // relative to the largest of the two levels involved.  Complex products by three real ones,
-// (a + i b)(c + i d): ac, bd and (a + b)(c + d) accumulate separately over all entries.
+// (a + i b)(c + i d): ac, bd and (a + b)(c + d) accumulate separately over all entries, modulo 2^64:
+// only their differences have to fit, and those are bounded by the sum of a row's entries over an entry
+// group's part of the list, 4 to 45 times the largest, not by their number (f64_pack_m2l).  So 56 + 57 bits
+// fit; with 52 + 54 the dropped low products were 2^-52 of the largest term and the far field's error up
+// to 20 times that of FP64 multiply-adds; now 0.5 to 1.1 times.
 // A CTA takes 32 targets of one child position (lane = target): warp = entry group x rows; four
 // entry groups of four warps, each staging its entries' sources (converted from FP64) and operator
 // in shared memory, one entry ahead.  Small grids split the entries further over a cluster of CTAs
-// that add their integer sums through distributed shared memory.  The S log|tau| terms stay FP64.
+// that add their integer sums through distributed shared memory.  The S log(|tau| side) terms stay FP64, a
+// logarithm each (log|tau| and log side apart cancel).
 // Bound by the integer multiply-adds, 9 per complex product: 390 us at 1024^2, p = 20, theta = 0.5
 // at the measured rate; 2665 us before on the FP64 pipe in one launch per level, 918 now.
 // ------------------------------------------------------------------------------------
 constexpr int kM2LPad = 33;
+constexpr int kM2LBits = 56;
 
 __host__ __device__ constexpr size_t m2l64_group_bytes(int P1) {  // one buffer of one entry group
     return sizeof(int4) * (size_t(P1) * kM2LPad + size_t(P1) * P1);
 }
 inline size_t m2l64_smem(int P1) {  // the staging buffers, later the groups' sums and S terms
     const size_t stage = 8 * m2l64_group_bytes(P1), rows = P1 <= 16 ? 16 : P1 <= 20 ? 20 : 24;
-    const size_t sums = 4 * rows * 4 * 32 * 8 + 4 * 2 * 32 * 8;
+    const size_t sums = 4 * rows * 4 * 32 * 8 + 4 * 32 * 8;
     return stage > sums ? stage : sums;
 }
 
@@ -491,7 +512,7 @@ __global__ void __launch_bounds__(512, 1) k_m2l64(Tree<double> t, F64Scales sc, 
     const int* le = level_exp(t);
     int E = max(le[l], le[l - 1]);
     const bool bad = E == kExpBad;
-    E = max(E, -900);
+    E = max(E, -840);  // so that every unit below is a normal number
     const M2LEntry* lst = t.il + int64_t(par) * t.il_stride;
     const int cnt = t.il_count[par];
     int4* const buf0 = smm + size_t(eg) * 2 * (P1 * kM2LPad + P1 * P1);
@@ -524,7 +545,8 @@ __global__ void __launch_bounds__(512, 1) k_m2l64(Tree<double> t, F64Scales sc, 
                 int4 x = make_int4(0, 0, 0, 0);
                 if (s >= 0 && !bad) {
                     const double2 m = t.mp[s * P1 + lane];
-                    const int2 re = split28(to_fixed(m.x, E - (lane >> 1), 52)), im = split28(to_fixed(m.y, E - (lane >> 1), 52));
+                    const int2 re = split28(to_fixed(m.x, E - (lane >> 1), kM2LBits)),
+                               im = split28(to_fixed(m.y, E - (lane >> 1), kM2LBits));
                     x = make_int4(re.x, re.y, im.x, im.y);
                 }
                 xs[lane * kM2LPad + j] = x;
@@ -534,7 +556,8 @@ __global__ void __launch_bounds__(512, 1) k_m2l64(Tree<double> t, F64Scales sc, 
     long long h1[NL], m1[NL], h2[NL], m2[NL], h3[NL], m3[NL];
 #pragma unroll
     for (int i = 0; i < NL; ++i) h1[i] = m1[i] = h2[i] = m2[i] = h3[i] = m3[i] = 0;
-    double a0 = 0.0, sumS = 0.0;
+    const double lnS = fma(double(-l), 0.69314718055994530941723212145818, sc.ln_root);  // log of the box side
+    double a0 = 0.0;
     const int l0 = lg * NL;  // this warp's rows l0 .. l0 + NL - 1 (those below P1)
     const int step = 4 * cs, first = int(rank) * 4 + eg;
     const auto fold = [&]() {  // mid's upper part into hh, 28 bits left
@@ -576,14 +599,12 @@ __global__ void __launch_bounds__(512, 1) k_m2l64(Tree<double> t, F64Scales sc, 
                 }
             }
         }
-        if ((++done & 3) == 0) fold();  // four entries of at most 24 terms stay below 2^63
+        if ((++done & sc.fold_mask) == 0) fold();  // that many entries of the cross terms stay below 2^63
         if (lg == 0) {
             const M2LEntry en = lst[e];
             const int64_t s = source(en, px, py, act);
             if (s >= 0) {
-                const double S = t.S[s];
-                a0 = fma(S, t.lnTau[en.op], a0);
-                sumS += S;
+                a0 = fma(t.S[s], t.lnTau[en.op] + lnS, a0);
             }
         }
     }
@@ -601,37 +622,37 @@ __global__ void __launch_bounds__(512, 1) k_m2l64(Tree<double> t, F64Scales sc, 
         o[64] = h3[i] - h1[i] - h2[i];
         o[96] = m3[i] - m1[i] - m2[i];
     }
-    if (lg == 0) {
-        redS[(eg * 2) * 32 + lane] = a0;
-        redS[(eg * 2 + 1) * 32 + lane] = sumS;
-    }
+    if (lg == 0) redS[eg * 32 + lane] = a0;
     if (cs > 1) cluster_sync_all();
     else __syncthreads();
     for (int ll = int(rank) + cs * warp; ll < P1; ll += 16 * cs) {
-        long long v[4] = {0, 0, 0, 0};
+        long long v[4] = {0, 0, 0, 0}, w[2] = {0, 0};  // w: the upper sums' low 16 bits (a group's may fill 64)
         for (int r = 0; r < cs; ++r) {
 #pragma unroll
             for (int g = 0; g < 4; ++g) {
                 const long long* o = red + ((size_t(g) * 4 * NL + ll) * 4) * 32 + lane;
 #pragma unroll
-                for (int u = 0; u < 4; ++u) v[u] += r == int(rank) ? o[32 * u] : ld_peer64(o + 32 * u, r);
+                for (int u = 0; u < 4; ++u) {
+                    const long long x = r == int(rank) ? o[32 * u] : ld_peer64(o + 32 * u, r);
+                    v[u] += u & 1 ? x : x >> 16;
+                    if (!(u & 1)) w[u >> 1] += x & 0xffff;
+                }
             }
         }
-        // units: 2^(E - 52) 2^-wbits 2^el(l)
-        const int s = E - 52 - sc.wbits + sc.el[ll];
-        double re = fma(double(v[0]), pow2(56 + s), double(v[1]) * pow2(28 + s));
-        double im = fma(double(v[2]), pow2(56 + s), double(v[3]) * pow2(28 + s));
+        // units: 2^(E - kM2LBits) 2^-wbits 2^el(l)
+        const int s = E - kM2LBits - sc.wbits + sc.el[ll];
+        double re = fma(double(v[0]), pow2(72 + s), double((w[0] << 28) + v[1]) * pow2(28 + s));
+        double im = fma(double(v[2]), pow2(72 + s), double((w[1] << 28) + v[3]) * pow2(28 + s));
         if (bad) re = im = __longlong_as_double(0x7ff8000000000000ll);
         if (ll == 0) {
-            double A = 0.0, B = 0.0;
+            double A = 0.0;
             for (int r = 0; r < cs; ++r)
 #pragma unroll
                 for (int g = 0; g < 4; ++g) {
-                    const double* o = redS + (g * 2) * 32 + lane;
-                    A += r == int(rank) ? o[0] : __longlong_as_double(ld_peer64(o, r));
-                    B += r == int(rank) ? o[32] : __longlong_as_double(ld_peer64(o + 32, r));
+                    const double* o = redS + g * 32 + lane;
+                    A += r == int(rank) ? *o : __longlong_as_double(ld_peer64(o, r));
                 }
-            re += fma(fma(double(-l), 0.69314718055994530941723212145818, sc.ln_root), B, A);
+            re += A;
             im = 0.0;
         }
         if (act) {
@@ -797,7 +818,7 @@ __global__ void __launch_bounds__(32 * kDown64Warps) k_down64(Tree<double> t, do
         __syncthreads();
     }
     if (!p_out) return;
-    // leaves transposed (lane = leaf), and their constants: Re b_0 plus log h times the near monopoles
+    // leaves transposed (lane = leaf), and their constants: Re b_0 plus near_ln times the near monopoles
     constexpr int lb = kBoxes - kLeaves, LS = kLeaves + 1;
     for (int i = tid; i < kLeaves * P1; i += kThreads) {
         const int lf = i / P1, kk = i - lf * P1;
@@ -810,12 +831,12 @@ __global__ void __launch_bounds__(32 * kDown64Warps) k_down64(Tree<double> t, do
     for (int lf = tid; lf < kLeaves; lf += kThreads) {
         const int LX = X * TL + (lf & (TL - 1)), LY = Y * TL + lf / TL;
         double s = 0.0;
-        for (int e = 0; e < t.n_near; ++e) {
+        for (int e = 0; t.near_ln != 0.0 && e < t.n_near; ++e) {
             const int2 o = t.near[e];
             const int sx = LX + o.x, sy = LY + o.y;
             if (sx >= 0 && sy >= 0 && sx < side && sy < side) s += t.S[level_offset(t.Lleaf) + int64_t(sy) * side + sx];
         }
-        Lt[lf] = fma(t.lnh, s, L0s[lb + lf]);
+        Lt[lf] = fma(t.near_ln, s, L0s[lb + lf]);
     }
     __syncthreads();
     constexpr int kGroups = (kLeaves + 31) / 32;
@@ -825,7 +846,7 @@ __global__ void __launch_bounds__(32 * kDown64Warps) k_down64(Tree<double> t, do
         const int a = orbit_of(orb).x, b = orbit_of(orb).y;
         const double* L = Lt + (act ? lf : 0);
         const double2* V = Vs + orb * P1;  // w^l
-        double g1 = L[0], g2 = 0.0, h1 = 0.0, h2 = 0.0, e1 = 0.0, e2 = 0.0, f1 = 0.0, f2 = 0.0;
+        double g1 = 0.0, g2 = 0.0, h1 = 0.0, h2 = 0.0, e1 = 0.0, e2 = 0.0, f1 = 0.0, f2 = 0.0;
 #pragma unroll 1
         for (int l = 1; l < P1; l += 4) {
             const double2 v1 = V[l];
@@ -854,9 +875,10 @@ __global__ void __launch_bounds__(32 * kDown64Warps) k_down64(Tree<double> t, do
         }
         if (!act) continue;
         double* P = p_out + int64_t((Y * TL + lf / TL) * 8) * t.n + (X * TL + (lf & (TL - 1))) * 8;
+        // the constant meets the near field, which it mostly cancels, before the series does
         const auto put = [&](int x2, int y2, double v) {
             double* d = P + int64_t((y2 + 7) >> 1) * t.n + ((x2 + 7) >> 1);
-            *d = fma(v, kInv2Pi, *d);
+            *d = ((*d + L[0]) + v) * kInv2Pi;
         };
         {
             const double s = (g1 - g2) + (h1 - h2), d = (g1 - g2) - (h1 - h2), E = e1 - e2, F = f1 + f2;
@@ -879,10 +901,13 @@ bool f64_ok(int P1, int Lleaf) { return P1 <= f64::kMaxP && Lleaf >= 2; }
 size_t f64_counter_words(int Lleaf) { return 32 + size_t(level_offset(Lleaf - 1)); }
 
 // The multipole-to-local operators [op][k][l] (FP64 complex, row scaling as in k_m2l64) as fixed
-// point, in place of the FP64 values (16 bytes each either way).
-void f64_pack_m2l(double2* B, int n_ops, int P1, int max_entries, F64Scales* sc) {
-    sc->wbits = 54;
-    while (sc->wbits > 40 && std::ldexp(double(P1) * max_entries, sc->wbits) > std::ldexp(1.0, 64)) --sc->wbits;
+// point, in place of the FP64 values (16 bytes each either way).  wbits: the largest for which a row's sum
+// over an entry group (every fourth of the list, or fewer), sum (|Re| + |Im|) of its entries, times the
+// multipoles' 2^kM2LBits stays below 2^63 in units of 2^56, and the halves' sums below 2^31.  An entry's
+// cross terms are below P1 2^(kM2LBits + 1) + 2^wbits sum (|Re| + |Im|); fold_mask + 1 entries of them stay
+// below 2^63.
+void f64_pack_m2l(double2* B, int n_ops, int P1, const M2LEntry* il, const int* il_count, int il_stride, F64Scales* sc) {
+    const auto size = [](double2 b) { return std::fabs(b.x) + std::fabs(b.y); };
     double big[32] = {};  // largest scaled entry of each row
     for (int op = 0; op < n_ops; ++op)
         for (int k = 0; k < P1; ++k) {
@@ -891,6 +916,26 @@ void f64_pack_m2l(double2* B, int n_ops, int P1, int max_entries, F64Scales* sc)
             for (int l = 0; l < P1; ++l) big[l] = std::max(big[l], f * std::max(std::fabs(b[l].x), std::fabs(b[l].y)));
         }
     for (int l = 0; l < 32; ++l) sc->el[l] = l < P1 && big[l] > 0.0 ? std::ilogb(big[l]) + 1 : 0;
+    std::vector<double> row(size_t(n_ops) * P1, 0.0);  // an entry's sums, in units of the row's scale
+    double one = 0.0, all = 1.0;
+    for (int op = 0; op < n_ops; ++op)
+        for (int l = 0; l < P1; ++l) {
+            double& r = row[size_t(op) * P1 + l];
+            for (int k = 0; k < P1; ++k) r += size(B[(size_t(op) * P1 + k) * P1 + l]) * pow2(-(k >> 1) - sc->el[l]);
+            one = std::max(one, r);
+        }
+    for (int c = 0; c < 16; ++c)
+        for (int l = 0; l < P1; ++l) {
+            double s = 0.0;
+            for (int e = c >> 2; e < il_count[c & 3]; e += 4)
+                s += row[size_t(il[size_t(c & 3) * il_stride + e].op) * P1 + l];
+            all = std::max(all, s);
+        }
+    sc->wbits = 57;
+    while (std::ldexp(all, f64::kM2LBits + sc->wbits - 56) > 9.2e18) --sc->wbits;
+    const double cross = std::ldexp(double(P1), f64::kM2LBits + 1) + std::ldexp(one, sc->wbits);
+    sc->fold_mask = 3;
+    while (sc->fold_mask > 0 && cross * (sc->fold_mask + 1) > 9.2e18) sc->fold_mask >>= 1;
     for (int k = 0; k < P1; ++k)
         for (int l = 0; l < P1; ++l) {
             const double f = pow2(sc->wbits - (k >> 1) - sc->el[l]);
@@ -903,15 +948,25 @@ void f64_pack_m2l(double2* B, int n_ops, int P1, int max_entries, F64Scales* sc)
         }
 }
 
-// The near field's kernel table as a quadrant of fixed-point values: [|my|][|mx|], rows of R + 2.
-void f64_pack_near(double* K, int R) {
+// The near field's kernel table as a quadrant of fixed-point values: [|my|][|mx|], rows of R + 2; near_ln,
+// the part of log h that is not in it.  Log h in long double: its error would be the same in every entry.
+// The bits of weights (q) and values (k) by the table's largest value K: 128 terms of sum hh are below
+// 2^(q + k + 7 - 56) K and of the cross terms below 2^(q + 6) + 2^(k + 6) K; with 56 + 53 bits and K < 6 (h
+// above 1 / 140 where h < 1), 56 + 52 and K < 8, 55 + 52 and K < 16, both stay below 2^62.9.
+void f64_pack_near(double* K, int R, double h, double* near_ln, int* near_q, int* near_k) {
+    const long double lnh = std::log((long double)h);
+    const long double in = std::min(std::max(lnh, (long double)-f64::kNearLn), (long double)f64::kNearLn);
+    const auto value = [in](int x, int y) {
+        return in + (x + y == 0 ? 0.78539816339744830962L - 1.5L - 0.34657359027997265471L
+                                : (long double)(0.5 * std::log(double(x * x + y * y))));
+    };
+    const long double big = std::max(std::fabs(value(0, 0)), std::fabs(value(R + 1, R + 1)));
+    *near_ln = double(lnh - in);
+    *near_q = big < 8.0L ? 56 : 55;
+    *near_k = big < 6.0L ? 53 : 52;
     int2* o = reinterpret_cast<int2*>(K);
     for (int y = 0; y <= R; ++y)
-        for (int x = 0; x <= R + 1; ++x) {
-            const double r = std::sqrt(double(x * x + y * y));
-            const double v = x + y == 0 ? 0.78539816339744830962 - 1.5 - 0.34657359027997265471 : std::log(r);
-            o[size_t(y) * (R + 2) + x] = split28(std::llrint(std::ldexp(v, 52)));
-        }
+        for (int x = 0; x <= R + 1; ++x) o[size_t(y) * (R + 2) + x] = split28(std::llrint(std::ldexp(value(x, y), *near_k)));
 }
 
 cudaError_t launch_rhs64(const Tree<double>& t, const double* u, const double* v, const double* chi, const double* usx,
