@@ -46,6 +46,7 @@ constexpr int kTP = 32;  // stride (coefficients) of the expansion arrays and of
 constexpr double kInv2PiA = 0.15915494309189533576888376337251;
 constexpr double kC0A = 0.78539816339744830962 - 1.5 - 0.34657359027997265471;  // pi/4 - 3/2 - ln2/2
 constexpr double kLn2A = 0.69314718055994530941723212145818;
+constexpr double kLn2Lo = 2.319046813846299558417771e-17;  // log 2 - kLn2A
 
 struct AGeo {
     double cx, cy, s;     // centre and side
@@ -108,11 +109,12 @@ constexpr int kMaxOddSide = 192;  // its largest side
 // G_r[j] = sum_q i^(m(q) r) M_j of child q the four shifts are one real product,
 //   M_k = zeta_3^k [G_k[0] / k + sum_j C(k-1, j-1) (2 zeta_3)^-j G_(k-j)[j]]
 // (indices of G mod 4, G[0] from the monopoles): 76 FP64 instructions a parent instead of 192.
-// FP64 solves also write each leaf's weights in fixed point for the near field: v = q 2^(54-e)
+// FP64 solves also write each leaf's weights in fixed point for the near field: v = q 2^(kNearBitsA - e)
 // rounded, e the leaf's exponent (|q| < 2^e), kBadExp for a leaf with a non-finite weight.
 // ------------------------------------------------------------------------------------
 // Mixed solves copy theirs (q need not be aligned for the near field's 16-byte reads).
 constexpr int kBadExp = INT_MAX;
+constexpr int kNearBitsA = 56, kNearLogBitsA = 53;
 
 template <typename T>
 struct NearSrc {
@@ -151,7 +153,7 @@ __global__ void __launch_bounds__(128) k_aup(int nleaf, const int* __restrict__ 
         for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
         int e = -900;
         if (!bad && m > 0.0) e = max(ilogb(m) + 1, -900);
-        const double f = __hiloint2double((1023 + 54 - (bad ? 0 : e)) << 20, 0);  // 2^(54 - e)
+        const double f = __hiloint2double((1023 + kNearBitsA - (bad ? 0 : e)) << 20, 0);  // 2^(kNearBitsA - e)
         qfix[int64_t(leaf) * 64 + k] = bad ? 0 : __double2ll_rn(q0 * f);
         qfix[int64_t(leaf) * 64 + 32 + k] = bad ? 0 : __double2ll_rn(q1 * f);
         if (k == 0) qexp[leaf] = bad ? kBadExp : e;
@@ -361,10 +363,10 @@ __global__ void __launch_bounds__(64 * M2LUnits<T>::value) k_am2l(const int* __r
 // cell pairs need 15 (same level) or 22 (kappa 1) kernel values, kept in registers.  Before, each
 // pair took its own table read, and pairs of different levels a square root and a logarithm.
 //
-// FP64 runs the cell pairs in fixed point on the integer pipe (pp_fixed.cuh).  Source weights are
-// 55-bit integers (relative to the largest exponent et of the target's sources), kernel values
-// 56-bit integers (2^-52 units, |log| < 8); 32 source leaves a thread are summed before they are
-// added to the FP64 sum.
+// FP64 runs the cell pairs in fixed point on the integer pipe (pp_fixed.cuh), each product exact.  Source
+// weights are 57-bit integers (relative to the largest exponent et of the target's sources), kernel
+// values 57-bit integers (2^-53 units, |log| < 6.3); 16 source leaves a thread are summed before they
+// are added to the FP64 sum.
 // ------------------------------------------------------------------------------------
 template <typename T>
 struct NearAcc;
@@ -402,13 +404,13 @@ struct NearAcc<float> {
 template <>
 struct NearAcc<double> {
     typedef int2 Kv;  // (high, low) halves
-    long long hh[8], mid[8];
+    pp::FixedSum sum[8];
     double acc[8];
-    int qh[8], ql[8];
+    int2 q[8];
     __device__ void init() {
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            hh[j] = mid[j] = 0;
+            sum[j].clear();
             acc[j] = 0.0;
         }
     }
@@ -421,27 +423,26 @@ struct NearAcc<double> {
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
                 if (sh > 0) v[u] = sh > 60 ? 0 : (v[u] + (1ll << (sh - 1))) >> sh;
-                const int2 h = pp::split28(v[u]);
-                qh[2 * i + u] = h.x;
-                ql[2 * i + u] = h.y;
+                q[2 * i + u] = pp::split28(v[u]);
             }
         }
     }
-    __device__ __forceinline__ void add(int j, int r, int2 k) {
-        mad_wide(hh[j], qh[r], k.x);
-        mad_wide(mid[j], qh[r], k.y);
-        mad_wide(mid[j], ql[r], k.x);
-    }
+    __device__ __forceinline__ void add(int j, int r, int2 k) { sum[j].add(q[r], q[r].x + q[r].y, k, k.x + k.y); }
+    // units: 2^(et - kNearBitsA - kNearLogBitsA)
     __device__ void drain(int et) {
-        const double f1 = __hiloint2double((1023 + et - 50) << 20, 0), f2 = f1 * 3.7252902984619140625e-09;  // 2^-28
+        const double f1 = __hiloint2double((1023 + et + 56 - kNearBitsA - kNearLogBitsA) << 20, 0);
+        const double f2 = f1 * 3.7252902984619140625e-09;  // 2^-28
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            acc[j] = fma(double(hh[j]), f1, fma(double(mid[j]), f2, acc[j]));
-            hh[j] = mid[j] = 0;
+            long long hi;
+            int lo;
+            sum[j].digits(hi, lo);
+            acc[j] = fma(double(hi), f1, fma(double(lo), f2, acc[j]));
+            sum[j].clear();
         }
     }
     __device__ void leaf_done(int n, int et) {
-        if ((n & 31) == 31) drain(et);
+        if ((n & 15) == 15) drain(et);  // 128 terms, |log| < 6.3: sum hh below 2^62.7, cross terms below 2^62.9
     }
     __device__ void finish(int et) { drain(et); }
 };
@@ -504,26 +505,47 @@ k_aleaf(const int* __restrict__ leafbox, const int* __restrict__ anc, int nlev, 
                     const Kv* kr = tab + abs(pr.oy + sy - ty) * W;
                     Kv kc[15];
 #pragma unroll
-                    for (int m = 0; m < 15; ++m) kc[m] = kr[abs(pr.ox - 7 + m)];
+                    for (int m = 0; m < 7; ++m) kc[m] = kr[abs(pr.ox - 7 + m)];
 #pragma unroll
-                    for (int r = 0; r < 8; ++r)
+                    for (int r = 0; r < 8; ++r) {
+                        kc[r + 7] = kr[abs(pr.ox + r)];
 #pragma unroll
                         for (int j = 0; j < 8; ++j) A.add(j, r, kc[r - j + 7]);
+                    }
                 } else {
                     const int kap = abs(pr.kind);
                     const int my = pr.kind < 0 ? pr.oy + (sy << kap) - ty : pr.oy + sy - (ty << kap);
                     const Kv* kr = to + (my ^ (my >> 31)) * Wo;
-                    if (kap == 1) {
+                    const auto kernel = [&](int m) { return __ldg(kr + (m ^ (m >> 31))); };
+                    if (kap == 1 && pr.kind < 0) {  // source column r, target column j: kc[2 r - j + 7]
                         Kv kc[22];
-                        const int m0 = pr.kind < 0 ? pr.ox - 7 : pr.ox - 14;
 #pragma unroll
-                        for (int m = 0; m < 22; ++m) kc[m] = __ldg(kr + ((m0 + m) ^ ((m0 + m) >> 31)));
-                        if (pr.kind < 0) {
+                        for (int m = 0; m < 6; ++m) kc[m] = kernel(pr.ox - 7 + m);
 #pragma unroll
-                            for (int r = 0; r < 8; ++r)
+                        for (int r = 0; r < 8; ++r) {
+                            kc[2 * r + 6] = kernel(pr.ox - 1 + 2 * r);
+                            kc[2 * r + 7] = kernel(pr.ox + 2 * r);
 #pragma unroll
-                                for (int j = 0; j < 8; ++j) A.add(j, r, kc[2 * r - j + 7]);
+                            for (int j = 0; j < 8; ++j) A.add(j, r, kc[2 * r - j + 7]);
+                        }
+                    } else if (kap == 1) {  // kc[r - 2 j + 14]
+                        if constexpr (sizeof(T) == 8) {  // even columns, then odd ones: half the values at once
+#pragma unroll
+                            for (int u = 0; u < 2; ++u) {
+                                Kv kc[11];
+#pragma unroll
+                                for (int m = 0; m < 7; ++m) kc[m] = kernel(pr.ox - 14 + u + 2 * m);
+#pragma unroll
+                                for (int i = 0; i < 4; ++i) {
+                                    kc[i + 7] = kernel(pr.ox + u + 2 * i);
+#pragma unroll
+                                    for (int j = 0; j < 8; ++j) A.add(j, 2 * i + u, kc[i - j + 7]);
+                                }
+                            }
                         } else {
+                            Kv kc[22];
+#pragma unroll
+                            for (int m = 0; m < 22; ++m) kc[m] = kernel(pr.ox - 14 + m);
 #pragma unroll
                             for (int r = 0; r < 8; ++r)
 #pragma unroll
@@ -612,19 +634,20 @@ k_aleaf(const int* __restrict__ leafbox, const int* __restrict__ anc, int nlev, 
             cur.y += m.y;
             c0 += m0;
         }
-        // log(unit) S over the near sources served from a table
+        // log(unit) S over the near sources served from a table, unit = 2^-u: log 2 enters once, to more than
+        // FP64's digits (the sums it multiplies cancel much of the table's)
         double sl = 0.0;
         for (int e = e0 + lane; e < e1; e += 32) {
             const APair pr = pairs[e];
             bool direct = pr.kind == kDirect;
             if constexpr (sizeof(T) == 8) direct = direct || qexp[pr.src] == kBadExp;
             const int unit = pr.kind == 0 ? lev + 3 : lev + 4 + max(pr.kind, 0);
-            if (!direct) sl += S[leafbox[pr.src]] * (-kLn2A * unit);
+            if (!direct) sl = fma(S[leafbox[pr.src]], double(unit), sl);
         }
         for (int o = 16; o > 0; o >>= 1) sl += __shfl_xor_sync(0xffffffffu, sl, o);
         __syncwarp();
         Ls[lane] = cur;
-        if (lane == 0) c0s = c0 + sl;
+        if (lane == 0) c0s = fma(-kLn2A, sl, fma(-kLn2Lo, sl, c0));
     }
     __syncthreads();
     if (tid < 64) {
@@ -987,9 +1010,7 @@ AConst<T>* fill_const() {
 void put_log(double& d, double v) { d = v; }
 void put_log(float2& d, double v) { d = make_float2(float(v), float(v - double(float(v)))); }
 void put_kernel(float& d, double v) { d = float(v); }
-void put_kernel(int2& d, double v) {  // 2^-52 units as h 2^28 + l, |l| <= 2^27
-    d = pp::split28(std::llrint(std::ldexp(v, 52)));
-}
+void put_kernel(int2& d, double v) { d = pp::split28(std::llrint(std::ldexp(v, kNearLogBitsA))); }
 
 template <typename T>
 cudaError_t setup_side(AdaptiveState* s, AdaptiveSide<T>& d, cudaStream_t st) {

@@ -1,9 +1,12 @@
-"""Rounding of the FP64 path, without the truncation that hides it elsewhere: plans against the same
-multipole sum (lists, order, truncation) in long double.
+"""Rounding of the FP64 paths, without the truncation that hides it elsewhere: plans against the same
+multipole sum (lists, order, truncation) in long double, adaptive solves at an acceptance and order whose
+truncation (0.25^31) is below rounding against the direct sum in long double.
 
-Allowed: 10 units (2^-53) of the field in l2.  A value is the sum of a constant, a far and a near part, each
+Allowed for plans: 10 units (2^-53) of the field in l2.  A value is the sum of a constant, a far and a near part, each
 up to a few times the field and each rounded once or twice at its own size, and of sums of some hundred
-terms whose roundings add up to a few units more.  The fields cover what weights relative to a
+terms whose roundings add up to a few units more.  Allowed for adaptive solves, where the terms of some
+fields cancel to a hundredth of their size: the error of the direct sum in FP64, term after term.
+The fields cover what weights relative to a
 common exponent could lose: smooth ones, a wall of large weights in small ones, a violent patch, halves of
 very different size, and noise.
 """
@@ -71,6 +74,34 @@ def test_plan(n, order, theta, kind):
     print(f"{kind} n {n} p {order} theta {theta}: {e / 2 ** -53:.1f} units (far {e_far / 2 ** -53:.1f}, near {e_near / 2 ** -53:.1f})")
     assert e <= ALLOWED and e_far <= ALLOWED and e_near <= ALLOWED
     plan.destroy()
+
+
+@pytest.mark.parametrize("kind", ["noise", "patch", "smooth", "levels"])
+@pytest.mark.parametrize("levels", [(2, 4), (1, 5)])
+def test_adaptive(levels, kind):
+    lv, ix, iy = synth.adaptive_blocks(*levels, centre=(0.4, 0.5), radius=0.1, band=2.0)
+    xs, ys, hs = synth.block_cells(lv, ix, iy)
+    rng = np.random.default_rng(len(lv))
+    q = rng.normal(size=xs.size)
+    if kind == "smooth":
+        q = np.exp(-((xs - 0.4) ** 2 + (ys - 0.5) ** 2) / 0.02)
+    if kind != "levels":  # else weights of one size on cells of all sizes
+        q *= hs ** 2
+    if kind == "patch":
+        q[np.hypot(xs - 0.45, ys - 0.5) < 0.03] *= 1e6
+    tree = api.AdaptiveTree(lv, ix, iy, theta=0.25)
+    P = torch.empty(q.size, dtype=torch.float64, device="cuda")
+    tree.solve(torch.tensor(q, device="cuda"), 30, P)
+    at = np.sort(rng.choice(q.size, 200, replace=False))
+    X, Y, Q = (a.astype(ref.LD) for a in (xs, ys, q))
+    rho = np.exp(ref.C0) * hs.astype(ref.LD)
+    r2 = np.maximum((X[at, None] - X) ** 2 + (Y[at, None] - Y) ** 2, rho ** 2)
+    K, two_pi = np.log(r2) / 2, 8 * np.arctan(ref.LD(1))
+    want = K @ Q / two_pi
+    plain = np.add.accumulate(K.astype(np.float64) * q, axis=1)[:, -1] / two_pi
+    e, allowed = rel(P.cpu().numpy()[at], want), rel(plain, want)
+    print(f"{kind} levels {levels} ({len(lv)} leaves): {e / 2 ** -53:.1f} units, allowed {allowed / 2 ** -53:.1f}")
+    assert e <= allowed
 
 
 @pytest.mark.parametrize("h", [1e-9, 3.7, 1e8])
