@@ -395,10 +395,17 @@ struct NearAcc<float> {
             part[j] = 0.f;
         }
     }
-    __device__ void finish(int) {
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[j] -= comp[j];
+    __device__ void finish(int) {}
+    typedef float2 Out;  // a double-float pair
+    __device__ __forceinline__ Out out(int j) const { return make_float2(acc[j], -comp[j]); }
+    __device__ static __forceinline__ Out add(Out a, Out b) {
+        df_add(a.x, a.y, b.x, b.y);
+        return a;
     }
+    __device__ static __forceinline__ Out shfl(Out a, int o) {
+        return make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
+    }
+    __device__ static __forceinline__ double value(Out a) { return df_to(a.x, a.y); }
 };
 
 template <>
@@ -445,6 +452,19 @@ struct NearAcc<double> {
         if ((n & 15) == 15) drain(et);  // 128 terms, |log| < 6.3: sum hh below 2^62.7, cross terms below 2^62.9
     }
     __device__ void finish(int et) { drain(et); }
+    typedef double Out;
+    __device__ __forceinline__ Out out(int j) const { return acc[j]; }
+    __device__ static __forceinline__ Out add(Out a, Out b) { return a + b; }
+    __device__ static __forceinline__ Out shfl(Out a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+    __device__ static __forceinline__ double value(Out a) { return a; }
+};
+
+// Mixed solves take the table's offsets in units of 2^same cells (2^odd half cells), so that its values are
+// small and their FP32 sums do not cancel against log(unit) S (noise on cells of five sizes, p = 20, theta =
+// 0.5: relative l2 error 2.7e-7, in cells 3.8e-7).
+template <typename T>
+struct NearUnit {
+    static constexpr int same = sizeof(T) == 4 ? 3 : 0, odd = sizeof(T) == 4 ? 5 : 0;
 };
 
 // Pairs of near-field warps per CTA, and the path's warp: FP64 needs 128 registers a thread, and
@@ -468,7 +488,7 @@ k_aleaf(const int* __restrict__ leafbox, const int* __restrict__ anc, int nlev, 
     extern __shared__ __align__(16) unsigned char smem_leaf[];
     Kv* tab = reinterpret_cast<Kv*>(smem_leaf);  // (R + 1) rows of stride R + 2
     constexpr int kGroups = LeafCta<T>::groups;
-    __shared__ T near[kGroups][64];
+    __shared__ typename NearAcc<T>::Out near[kGroups][64];
     __shared__ C Ls[kTP];
     __shared__ double c0s;
     const int i = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -596,14 +616,18 @@ k_aleaf(const int* __restrict__ leafbox, const int* __restrict__ anc, int nlev, 
             A.leaf_done(n++, et);
         }
         A.finish(et);
+        // the eight source rows are lanes of one target row: a lane ends with one target's sum
+        typename NearAcc<T>::Out v[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {  // the eight source rows (lanes of one target row), then one lane a target
-            T v = A.acc[j];
-            v += __shfl_xor_sync(0xffffffffu, v, 1);
-            v += __shfl_xor_sync(0xffffffffu, v, 2);
-            v += __shfl_xor_sync(0xffffffffu, v, 4);
-            if (sy == j) near[g][ty * 8 + j] = v;
-        }
+        for (int j = 0; j < 8; ++j) v[j] = A.out(j);
+#pragma unroll
+        for (int o = 4; o >= 1; o >>= 1)
+#pragma unroll
+            for (int j = 0; j < o; ++j) {
+                const bool up = (sy & o) != 0;
+                v[j] = NearAcc<T>::add(up ? v[j + o] : v[j], NearAcc<T>::shfl(up ? v[j] : v[j + o], o));
+            }
+        near[g][ty * 8 + sy] = v[0];
     } else {
         // the path's locals: cur is this lane's coefficient of the box above
         const int lev = geo[b].level;
@@ -641,7 +665,7 @@ k_aleaf(const int* __restrict__ leafbox, const int* __restrict__ anc, int nlev, 
             const APair pr = pairs[e];
             bool direct = pr.kind == kDirect;
             if constexpr (sizeof(T) == 8) direct = direct || qexp[pr.src] == kBadExp;
-            const int unit = pr.kind == 0 ? lev + 3 : lev + 4 + max(pr.kind, 0);
+            const int unit = pr.kind == 0 ? lev + 3 - NearUnit<T>::same : lev + 4 + max(pr.kind, 0) - NearUnit<T>::odd;
             if (!direct) sl = fma(S[leafbox[pr.src]], double(unit), sl);
         }
         for (int o = 16; o > 0; o >>= 1) sl += __shfl_xor_sync(0xffffffffu, sl, o);
@@ -657,9 +681,9 @@ k_aleaf(const int* __restrict__ leafbox, const int* __restrict__ anc, int nlev, 
             const C v = ct->V[l][tid], m = Ls[l];
             ser = fma(m.x, v.x, fma(-m.y, v.y, ser));
         }
-        T nr = near[0][tid] + near[1][tid];
-        if constexpr (kGroups == 4) nr += near[2][tid] + near[3][tid];
-        p_out[int64_t(i) * 64 + tid] = T((c0s + double(ser) + double(nr)) * kInv2PiA);
+        typename NearAcc<T>::Out nr = NearAcc<T>::add(near[0][tid], near[1][tid]);
+        if constexpr (kGroups == 4) nr = NearAcc<T>::add(nr, NearAcc<T>::add(near[2][tid], near[3][tid]));
+        p_out[int64_t(i) * 64 + tid] = T((c0s + double(ser) + NearAcc<T>::value(nr)) * kInv2PiA);
     }
 }
 
@@ -1039,10 +1063,12 @@ cudaError_t setup_side(AdaptiveState* s, AdaptiveSide<T>& d, cudaStream_t st) {
         std::vector<typename NearAcc<T>::Kv> te(size_t(a.R + 1) * (a.R + 2)), to(size_t(a.Wo) * a.Wo);
         for (int y = 0; y <= a.R; ++y)
             for (int x = 0; x <= a.R; ++x)
-                put_kernel(te[size_t(y) * (a.R + 2) + x], x + y == 0 ? kC0A : 0.5 * std::log(double(x * x + y * y)));
+                put_kernel(te[size_t(y) * (a.R + 2) + x],
+                           (x + y == 0 ? kC0A : 0.5 * std::log(double(x * x + y * y))) - NearUnit<T>::same * kLn2A);
         for (int y = 0; y < a.Wo; ++y)
             for (int x = 0; x <= y; ++x) {
-                const double v = 0.5 * std::log(double((2 * x + 1) * (2 * x + 1) + (2 * y + 1) * (2 * y + 1)));
+                const double v = 0.5 * std::log(double((2 * x + 1) * (2 * x + 1) + (2 * y + 1) * (2 * y + 1))) -
+                                 NearUnit<T>::odd * kLn2A;
                 put_kernel(to[size_t(y) * a.Wo + x], v);
                 put_kernel(to[size_t(x) * a.Wo + y], v);
             }
