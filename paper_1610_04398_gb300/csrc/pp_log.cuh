@@ -6,7 +6,7 @@
 // most 2^-8), and with e + 1 and 2 c in place of e and c where m is above 1 + 106/256 (about sqrt 2)
 //   log x = e log 2 - log c + (r - r^2/2 + ... + r^7/7)   (truncation below 2^-67):
 // ten FP64 instructions.  c is exact and |log c| at most 0.35, so the result keeps its relative accuracy
-// around 1: within 1.6 units in the last place.
+// around 1: within 1.4 units in the last place.
 // Subnormal, infinite, NaN and non-positive arguments take the library's log.
 #pragma once
 
@@ -50,7 +50,8 @@ __device__ __forceinline__ double log_table(double x) {
     s = fma(r, s, 1.0 / 3.0);
     s = fma(r, s, -0.5);
     s = fma(r * r, s, r);
-    return fma(e, 0.69314718055994530941723212145818, __ldg(&g_log_table.lc[i])) + s;
+    // the small terms first: one rounding at the size of the result
+    return fma(e, 0.69314718055994530941723212145818, __ldg(&g_log_table.lc[i]) + s);
 }
 
 }  // namespace pp

@@ -1,8 +1,9 @@
 """The table logarithm of the FP64 tree walks against CUDA's log, over the whole range of normal numbers
 and around 1, and the arguments that it hands to the library.
 
-Tolerance: two units in the last place: half a unit from each of the table's two additions, a quarter from
-log 2 rounded, and what the library's own result (documented: one unit) is off.
+Tolerance: two units in the last place: half a unit from the table's last addition, a quarter from log 2
+rounded, a quarter from the table and the series, and what the library's own result (documented: one unit)
+is off.
 """
 import ctypes
 import os
