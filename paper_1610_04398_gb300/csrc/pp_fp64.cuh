@@ -151,7 +151,8 @@ __device__ __forceinline__ void p2m_class(const double* qs, const double2* W, in
     for (int i = 0; i < KN; ++i) M[i] = double2{0.0, 0.0};
     S = 0.0;
 #pragma unroll 1
-    for (int a = 1; a <= 7; a += 2)
+    for (int a = 1; a <= 7; a += 2) {
+        double Sa = 0.0;  // the sum in blocks: fewer roundings at its full size
 #pragma unroll 1
         for (int b = 1; b <= a; b += 2, W += P1) {
             const double q0 = qs[cell_at(a, b)], q1 = qs[cell_at(-b, a)], q2 = qs[cell_at(-a, -b)], q3 = qs[cell_at(b, -a)];
@@ -166,7 +167,7 @@ __device__ __forceinline__ void p2m_class(const double* qs, const double2* W, in
                 for (int i = 0; i < KN; ++i) {
                     const int k = 4 * i + R;
                     if (k == 0) {
-                        S += A;
+                        Sa += A;
                     } else if (k < P1) {
                         const double2 z = w[k];
                         M[i].x = fma(A, z.x, M[i].x);
@@ -188,6 +189,8 @@ __device__ __forceinline__ void p2m_class(const double* qs, const double2* W, in
                 }
             }
         }
+        S += Sa;
+    }
 }
 
 template <int R, int KN>
