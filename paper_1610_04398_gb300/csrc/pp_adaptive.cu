@@ -698,7 +698,7 @@ k_aleaf(const int* __restrict__ leafbox, const int* __restrict__ anc, int nlev, 
 // within s / (sqrt 2 theta) of the point: at most 37 for theta >= 0.25, 148 children.
 constexpr int kSurfCand = 256;
 
-__global__ void __launch_bounds__(128) k_asurf(int npts, const double* __restrict__ pts, const AGeo* __restrict__ geo,
+__global__ void __launch_bounds__(128) k_asurf(int npts, int nb, const double* __restrict__ pts, const AGeo* __restrict__ geo,
                                                const int* __restrict__ fchild, const int* __restrict__ boxleaf, int p,
                                                const double* __restrict__ S, const double2* __restrict__ M,
                                                const double* __restrict__ q, double theta, double* __restrict__ P_out,
@@ -727,9 +727,24 @@ __global__ void __launch_bounds__(128) k_asurf(int npts, const double* __restric
         }
         acc = fma(S[b], 0.5 * pp::log_table(d2), acc) - (h.x * u.x - h.y * u.y);
     };
+    const auto direct = [&](int lb) {  // a leaf's 64 cells, two a lane
+        const AGeo g = geo[lb];
+        const double* qs = q + int64_t(boxleaf[lb]) * 64;
+        const double rho = g.s * rho8, rho2 = rho * rho;
+        const double2 c0 = cell_w(lane);
+        const double ex = zx - fma(g.s, c0.x, g.cx), ey = zy - fma(g.s, c0.y, g.cy), ey1 = ey - 0.5 * g.s;
+        const double x2 = ex * ex;  // cells `lane` and `lane + 32`, four rows on
+        acc = fma(qs[lane], 0.5 * pp::log_table(fmax(fma(ey, ey, x2), rho2)), acc);
+        acc = fma(qs[lane + 32], 0.5 * pp::log_table(fmax(fma(ey1, ey1, x2), rho2)), acc);
+    };
     if (lane == 0) cand[w][0][0] = 0;
     __syncwarp();
     int cur = 0, n = 1, na = 0;
+    if (isnan(zx) || isnan(zy)) {  // accepts no box and is within every clamp (fmax): every leaf, beyond what a list holds
+        for (int b = 0; b < nb; ++b)
+            if (fchild[b] < 0) direct(b);
+        n = 0;
+    }
     while (n > 0) {
         int next = 0;
         for (int base = 0; base < n; base += 32) {
@@ -757,17 +772,8 @@ __global__ void __launch_bounds__(128) k_asurf(int npts, const double* __restric
                 acc_list[w][lane] = v;
                 __syncwarp();
             }
-            for (unsigned lm = __ballot_sync(0xffffffffu, leaf); lm; lm &= lm - 1) {
-                const int lb = __shfl_sync(0xffffffffu, b, __ffs(lm) - 1);
-                const AGeo g = geo[lb];
-                const double* qs = q + int64_t(boxleaf[lb]) * 64;
-                const double rho = g.s * rho8, rho2 = rho * rho;
-                const double2 c0 = cell_w(lane);
-                const double ex = zx - fma(g.s, c0.x, g.cx), ey = zy - fma(g.s, c0.y, g.cy), ey1 = ey - 0.5 * g.s;
-                const double x2 = ex * ex;  // cells `lane` and `lane + 32`, four rows on
-                acc = fma(qs[lane], 0.5 * pp::log_table(fmax(fma(ey, ey, x2), rho2)), acc);
-                acc = fma(qs[lane + 32], 0.5 * pp::log_table(fmax(fma(ey1, ey1, x2), rho2)), acc);
-            }
+            for (unsigned lm = __ballot_sync(0xffffffffu, leaf); lm; lm &= lm - 1)
+                direct(__shfl_sync(0xffffffffu, b, __ffs(lm) - 1));
             const unsigned im = __ballot_sync(0xffffffffu, inner);
             if (inner) {
                 const int at = next + 4 * __popc(im & below);
@@ -1179,7 +1185,7 @@ extern "C" int pp_atree_surface_pressure(pp_atree tree, const double* q, int npt
     if (!s || s->last_p < 1) return PP_ERR_STATE;  // the multipoles come from a solve
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (cudaMemsetAsync(s->d_err, 0, sizeof(int), st) != cudaSuccess) return PP_ERR_CUDA;
-    k_asurf<<<(npts + 3) / 4, 128, 0, st>>>(npts, points, s->d_geo, s->d_fchild, s->d_boxleaf, s->last_p, s->d_S,
+    k_asurf<<<(npts + 3) / 4, 128, 0, st>>>(npts, s->a.nb, points, s->d_geo, s->d_fchild, s->d_boxleaf, s->last_p, s->d_S,
                                                s->f64.M, q, theta, P_out, s->d_err);
     if (cudaGetLastError() != cudaSuccess) return PP_ERR_CUDA;
     int err = 0;

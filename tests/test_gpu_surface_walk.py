@@ -121,3 +121,24 @@ def test_captured_step_outlives_a_larger_call(precision):
     assert torch.equal(per, first[0]) and torch.equal(forces, first[1]) and torch.isnan(spoil).all()
     step.destroy()
     plan.destroy()
+
+
+def test_adaptive_walk_takes_nan_points():
+    """A point with a NaN coordinate accepts no box and lies within every cell's clamp: its value is sum q
+    log rho_h / (2 pi), the call succeeds and the other points are what they are without it."""
+    lv, ix, iy = synth.adaptive_blocks(3, 6, centre=(0.4, 0.5), radius=0.1, band=2.0)
+    _, _, hs = synth.block_cells(lv, ix, iy)
+    q = np.random.default_rng(0).normal(size=hs.size) * hs ** 2
+    tree = api.AdaptiveTree(lv, ix, iy, theta=0.5)
+    qd = to_dev(q, torch.float64)
+    tree.solve(qd, 12)
+    pts = synth.circle_surface(40, (0.4, 0.5), 0.1)[0]
+    clean = tree.surface_pressure(qd, to_dev(pts, torch.float64), 0.5).cpu().numpy()
+    bad = [3, 17]
+    pts[3, 0] = pts[17, 1] = np.nan
+    P = tree.surface_pressure(qd, to_dev(pts, torch.float64), 0.5).cpu().numpy()
+    keep = np.setdiff1d(np.arange(40), bad)
+    assert np.array_equal(P[keep], clean[keep])
+    terms = q * np.log(oracle.rho_h(1.0) * hs) / (2 * np.pi)
+    assert np.max(np.abs(P[bad] - terms.sum())) < 1e-14 * np.abs(terms).sum()
+    tree.destroy()
