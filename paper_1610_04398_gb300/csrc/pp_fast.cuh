@@ -1312,12 +1312,7 @@ __device__ __forceinline__ float m2m_parent(const Tree<T>& t, int l, int64_t b, 
 #pragma unroll
         for (int k = 1; k < P1; k += 2) {
             const float4 v = make_float4(Br[k], Bi[k], Br[k + 1], Bi[k + 1]);
-            if (l > 0) {
-                *out.pair(k) = v;
-            } else {  // the root's pairs are not aligned
-                out[k] = cmake<T>(v.x, v.y);
-                out[k + 1] = cmake<T>(v.z, v.w);
-            }
+            *out.pair(k) = v;
             if constexpr (kMax) mx = fmaxf(mx, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
         }
     }

@@ -99,30 +99,20 @@ __device__ __forceinline__ void surf_walk(const Tree<T>& t, const SurfaceArgs& a
         C h;
         if constexpr (P1T > 0 && sizeof(T) == 4) {
             static_assert(P1T % 2 == 1, "columns 1 .. P1 - 1 in pairs");
-            if (l > 0) {
 #pragma unroll
-                for (int k = P1T - 2; k >= 1; k -= 2) {
-                    const float4 m = *M.pair(k);  // coefficients k and k + 1
-                    if (k == P1T - 2) {
-                        h.x = m.z;
-                        h.y = m.w;
-                    } else {
-                        const T hr = fma(h.x, ux, fma(-h.y, uy, T(m.z)));
-                        h.y = fma(h.x, uy, fma(h.y, ux, T(m.w)));
-                        h.x = hr;
-                    }
-                    const T hr = fma(h.x, ux, fma(-h.y, uy, T(m.x)));
-                    h.y = fma(h.x, uy, fma(h.y, ux, T(m.y)));
+            for (int k = P1T - 2; k >= 1; k -= 2) {
+                const float4 m = *M.pair(k);  // coefficients k and k + 1
+                if (k == P1T - 2) {
+                    h.x = m.z;
+                    h.y = m.w;
+                } else {
+                    const T hr = fma(h.x, ux, fma(-h.y, uy, T(m.z)));
+                    h.y = fma(h.x, uy, fma(h.y, ux, T(m.w)));
                     h.x = hr;
                 }
-            } else {  // the root (its pairs are not aligned)
-                h = M[P1 - 1];
-                for (int k = P1 - 2; k >= 1; --k) {
-                    const C m = M[k];
-                    const T hr = fma(h.x, ux, fma(-h.y, uy, m.x));
-                    h.y = fma(h.x, uy, fma(h.y, ux, m.y));
-                    h.x = hr;
-                }
+                const T hr = fma(h.x, ux, fma(-h.y, uy, T(m.x)));
+                h.y = fma(h.x, uy, fma(h.y, ux, T(m.y)));
+                h.x = hr;
             }
         } else {
             h = M[P1 - 1];
