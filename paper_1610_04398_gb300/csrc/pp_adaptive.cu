@@ -101,8 +101,8 @@ constexpr int kMaxOddSide = 192;  // its largest side
 
 // ------------------------------------------------------------------------------------
 // Upward pass, one warp per leaf: the leaf's multipole from the table of w^k / k (lane k
-// forms M_k), then up the tree: the warp that arrives last at a parent (an arrival counter it
-// resets; no warp waits) shifts the four children, whichever warp that is: the arithmetic and
+// forms M_k), then up the tree: the warp that arrives last at a parent (an arrival counter, cleared by
+// k_am2l for the next solve; no warp waits) shifts the four children, whichever warp that is: the arithmetic and
 // its order do not depend on it.  One launch in place of one per level: 0.24 ms (FP64) and 21 us
 // (mixed) a level for 1629 boxes before, most of it latency and powers formed per lane.
 // The children's zeta are 90 degree rotations of each other, zeta_q = i^m(q) zeta_3, so with
@@ -186,7 +186,6 @@ __global__ void __launch_bounds__(128) k_aup(int nleaf, const int* __restrict__ 
         if (k == 0) arrived = atomicAdd(cnt + pa, 1u);
         if (__shfl_sync(0xffffffffu, arrived, 0) != 3u) return;
         __threadfence();  // the other children's after it
-        if (k == 0) cnt[pa] = 0u;
         b = pa;
         const int fc = first_child[b];
         C m[4];
@@ -264,7 +263,8 @@ __global__ void __launch_bounds__(64 * M2LUnits<T>::value) k_am2l(const int* __r
                                               const AConst<T>* __restrict__ ct, const double* __restrict__ S,
                                               const float2* __restrict__ Sf,
                                               const typename cplx_of<T>::type* __restrict__ M,
-                                              typename cplx_of<T>::type* __restrict__ L, double* __restrict__ L0) {
+                                              typename cplx_of<T>::type* __restrict__ L, double* __restrict__ L0,
+                                              unsigned* __restrict__ cnt) {
     typedef typename cplx_of<T>::type C;
     constexpr int kUnits = M2LUnits<T>::value, kThreads = 64 * kUnits;
     __shared__ T R[kTP][kTP];
@@ -273,6 +273,7 @@ __global__ void __launch_bounds__(64 * M2LUnits<T>::value) k_am2l(const int* __r
     __shared__ float4 red0[sizeof(T) == 4 ? kThreads : 1];  // mixed: constant term and sum of S, pairs
     const int a = blockIdx.x, tid = threadIdx.x, unit = tid >> 6;
     const int e0 = ptr[a], e1 = ptr[a + 1];
+    if (tid == 0) cnt[a] = 0u;  // the upward pass's arrivals
     if (e0 == e1) {  // no sources (block-uniform)
         if (tid <= p) L[int64_t(a) * kTP + tid] = cx<T>(T(0), T(0));
         if (tid == 0) L0[a] = 0.0;
@@ -979,7 +980,7 @@ struct AdaptiveState {
         *d_anc = nullptr, *d_boxleaf = nullptr, *d_err = nullptr, *d_qexp = nullptr;
     int2* d_mpair = nullptr;
     APair* d_ppair = nullptr;
-    unsigned* d_cnt = nullptr;  // arrivals per box, zero between solves
+    unsigned* d_cnt = nullptr;  // arrivals per box, zero when a solve starts
     AGeo* d_geo = nullptr;
     double *d_S = nullptr, *d_L0 = nullptr;
     float2* d_Sf = nullptr;
@@ -1147,7 +1148,7 @@ int solve_adaptive(AdaptiveState* s, const AdaptiveSide<T>& d, int p, const T* q
     k_aup<T><<<(a.nleaf + 3) / 4, 128, 0, st>>>(a.nleaf, s->d_leafbox, s->d_parent, s->d_fchild, q, p, d.ct, s->d_S,
                                                s->d_Sf, d.M, s->d_cnt, qs, s->d_qexp);
     k_am2l<T><<<a.nb, 64 * M2LUnits<T>::value, 0, st>>>(s->d_mptr, s->d_mpair, s->d_geo, d.oplog, d.op, p, d.ct, s->d_S, s->d_Sf, d.M,
-                                    d.L, s->d_L0);
+                                    d.L, s->d_L0, s->d_cnt);
     const size_t smem = sizeof(typename NearAcc<T>::Kv) * size_t(a.R + 1) * (a.R + 2);
     k_aleaf<T><<<a.nleaf, LeafCta<T>::threads, smem, st>>>(s->d_leafbox, s->d_anc, a.L + 1, s->d_pptr, s->d_ppair, s->d_geo,
                                                     p, d.ct, d.L, s->d_L0, d.te, a.R, d.to, a.Wo, s->d_S, q,

@@ -231,6 +231,7 @@ pp::Tree<T> make_tree(const pp_plan p) {
     t.P1 = p->P1;
     t.h = p->h;
     t.lnh = std::log(p->h);
+    t.surf_counter = reinterpret_cast<unsigned*>(p->forces_dev + 6);
     t.near_ln = p->near_ln;
     t.near_q = p->near_q;
     t.near_k = p->near_k;
@@ -903,7 +904,6 @@ int run_surface(pp_plan p, const void* u, const void* v, int npts, const double*
     a.nrm = nrm;
     a.dS = dS;
     a.Psurf = p->Psurf;
-    a.counter = reinterpret_cast<unsigned*>(p->forces_dev + 6);
     a.per_point = per_point;
     a.partial = nullptr;
     a.forces = dev_forces ? forces : p->forces_dev;

@@ -80,6 +80,7 @@ struct Tree {
     int ig_groups[4];      // the groups of two to four first,
     int ig_count[4];       // then the single sources
     const T* Ktab;         // [(2 Rk + 1)^2]: log max(h |Delta|, rho_h) for integer cell offsets
+    unsigned* surf_counter;  // the surface pass's arrivals: cleared by its last CTA and by every source kernel
     double near_ln;        // fixed-point FP64 plans: the part of log h that is not in the near-field table,
     int near_q, near_k;    // and the bits of its weights and kernel values
     const T* Krel;         // same offsets, log max(|Delta|, rho_h / h) = Ktab - log h (split solve: the
@@ -273,7 +274,6 @@ struct SurfaceArgs {
     const double* nrm;
     const double* dS;      // may be null: trapezoid weights
     double* Psurf;         // k_traction: [npts] pressure at the points; k_surface: the CTAs' partial sums
-    unsigned* counter;     // k_surface: arrivals, zero between calls
     double* per_point;     // [npts][5] or null
     double* partial;       // [blocks][4]
     double* forces;        // [6] device

@@ -523,6 +523,7 @@ __global__ void __launch_bounds__(32 * kRhsWarps, (P1 <= 17 ? 16 : 8) / kRhsWarp
     const int strips = (n + 127) >> 7;
     const int LY0 = int(wid / strips) * kRows, sxi = int(wid % strips);
     const bool live = LY0 < t.nL;                   // warp-uniform
+    if (blockIdx.x == 0 && threadIdx.x == 0) *t.surf_counter = 0u;
     const int nly = min(kRows, t.nL - LY0);  // leaf rows of this warp
     const int xs = sxi * 128, x0 = xs + 4 * lane;
     const bool act = x0 < n;

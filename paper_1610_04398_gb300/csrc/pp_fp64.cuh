@@ -46,6 +46,7 @@ __global__ void __launch_bounds__(128) k_rhs64(Tree<double> t, const double* __r
                                                const double* __restrict__ usy, double rho, double lam,
                                                double* __restrict__ f_out) {
     if (blockIdx.x == 0 && threadIdx.x < 32) level_exp(t)[threadIdx.x] = kExpZero;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *t.surf_counter = 0u;
     const int n = t.n, lane = threadIdx.x & 31;
     const int64_t w = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int strips = n >> 5;
@@ -218,6 +219,8 @@ __global__ void __launch_bounds__(128) k_p2m64(Tree<double> t) {
     __shared__ double2 Ws[10 * kMaxP];
     const int64_t leaf0 = int64_t(blockIdx.x) * 32, nleaf = int64_t(t.nL) * t.nL;
     const int lane = threadIdx.x & 31, r = threadIdx.x >> 5;
+    const int64_t box0 = int64_t(blockIdx.x) * 128 + threadIdx.x;  // four threads a leaf: one a box above
+    if (box0 < level_offset(t.Lleaf - 1)) arrivals(t)[box0] = 0u;
     for (int i = threadIdx.x; i < 32 * 64; i += 128)
         qs[(i >> 6) * 65 + (i & 63)] = leaf0 + (i >> 6) < nleaf ? t.q[leaf0 * 64 + i] : 0.0;
     stage_orbits(Ws, t.Wp2m, t.P1);
@@ -238,7 +241,7 @@ __global__ void __launch_bounds__(128) k_p2m64(Tree<double> t) {
 
 // ------------------------------------------------------------------------------------
 // Upward pass in one launch: a warp per box of level L - 1 shifts its four leaves' multipoles;
-// the warp that arrives last at a parent (arrival counters, reset by it; no warp waits) goes on
+// the warp that arrives last at a parent (arrival counters, cleared by k_p2m64; no warp waits) goes on
 // with it.  With zeta_q = i^m(q) zeta_3 the four shifts are one real product over
 // G_r[j] = sum_q i^(m(q) r) M_j (child q), lane k forming coefficient k:
 //   M_k = zeta_3^k [G_k[0] / k + sum_j C(k-1, j-1) (2 zeta_3)^-j G_(k-j)[j]].
@@ -312,7 +315,6 @@ __global__ void __launch_bounds__(128) k_up64(Tree<double> t) {
         if (k == 0) arrived = atomicAdd(cnt, 1u);
         if (__shfl_sync(0xffffffffu, arrived, 0) != 3u) return;
         __threadfence();  // the other children's after it
-        if (k == 0) *cnt = 0u;
         b = pa;
         --l;
     }

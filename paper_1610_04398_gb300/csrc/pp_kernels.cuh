@@ -77,6 +77,7 @@ k_rhs_p2m(Tree<T> t, const T* __restrict__ u, const T* __restrict__ v, const T* 
     const int tx0 = blockIdx.x * kRT;
     const int ty0 = blockIdx.y * kRT;
     const int tid = threadIdx.x;
+    if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *t.surf_counter = 0u;
 
     for (int idx = tid; idx < kRW * kRW; idx += blockDim.x) {
         const int hi = idx % kRW, hj = idx / kRW;

@@ -392,7 +392,7 @@ k_surface(Tree<T> t, const T* __restrict__ u, const T* __restrict__ v, SurfaceAr
         if (lane == 0) {
             for (int k = 0; k < 4; ++k) a.Psurf[4 * int64_t(blockIdx.x) + k] = sum[k];
             __threadfence();
-            last = atomicAdd(a.counter, 1u) == gridDim.x - 1;
+            last = atomicAdd(t.surf_counter, 1u) == gridDim.x - 1;
         }
     }
     __syncthreads();
@@ -418,7 +418,7 @@ k_surface(Tree<T> t, const T* __restrict__ u, const T* __restrict__ v, SurfaceAr
         for (int k = 0; k < 4; ++k) a.forces[k] = F[k];
         a.forces[4] = Fx * a.uhat_x + Fy * a.uhat_y;
         a.forces[5] = -Fx * a.uhat_y + Fy * a.uhat_x;
-        *a.counter = 0u;
+        *t.surf_counter = 0u;
     }
 }
 
