@@ -353,10 +353,10 @@ int pp_atree_destroy(pp_atree tree);
  * p_out: nleaf*64 device doubles, same layout.  order: 2..30.  stream: a CUDA stream or NULL.
  * Near field: from tables of log|D| over the integer offsets of the cells of a leaf pair, in
  * cells or half cells of the finer leaf (built once in FP64); leaf pairs beyond the tables directly.
- * The first solve on a tree uploads the tree, the lists and the tables and allocates the
- * expansions (synchronising the stream); so does a solve at a higher order than before.  They
- * stay with the tree until pp_atree_destroy, so later solves allocate nothing and only launch
- * kernels on the stream.  Solves on one tree share its arrays: order them on one stream.
+ * The first solve on a tree in each precision uploads the tree, the lists and the tables and
+ * allocates the expansions (synchronising the stream).  They stay with the tree until
+ * pp_atree_destroy, so later solves of any order allocate nothing and only launch kernels on
+ * the stream.  Solves on one tree share its arrays: order them on one stream.
  * Errors: PP_ERR_ARG (NULL tree, q or p_out, order out of range), PP_ERR_OOM, PP_ERR_CUDA.
  */
 int pp_atree_solve(pp_atree tree, int order, const double* q, double* p_out, void* stream);

@@ -152,7 +152,7 @@ struct CoefIndex {
 // ------------------------------------------------------------------------------------
 // Double-float arithmetic: a value hi + lo held in two floats (|lo| <= ulp(hi) / 2), about
 // 48 significant bits, on the FP32 pipe.  The FP64 constant-term sums of the translations
-// use it: an FP64 instruction costs a warp some 20 cycles of its SM's narrow FP64 pipe
+// use it: an FP64 instruction costs a warp some 19 cycles of its SM's narrow FP64 pipe
 // (about 1/64 of the FP32 rate), whatever its number of active lanes.  Error-free sum
 // (Knuth's two-sum) and product (by a fused multiply-add).
 // ------------------------------------------------------------------------------------

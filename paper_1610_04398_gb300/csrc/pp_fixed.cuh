@@ -1,5 +1,5 @@
 // Fixed-point arithmetic that stands in for FP64 multiply-adds in the long sums of the FP64 path.
-// GB300 issues FP64 multiply-adds at 1.9 lanes a clock and SM and 32 x 32 + 64 bit integer ones, two
+// GB300 issues FP64 multiply-adds at 1.67 lanes a clock and SM and 32 x 32 + 64 bit integer ones, two
 // instructions each, at 28 (measured), so three integer ones in place of an FP64 one are five times
 // faster.  A value is an integer v relative to a common power of two, split v = h 2^28 + l with l in
 // [-2^27, 2^27).  Three multiply-adds a product, in 64-bit sums that do not depend on the order:

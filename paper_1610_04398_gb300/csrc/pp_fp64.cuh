@@ -1,5 +1,5 @@
 // The FP64 path's kernels (orders up to 23, leaf level >= 2; other orders keep the generic
-// kernels).  GB300's FP64 pipe issues 1.9 lanes a clock and SM (one warp instruction in about 17
+// kernels).  GB300's FP64 pipe issues 1.67 lanes a clock and SM (one warp instruction in about 19
 // cycles), so the design counts FP64 instructions: the two long sums, the near field and the
 // multipole-to-local translations, run in fixed point on the integer pipe (pp_fixed.cuh), and
 // the remaining steps use the symmetry of their geometry to share products:
@@ -37,7 +37,7 @@ __device__ __forceinline__ int coef_exp(double2 m, int k) {
 // ------------------------------------------------------------------------------------
 // (a1) Source, one warp per strip of 32 columns and kSrcRows rows (fewer on small grids), marching down with the rows above,
 // at and below in registers; x neighbours by shuffles (the strip's outer columns read by lanes
-// 0 and 31).  About 21 FP64 instructions a cell, which bound it (36 us at 1024^2 at the pipe's
+// 0 and 31).  About 21 FP64 instructions a cell, which bound it (42 us at 1024^2 at the pipe's
 // rate; 129 us before, 72 now).  Also clears the level exponents.
 // ------------------------------------------------------------------------------------
 template <int kSrcRows>
@@ -454,7 +454,7 @@ __global__ void __launch_bounds__(256, 2) k_near64(Tree<double> t, double* __res
 // that add their integer sums through distributed shared memory.  The S log(|tau| side) terms stay FP64, a
 // logarithm each (log|tau| and log side apart cancel).
 // Bound by the integer multiply-adds, 9 per complex product: 390 us at 1024^2, p = 20, theta = 0.5
-// at the measured rate; 2665 us before on the FP64 pipe in one launch per level, 918 now.
+// at the measured rate; 2665 us before on the FP64 pipe in one launch per level, 922 now.
 // ------------------------------------------------------------------------------------
 constexpr int kM2LPad = 33;
 constexpr int kM2LBits = 56;

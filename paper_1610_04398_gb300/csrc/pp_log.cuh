@@ -1,5 +1,5 @@
 // Natural logarithm in FP64 from a table, for sums of q log r on GB300's narrow FP64 pipe (an
-// FP64 instruction occupies an SM's pipe for about 17 cycles, so the library's log, some thirty
+// FP64 instruction occupies an SM's pipe for about 19 cycles, so the library's log, some thirty
 // of them, is what the direct sums and multipole evaluations spend their time on).  Table-driven
 // method of Tang (ACM TOMS 16, 1990): x = 2^e m, m in [1, 2), c the reciprocal of the midpoint of m's
 // 1/256 bin to ten bits, 1 in the first bin and 1/2 in the last, r = m c - 1 (one fused multiply-add, at

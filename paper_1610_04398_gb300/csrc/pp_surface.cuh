@@ -58,7 +58,7 @@ struct SurfPhi {
 //
 // Mixed plans, points inside the domain: offsets in cell units, an exact integer difference plus
 // the point's fraction of a cell (split by the traction warp), and the monopole sums as double-float
-// pairs, so the walk has no FP64 (an FP64 instruction holds its SM's pipe for 17 cycles, and sixty
+// pairs, so the walk has no FP64 (an FP64 instruction holds its SM's pipe for 19 cycles, and sixty
 // of them a point were 13 of the walk's 25 us).  The log h parts of every accepted box and near cell add up to log h times
 // the root monopole (they partition the domain) and enter once at the end.
 // kCell: the cell-unit walk, without FP64 even in code that is predicated off.
