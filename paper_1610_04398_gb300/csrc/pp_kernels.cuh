@@ -147,12 +147,8 @@ __global__ void __launch_bounds__(256) k_p2m(Tree<T> t) {
         store_S_leaf(t, off + leaf, s0);
         multipole(t, t.Lleaf, leaf)[0] = cmake<T>(s0, T(0));
     }
-    // Mixed plans collect the four leaves of a warp and store them as planes; FP64 ones store at once.
-    __shared__ C stage[sizeof(T) == 4 ? 8 : 1][sizeof(T) == 4 ? 4 : 1][kMaxP1 + 1];
-    const int lane = threadIdx.x & 31, w = sizeof(T) == 4 ? threadIdx.x >> 5 : 0;
-    C* rec = sizeof(T) == 4 ? stage[w][(lane >> 3) & (sizeof(T) == 4 ? 3 : 0)] : t.mp + (off + leaf) * P1;
-    for (int k = 1; k < P1; ++k) {
-        T ar = T(0), ai = T(0);
+    const auto power_sum = [&](T& ar, T& ai) {  // of the next powers, over the leaf's eight rows
+        ar = ai = T(0);
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
             const T nr = pr[c] * zr[c] - pi[c] * zi;
@@ -166,12 +162,28 @@ __global__ void __launch_bounds__(256) k_p2m(Tree<T> t) {
             ar += __shfl_xor_sync(0xffffffffu, ar, o);
             ai += __shfl_xor_sync(0xffffffffu, ai, o);
         }
-        if ((sizeof(T) == 4 || act) && row == (k & 7)) {
-            const T ik = T(1) / T(k);
-            rec[k] = cmake<T>(ar * ik, ai * ik);
+    };
+    if constexpr (sizeof(T) == 8) {
+        for (int k = 1; k < P1; ++k) {
+            T ar, ai;
+            power_sum(ar, ai);
+            if (act && row == (k & 7)) {
+                const T ik = T(1) / T(k);
+                multipole(t, t.Lleaf, leaf)[k] = cmake<T>(ar * ik, ai * ik);
+            }
         }
-    }
-    if constexpr (sizeof(T) == 4) {
+    } else {  // the four leaves of a warp are collected and stored as planes
+        __shared__ C stage[8][4][kMaxP1 + 1];
+        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+        C* rec = stage[w][lane >> 3];
+        for (int k = 1; k < P1; ++k) {
+            T ar, ai;
+            power_sum(ar, ai);
+            if (row == (k & 7)) {
+                const T ik = T(1) / T(k);
+                rec[k] = cmake<T>(ar * ik, ai * ik);
+            }
+        }
         __syncwarp();
         const int lf = lane & 3;
         const int64_t mine = leaf - (lane >> 3) + lf;
