@@ -276,7 +276,7 @@ __device__ __forceinline__ void surf_barrier() {
 // lifted point, the dS), then the tractions and their sums.  The CTA that finishes last (a counter it
 // resets; no CTA waits) adds the CTAs' sums in a fixed order and forms drag and lift.  Before, the
 // walk, the tractions (8.5 us, a chain of FP64 latencies) and the final sum (4.8 us) ran one after the
-// other: 39 us for 2048 points at 2048^2, p = 12, theta 0.5, 21 now (4096 points at 256^2: 37, 23 now).
+// other: 39 us for 2048 points at 2048^2, p = 12, theta 0.5, 19 now (4096 points at 256^2: 37, 21 now).
 template <typename T, int P1T, bool kMany>
 __global__ void __launch_bounds__((SurfCta<T, kMany>::threads), (SurfCta<T, kMany>::ctas))
 k_surface(Tree<T> t, const T* __restrict__ u, const T* __restrict__ v, SurfaceArgs a) {
