@@ -6,7 +6,7 @@
 //   exact (FixedSum):  hh, ll and (h + l)(h' + l') of two values, whose cross terms are the third sum less
 //     the other two (Karatsuba and Ofman's product, modulo 2^64: only what is left has to fit);
 //   to the cross terms: hh and hl + lh; ll, up to 2^54 of either sign, is dropped: 2^(54 - bits) of a
-//     full-scale product of `bits` bits (the translations: 111 bits, 2^-57).
+//     full-scale product of `bits` bits (the translations: 113 bits, 2^-59).
 // Rounding the values is then what the sums lose.
 #pragma once
 
